@@ -237,6 +237,7 @@ __global__ void __launch_bounds__(256, 1) k_adjoint_step(const StepParams<T> p, 
         const int g = tid % G;
         const bool vec = p.vec != 0;
         for (int base = 1; base <= TR; base += rpp) {
+            if (base + (tid & ~31) / G > TR) continue;   // no row for this warp
             int lr = base + tid / G;
             bool in_tile = lr <= TR && i0 - 1 + lr < Nr;
             int gi = i0 - 1 + lr;
@@ -598,6 +599,7 @@ __global__ void __launch_bounds__(256, 1) k_adjoint_spin(const StepParams<T> p, 
     if (SPIN && !tape) {
         const int rpp = NT / G;
         for (int base = 0; base < R; base += rpp) {
+            if (base + (tid & ~31) / G >= R) continue;   // no row for this warp
             const int lr = base + tid / G;
             const bool in_tile = lr < R;
             const int gi = i0 - 1 + lr;
@@ -755,6 +757,7 @@ __global__ void __launch_bounds__(256, 1) k_adjoint_spin(const StepParams<T> p, 
     {
         const int rpp = NT / G;
         for (int base = 1; base <= TR; base += rpp) {
+            if (base + (tid & ~31) / G > TR) continue;   // no row for this warp
             const int lr = base + tid / G;
             const bool in_tile = lr <= TR && i0 - 1 + lr < Nr;
             const int gi = i0 - 1 + lr;

@@ -259,6 +259,7 @@ __global__ void __launch_bounds__(NTH, (NTH == 256 && sizeof(T) == 4 && S <= 4) 
                     if (last > hi - 1) last = hi - 1;
                     for (int c = base / cr; c <= last / cr; ++c) ok &= (int)mbar_wait(&s_full[b][c], par, wait_lim);
                 }
+                if (base + (tid & ~31) / G >= hi) continue;   // no row for this warp
                 const int lr = base + tid / G;
                 const bool in_tile = lr < hi;
                 const int gi = g0 + lr;

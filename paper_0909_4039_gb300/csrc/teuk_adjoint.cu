@@ -21,9 +21,10 @@ __device__ __forceinline__ int tile_of_block(int b, int nt, int i_ext, int tile_
 
 // h = E u with u = s (physical) or u = C_{dt/2} s on the extraction row; one
 // warp.  The sum is the one the step kernels write to the waveform buffer.
+// The row's planes at (f, g); without h_out the sample goes to the ring buffer, as `step`'s.
 template <typename T, int S>
-__global__ void __launch_bounds__(32) k_sample(const StepParams<T> p, const typename V2<T>::t *s, int physical,
-                                               double2 *h_out)
+__device__ __forceinline__ void sample_row(const StepParams<T> &p, const typename V2<T>::t *f, const typename V2<T>::t *g,
+                                           int physical, double2 *h_out, long long step)
 {
     typedef typename V2<T>::t c2;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -31,10 +32,12 @@ __global__ void __launch_bounds__(32) k_sample(const StepParams<T> p, const type
     c2 *xPhi = (c2 *)smem_raw;
     c2 *xPi = xPhi + ((N + 1) & ~1);
     T *xF = (T *)(xPi + ((N + 1) & ~1));
-    T *xTh = xF + NSF;
+    unsigned long long *xTh2 = (unsigned long long *)(xF + NSF);
+    T *xTh = (T *)(xTh2 + pair_th_bytes(N, (int)sizeof(T)) / 8);
+    if constexpr (kPaired<T, S>) pair_th_fill(xTh2, p.thtab, N, tid, 32);
     for (int j = tid; j < N; j += 32) {
-        xPhi[j] = s[(size_t)i * N + j];
-        xPi[j] = s[((size_t)Nr + i) * N + j];
+        xPhi[j] = f[j];
+        xPi[j] = g[j];
     }
     if (tid < NSF) xF[tid] = p.stab[(size_t)(2 * i) * NSF + tid];
     for (int k = tid; k < NTF * N; k += 32) xTh[k] = p.thtab[k];
@@ -43,12 +46,62 @@ __global__ void __launch_bounds__(32) k_sample(const StepParams<T> p, const type
         const int G = p.group;
         const bool mine = tid < G;
         const bool active = mine && i >= 1 && i <= Nr - 2;
-        implicit_row_fwd<T, S>(p.half, xPhi, xPi, p.half.piv + (size_t)i * N, xF, xTh, N, active, mine, tid % G, G,
-                                 p.vec != 0, p.half.plan[i]);
+        implicit_row_one<T, S>(p.half, xPhi, xPi, i, xF, xTh, xTh2, N, active, mine, tid % G, G, p.vec != 0,
+                               p.half.plan[i]);
         __syncwarp();
+    }
+    if (!h_out) {
+        extract_warp<T>(p, xPhi, step);
+        return;
     }
     double2 h = sample_warp<T>(p, xPhi);
     if (tid == 0) *h_out = h;
+}
+
+template <typename T, int S>
+__global__ void __launch_bounds__(32) k_sample(const StepParams<T> p, const typename V2<T>::t *s, int physical,
+                                               double2 *h_out)
+{
+    const size_t o = (size_t)p.i_ext * p.Nth;
+    sample_row<T, S>(p, s + o, s + (size_t)p.Nr * p.Nth + o, physical, h_out, 0);
+}
+
+// CTA (b, instance): the b-th step after ctl->sampled, if it has been taken.
+// The last CTA of an instance moves ctl->sampled on.
+template <typename T, int S>
+__device__ __forceinline__ void sample_step(const StepParams<T> &p)
+{
+    const long long n0 = *((volatile long long *)&p.ctl->sampled), n1 = *((volatile long long *)&p.ctl->step);
+    const long long n = n0 + 1 + blockIdx.x;
+    // (only the last wave_cap samples stay in the ring: two steps of one slot do not race)
+    if (n <= n1 && n > n1 - p.wave_cap) {
+        const typename V2<T>::t *r = p.raw + (size_t)(n % kRawSlots) * 2 * p.Nth;
+        sample_row<T, S>(p, r, r + p.Nth, 0, nullptr, n);
+    }
+    __syncwarp();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        if (atomicAdd(&p.ctl->sticket, 1u) == gridDim.x - 1u) {
+            p.ctl->sticket = 0u;
+            p.ctl->sampled = n1;
+        }
+    }
+}
+
+template <typename T, int S>
+__global__ void __launch_bounds__(32) k_sample_steps(const StepParams<T> p)
+{
+    sample_step<T, S>(p);
+}
+
+template <typename T, int S>
+__global__ void __launch_bounds__(32) k_sample_steps_batch(const StepParams<T> *params)
+{
+    __shared__ __align__(16) StepParams<T> sp;
+    for (int k = threadIdx.x; k < (int)(sizeof(StepParams<T>) / 4); k += 32)
+        reinterpret_cast<int *>(&sp)[k] = reinterpret_cast<const int *>(params + blockIdx.y)[k];
+    __syncwarp();
+    sample_step<T, S>(sp);
 }
 
 // Adds conj(lam) * coef * (unit source) * phase to the amplitude sum cA and
@@ -549,6 +602,8 @@ __global__ void __launch_bounds__(256, 1) k_adjoint_spin(const StepParams<T> p, 
     T *sSt = (T *)(fmG + plane);
     T *sDSt = sSt + (2 * R - 1) * NSF;
     T *sTh = sDSt + (2 * R - 1) * NSF;
+    unsigned long long *sTh2 = (unsigned long long *)(sTh + NTF * N);   // FP32 rows of 128 < Ntheta <= 256 (teuk_pair.cuh)
+    if constexpr (kPaired<T, S> && SPIN) pair_th_fill(sTh2, p.thtab, N, tid, NT);
 
     // ---- lam_{n+1} and s_n (with a tape: the forward stage values U2 and U1
     // the forward step recorded) on rows i0-1 .. i0+TR, the step tables,
@@ -605,10 +660,15 @@ __global__ void __launch_bounds__(256, 1) k_adjoint_spin(const StepParams<T> p, 
             const int gi = i0 - 1 + lr;
             const bool active = in_tile && gi >= 1 && gi <= Nr - 2;
             const int lrc = in_tile ? lr : 0;
-            implicit_row_fwd<T, S, MAT>(K, vF + lrc * P, vG + lrc * P, K.piv + (size_t)(active ? gi : 1) * N,
-                                        sSt + 2 * lrc * NSF, sTh, N, active, in_tile, g, G, vec,
-                                        active ? K.plan[gi] : 0, &A.m, active ? gi : 1, u1F + lrc * P,
-                                        u1G + lrc * P);
+            if constexpr (kPaired<T, S>)
+                implicit_row_one<T, S>(K, vF + lrc * P, vG + lrc * P, active ? gi : 1,
+                                       sSt + 2 * interior_row(lrc, i0 - 1, Nr) * NSF, sTh, sTh2, N, active, in_tile, g, G,
+                                       vec, active ? K.plan[gi] : 0, u1F + lrc * P, u1G + lrc * P);
+            else
+                implicit_row_fwd<T, S, MAT>(K, vF + lrc * P, vG + lrc * P, K.piv + (size_t)(active ? gi : 1) * N,
+                                            sSt + 2 * lrc * NSF, sTh, N, active, in_tile, g, G, vec,
+                                            active ? K.plan[gi] : 0, &A.m, active ? gi : 1, u1F + lrc * P,
+                                            u1G + lrc * P);
         }
     }
     __syncthreads();
@@ -800,9 +860,8 @@ __global__ void __launch_bounds__(256, 1) k_adjoint_spin(const StepParams<T> p, 
                 const bool active = mine && p.i_ext >= 1 && p.i_ext <= Nr - 2;
                 // forward C_{dt/2} on the row of s_n: (sF, sG) <- U2, (aF, aG) <- U1
                 if constexpr (SPIN)
-                    implicit_row_fwd<T, S>(p.half, sF, sG, p.half.piv + (size_t)p.i_ext * N, sSt + 2 * lx * NSF, sTh,
-                                           N, active, mine, tid % G, G, vec, active ? p.half.plan[p.i_ext] : 0,
-                                           nullptr, 0, aF, aG);
+                    implicit_row_one<T, S>(p.half, sF, sG, p.i_ext, sSt + 2 * lx * NSF, sTh, sTh2, N, active, mine, tid % G,
+                                           G, vec, active ? p.half.plan[p.i_ext] : 0, aF, aG);
                 __syncwarp();
                 const double d = implicit_row_adj_spin<T, S, false, SPIN>(p.half, xF, xG, aF, aG, sF, sG,
                                                              p.half.piv + (size_t)p.i_ext * N, sSt + 2 * lx * NSF,
@@ -926,17 +985,48 @@ __global__ void __launch_bounds__(32) k_dot_final(const double *part, int nblk, 
 }  // namespace
 
 template <typename T>
+static size_t sample_smem_bytes(int Nth)
+{
+    const size_t row = (size_t)((Nth + 1) & ~1);
+    return 2 * row * sizeof(typename V2<T>::t) + ((size_t)NSF + (size_t)NTF * Nth) * sizeof(T) +
+           pair_th_bytes(Nth, (int)sizeof(T));
+}
+
+template <typename T>
 cudaError_t launch_sample(const StepParams<T> &p, const typename V2<T>::t *s, int physical, double2 *h_out,
                           cudaStream_t st)
 {
-    typedef typename V2<T>::t c2;
     const int seg = implicit_seg(p.Nth);
     auto fn = seg == kSegNarrow ? k_sample<T, kSegNarrow> : (seg == kSeg ? k_sample<T, kSeg> : k_sample<T, kSegWide>);
     cudaError_t e = smem_limit_max((const void *)fn);
     if (e != cudaSuccess) return e;
-    const size_t row = (size_t)((p.Nth + 1) & ~1);
-    const size_t smem = 2 * row * sizeof(c2) + ((size_t)NSF + (size_t)NTF * p.Nth) * sizeof(T);
-    fn<<<1, 32, smem, st>>>(p, s, physical, h_out);
+    fn<<<1, 32, sample_smem_bytes<T>(p.Nth), st>>>(p, s, physical, h_out);
+    return cudaGetLastError();
+}
+
+template <typename T>
+cudaError_t launch_sample_steps(const StepParams<T> &p, int pending, cudaStream_t st)
+{
+    if (pending < 1 || pending > kRawSlots) return cudaErrorInvalidValue;
+    const int seg = implicit_seg(p.Nth);
+    auto fn = seg == kSegNarrow ? k_sample_steps<T, kSegNarrow>
+                                : (seg == kSeg ? k_sample_steps<T, kSeg> : k_sample_steps<T, kSegWide>);
+    cudaError_t e = smem_limit_max((const void *)fn);
+    if (e != cudaSuccess) return e;
+    fn<<<pending, 32, sample_smem_bytes<T>(p.Nth), st>>>(p);
+    return cudaGetLastError();
+}
+
+template <typename T>
+cudaError_t launch_sample_steps_batch(const StepParams<T> *d_params, int count, int Nmax, int pending, cudaStream_t st)
+{
+    if (pending < 1 || pending > kRawSlots) return cudaErrorInvalidValue;
+    const int seg = implicit_seg(Nmax);
+    auto fn = seg == kSegNarrow ? k_sample_steps_batch<T, kSegNarrow>
+                                : (seg == kSeg ? k_sample_steps_batch<T, kSeg> : k_sample_steps_batch<T, kSegWide>);
+    cudaError_t e = smem_limit_max((const void *)fn);
+    if (e != cudaSuccess) return e;
+    fn<<<dim3((unsigned)pending, (unsigned)count), 32, sample_smem_bytes<T>(Nmax), st>>>(d_params);
     return cudaGetLastError();
 }
 
@@ -976,7 +1066,8 @@ template <typename T>
 size_t adjoint_spin_smem_bytes(int tile_rows, int Nth)
 {
     const size_t R = (size_t)tile_rows + 2;
-    return 10 * R * Nth * sizeof(typename V2<T>::t) + (2 * (2 * R - 1) * NSF + (size_t)NTF * Nth) * sizeof(T);
+    return 10 * R * Nth * sizeof(typename V2<T>::t) + (2 * (2 * R - 1) * NSF + (size_t)NTF * Nth) * sizeof(T) +
+           pair_th_bytes(Nth, (int)sizeof(T));
 }
 
 template <typename T, bool MAT, bool SPIN = true>
@@ -1046,6 +1137,10 @@ cudaError_t launch_dot(const typename V2<T>::t *x, const typename V2<T>::t *y, c
 
 template cudaError_t launch_sample<float>(const StepParams<float> &, const float2 *, int, double2 *, cudaStream_t);
 template cudaError_t launch_sample<double>(const StepParams<double> &, const double2 *, int, double2 *, cudaStream_t);
+template cudaError_t launch_sample_steps<float>(const StepParams<float> &, int, cudaStream_t);
+template cudaError_t launch_sample_steps<double>(const StepParams<double> &, int, cudaStream_t);
+template cudaError_t launch_sample_steps_batch<float>(const StepParams<float> *, int, int, int, cudaStream_t);
+template cudaError_t launch_sample_steps_batch<double>(const StepParams<double> *, int, int, int, cudaStream_t);
 template size_t adjoint_smem_bytes<float>(int, int);
 template size_t adjoint_smem_bytes<double>(int, int);
 template int adjoint_grid<float>(int, int);

@@ -91,7 +91,8 @@ Layout make_layout(const teuk_grid_desc &d)
     L.plan = off; off = align256(off + sizeof(int) * Nr);
     L.planh = off; off = align256(off + sizeof(int) * Nr);
     {
-        const size_t lanes = (size_t)implicit_group((int)N);
+        // FP32 rows of 128 < Ntheta <= 256 have two segments a lane (teuk_pair.cuh)
+        const size_t lanes = (size_t)implicit_group((int)N) * (f32 && implicit_seg((int)N) == kSeg ? 2 : 1);
         L.seg = off; off = align256(off + c2 * 2 * lanes * Nr);
         L.segh = off; off = align256(off + c2 * 2 * lanes * Nr);
     }
@@ -99,6 +100,7 @@ Layout make_layout(const teuk_grid_desc &d)
     L.patchu = off; off = align256(off + c2 * 2 * N * patch_rows);
     L.w = off; off = align256(off + sizeof(double) * N);
     L.ctl = off; off = align256(off + sizeof(Ctl));
+    L.raw = off; off = align256(off + c2 * 2 * N * (size_t)kRawSlots);
     L.staging_elems = 0;
     L.staging = off;
     if (f32) {
@@ -469,7 +471,7 @@ StepParams<T> make_params(const teuk_ctx *c, int in_level)
     p.group = implicit_group((int)d.Ntheta);
     {
         const int seg = implicit_seg((int)d.Ntheta);
-        p.vec = (d.Ntheta % seg == 0 && d.Ntheta % 4 == 0) ? 1 : 0;
+        p.vec = ((seg == kSeg && sizeof(T) == 4) || d.Ntheta % seg == 0) && d.Ntheta % 4 == 0 ? 1 : 0;
     }
     p.first = c->shifted ? 0 : 1;
     p.imp_only = 0;
@@ -533,6 +535,7 @@ StepParams<T> make_params(const teuk_ctx *c, int in_level)
     p.uout = (c2 *)(c->state + (size_t)(1 - in_level) * c->level_bytes);
     p.mid = (c2 *)(c->coef + c->L.scratch);
     p.wave = c->wave;
+    p.raw = (c2 *)(c->coef + c->L.raw);
     p.ctl = (Ctl *)(c->coef + c->L.ctl);
     return p;
 }
@@ -619,6 +622,13 @@ cudaError_t extract_current(teuk_ctx *c, cudaStream_t st)
     }
     StepParams<double> p = make_params<double>(c, c->cur);
     return launch_extract<double>(p, p.uin, c->step, st);
+}
+
+// Samples the steps taken since the last such launch (at most kRawSlots).
+cudaError_t sample_steps(teuk_ctx *c, int pending, cudaStream_t st)
+{
+    if (c->d.precision == TEUK_FP32) return launch_sample_steps<float>(make_params<float>(c, c->cur), pending, st);
+    return launch_sample_steps<double>(make_params<double>(c, c->cur), pending, st);
 }
 
 void drop_graphs(teuk_ctx *c)
@@ -933,18 +943,30 @@ int teuk_step(teuk_ctx *c, int64_t nsteps, void *stream)
     if (nsteps < 0) return set_err(c, TEUK_E_INVAL, "nsteps must be >= 0");
     cudaStream_t st = (cudaStream_t)stream;
     int64_t left = nsteps;
+    int pending = 0;   // steps whose extraction rows wait for a sampling launch
     if (left > 0 && c->d.scheme == TEUK_SCHEME_SPLIT && !c->shifted) {
         // first step from a physical state: s_{n+1} = LW C_{dt/2} u_n
         CK(launch_one(c, c->cur, st), "first step launch");
         c->cur ^= 1;
         c->shifted = 1;
         left -= 1;
+        pending = 1;
     }
+    const bool split = c->d.scheme == TEUK_SCHEME_SPLIT;
+    // the pipelined and persistent kernels sample their own steps: what is left
+    // from before them comes first (as before a graph, whose chunk is its own)
+    auto flush = [&]() -> cudaError_t {
+        if (!split || pending == 0) return cudaSuccess;
+        const int n = pending;
+        pending = 0;
+        return sample_steps(c, n, st);
+    };
     // steps per launch from here on (the state is shifted)
     const int ks = (c->d.scheme == TEUK_SCHEME_SPLIT && c->ks >= 2) ? c->ks : 1;
     // steps per captured graph: a multiple of ks over an even number of launches
     const int chunk = ks == 3 ? 3 * kGraphChunk / 2 : kGraphChunk;
     bool use_graph = st != nullptr && c->d.scheme == TEUK_SCHEME_SPLIT && left >= 2 * chunk;
+    if (use_graph || c->pipe || c->persist) CK(flush(), "samples");
     if (use_graph) {
         int g = c->cur;
         if (c->graph[g] && c->graph_stream[g] != st) {
@@ -962,6 +984,7 @@ int teuk_step(teuk_ctx *c, int64_t nsteps, void *stream)
                 done += k;
                 lev ^= 1;
             }
+            if (le == cudaSuccess) le = sample_steps(c, chunk, st);
             cudaError_t ee = cudaStreamEndCapture(st, &graph);
             if (le != cudaSuccess) return cuda_err(c, le, "captured launch");
             if (ee != cudaSuccess) return cuda_err(c, ee, "end capture");
@@ -978,17 +1001,19 @@ int teuk_step(teuk_ctx *c, int64_t nsteps, void *stream)
             left -= chunk;
         }
     }
-    while (left >= ks) {
-        int k = 0;
-        CK(launch_unit(c, c->cur, st, &k), "step launch");
+    while (left > 0) {
+        int k = 1;
+        if (left >= ks) {
+            CK(launch_unit(c, c->cur, st, &k), "step launch");
+        } else {
+            CK(launch_one(c, c->cur, st), "step launch");
+        }
         c->cur ^= 1;
         left -= k;
+        pending += k;
+        if (pending + ks > kRawSlots) CK(flush(), "samples");
     }
-    while (left > 0) {
-        CK(launch_one(c, c->cur, st), "step launch");
-        c->cur ^= 1;
-        left -= 1;
-    }
+    CK(flush(), "samples");
     c->step += nsteps;
     return TEUK_OK;
 }
@@ -1612,6 +1637,7 @@ struct teuk_batch {
     std::vector<teuk_ctx *> c;
     std::vector<int> tr;             // tile height per instance
     int prec, seg;
+    bool paired;                     // every instance takes the FP32 kernels on packed pairs
     char *ws;                        // caller-owned device workspace
     size_t ws_bytes, par_bytes;      // par_bytes: one parameter table
     size_t off_par[3], off_tiles;    // tables: in = cur, in = cur ^ 1, first step; tile list
@@ -1716,6 +1742,7 @@ int batch_layout(teuk_batch *b)
     if (k >= 1 && b->ks == 2)
         k = b->prec == TEUK_FP32 ? split_batch_blocks_per_sm<float>(b->seg, smem, 1)
                                  : split_batch_blocks_per_sm<double>(b->seg, smem, 1);
+    if (k >= 1 && b->paired) k = pair_batch_blocks_per_sm(b->ks, smem);
     if (k < 1) return bset_err(b, TEUK_E_INVAL, "the batched kernel does not fit on this device with these tiles");
     b->htiles.clear();
     for (int t = 0; t < maxt; ++t)
@@ -1762,6 +1789,8 @@ cudaError_t batch_launch(teuk_batch *b, int table, int ks, cudaStream_t st)
 {
     const int2 *tiles = (const int2 *)(b->ws + b->off_tiles);
     if (table == 2) ks = 1;
+    if (b->paired && table != 2)
+        return launch_pair_batch((const StepParams<float> *)(b->ws + b->off_par[table]), tiles, b->ntot, b->smem, ks, st);
     if (b->prec == TEUK_FP32)
         return launch_split_batch<float>((const StepParams<float> *)(b->ws + b->off_par[table]), tiles, b->ntot, b->seg,
                                          b->smem, ks, st);
@@ -1775,6 +1804,16 @@ int batch_step_impl(teuk_batch *b, int64_t nsteps, cudaStream_t st)
     if (left <= 0) return TEUK_OK;
     int r = batch_tables(b, st);
     if (r != TEUK_OK) return r;
+    int Nmax = 1;
+    for (teuk_ctx *c : b->c) Nmax = (int)c->d.Ntheta > Nmax ? (int)c->d.Ntheta : Nmax;
+    int pending = 0;   // steps whose extraction rows wait for a sampling launch
+    // (any parameter table: it reads the rows, not the state)
+    auto samples = [&](int n) {
+        const char *tab = b->ws + b->off_par[0];
+        const int count = (int)b->c.size();
+        return b->prec == TEUK_FP32 ? launch_sample_steps_batch<float>((const StepParams<float> *)tab, count, Nmax, n, st)
+                                    : launch_sample_steps_batch<double>((const StepParams<double> *)tab, count, Nmax, n, st);
+    };
     bool any_first = false;
     for (teuk_ctx *c : b->c) any_first = any_first || !c->shifted;
     if (any_first) {
@@ -1785,10 +1824,13 @@ int batch_step_impl(teuk_batch *b, int64_t nsteps, cudaStream_t st)
             c->shifted = 1;
         }
         left -= 1;
+        pending = 1;
         r = batch_tables(b, st);
         if (r != TEUK_OK) return r;
     }
     if (st != nullptr && left >= 2 * kGraphChunk) {
+        if (pending > 0) BCK(samples(pending), "samples");
+        pending = 0;
         if (b->graph && b->graph_stream != st) {
             cudaGraphExecDestroy(b->graph);
             b->graph = nullptr;
@@ -1799,6 +1841,7 @@ int batch_step_impl(teuk_batch *b, int64_t nsteps, cudaStream_t st)
             cudaError_t le = cudaSuccess;
             // kGraphChunk / ks launches: an even count, so the level parity is unchanged
             for (int k = 0; k < kGraphChunk / b->ks && le == cudaSuccess; ++k) le = batch_launch(b, k & 1, b->ks, st);
+            if (le == cudaSuccess) le = samples(kGraphChunk);
             cudaError_t ee = cudaStreamEndCapture(st, &graph);
             if (le != cudaSuccess) return bcuda_err(b, le, "captured batched launch");
             if (ee != cudaSuccess) return bcuda_err(b, ee, "end capture");
@@ -1817,8 +1860,17 @@ int batch_step_impl(teuk_batch *b, int64_t nsteps, cudaStream_t st)
     }
     // each launch (one or two steps) flips every instance's level once
     int64_t launches = 0;
-    for (; left >= b->ks; left -= b->ks, ++launches) BCK(batch_launch(b, (int)(launches & 1), b->ks, st), "batched step");
-    for (; left > 0; --left, ++launches) BCK(batch_launch(b, (int)(launches & 1), 1, st), "batched step");
+    for (; left > 0; ++launches) {
+        const int k = left >= b->ks ? b->ks : 1;
+        BCK(batch_launch(b, (int)(launches & 1), k, st), "batched step");
+        left -= k;
+        pending += k;
+        if (left == 0 || pending + b->ks > kRawSlots) {
+            BCK(samples(pending), "samples");
+            pending = 0;
+        }
+    }
+    if (pending > 0) BCK(samples(pending), "samples");
     for (teuk_ctx *c : b->c) {
         c->cur ^= (int)(launches & 1);
         c->step += nsteps;
@@ -1876,6 +1928,8 @@ int teuk_batch_create(teuk_ctx *const *ctxs, int count, void *d_ws, size_t ws_by
     b->c.assign(ctxs, ctxs + count);
     b->prec = prec;
     b->seg = seg;
+    b->paired = prec == TEUK_FP32;
+    for (int i = 0; i < count; ++i) b->paired = b->paired && pair_eligible((int)ctxs[i]->d.Ntheta);
     b->ws = (char *)d_ws;
     b->ws_bytes = ws_bytes;
     batch_ws_bytes(ctxs, count, &b->par_bytes, &b->off_tiles);

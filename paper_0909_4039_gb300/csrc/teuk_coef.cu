@@ -428,6 +428,8 @@ __global__ void k_set_ctl(Ctl *c, long long step, int clear_flags)
 {
     c->step = step;
     c->ticket = 0u;
+    c->sampled = step;
+    c->sticket = 0u;
     if (clear_flags) c->flags = 0u;
 }
 

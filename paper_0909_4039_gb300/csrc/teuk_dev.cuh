@@ -13,6 +13,7 @@
 #include <stdio.h>
 
 #include <mutex>
+#include <type_traits>
 #include <utility>
 #include <vector>
 
@@ -472,7 +473,7 @@ __device__ __forceinline__ void row_store(typename V2<T>::t *phi, typename V2<T>
                                           int lenw, bool vec)
 {
     if (lenw <= 0) return;
-    if (vec) {
+    if (vec && lenw == S) {
         vstore<S>(phi + j0, w);
         vstore<S>(pi + j0, y);
     } else {
@@ -906,6 +907,64 @@ __device__ void implicit_row_fwd(const ImpConst<T> &K0, typename V2<T>::t *phi, 
 #pragma unroll
     for (int k = 0; k < S; ++k) w[k] = caxpy(K.gh, v[k], w[k]);
     if (in_tile) row_store<T, S>(phi, pi, w, v, j0, lenw, vec);
+}
+
+}  // namespace
+}  // namespace teuk
+
+#include "teuk_pair.cuh"
+
+namespace teuk {
+namespace {
+
+// Whether a kernel's row solves run on packed pairs (teuk_pair.cuh): the FP32
+// state with 128 < Ntheta <= 256.
+template <typename T, int S> constexpr bool kPaired = sizeof(T) == 4 && S == kSeg;
+
+// A valid interior tile row (for a step-table entry) near tile row lr.
+__device__ __forceinline__ int interior_row(int lr, int g0, int Nr)
+{
+    const int lo = 1 - g0, hi = Nr - 2 - g0;
+    return lr < lo ? lo : (lr > hi ? hi : lr);
+}
+
+// One row, by one warp, through the solve its grid's step kernels use
+// (128 < Ntheta <= 256 in FP32: HALVES, needing the paired theta table th2;
+// lane g of G = 32); else implicit_row_fwd.
+template <typename T, int S>
+__device__ __forceinline__ void implicit_row_one(const ImpConst<T> &K, typename V2<T>::t *phi, typename V2<T>::t *pi, int gi,
+                                                 const T *f, const T *th, const unsigned long long *th2, int N,
+                                                 bool active, bool in_tile, int g, int G, bool vec, int plan,
+                                                 typename V2<T>::t *u1f = nullptr, typename V2<T>::t *u1g = nullptr)
+{
+    if constexpr (kPaired<T, S>) {
+        PairRow A, B;
+        A.phi = phi;
+        A.pi = pi;
+        A.piv = K.piv + (size_t)gi * N;
+        A.seg = K.seg + ((size_t)gi * 32 + g) * 4;
+        A.f = f;
+        A.u1f = u1f;
+        A.u1g = u1g;
+        A.plan = active ? plan : 0;
+        A.n = 128;
+        A.active = active;
+        A.in_tile = in_tile;
+        B = A;
+        B.phi += 128;
+        B.pi += 128;
+        B.piv += 128;
+        B.seg += 2;
+        if (u1f) {
+            B.u1f += 128;
+            B.u1g += 128;
+        }
+        B.n = N - 128;
+        implicit_pair(K, A, B, th2, g, vec);
+    } else {
+        implicit_row_fwd<T, S>(K, phi, pi, K.piv + (size_t)gi * N, f, th, N, active, in_tile, g, G, vec,
+                               plan, nullptr, 0, u1f, u1g);
+    }
 }
 
 template <typename C> __device__ __forceinline__ C conj_c(C a) { return cmk<C>(a.x, -a.y); }
@@ -1412,7 +1471,6 @@ __device__ __forceinline__ void split_tile(const StepParams<T> &p, int tile, int
     static_assert(KS >= 1 && KS <= 3, "one to three steps per launch");
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ double2 sph[2 * KS];
-    __shared__ long long s_n;
     __shared__ __align__(8) unsigned long long s_mbar[kMaxChunks];
     __shared__ int s_plan[kMaxTileRows + 6];   // stored scan levels of the tile rows
     const int Nr = p.Nr, N = p.Nth, TR = p.tile_rows, R = TR + 2 * KS, P = p.pitch;
@@ -1425,8 +1483,7 @@ __device__ __forceinline__ void split_tile(const StepParams<T> &p, int tile, int
     c2 *sPi = (c2 *)(smem_raw + plan.pi);
     T *sSt = (T *)(smem_raw + plan.rt);   // step-table entries (SField) of the tile's positions
     T *sTh = (T *)(smem_raw + plan.th);
-    c2 *xPhi = (c2 *)(smem_raw + plan.total);   // KS > 1: copy of the extraction row
-    c2 *xPi = xPhi + N;
+    unsigned long long *sTh2 = (unsigned long long *)(smem_raw + plan.th2);   // paired theta table (kPaired)
     // implicit step of this launch: dt/2 for the first step and for the state
     // output (one step per launch only; with more steps per launch it is the
     // full step, chosen at compile time so that its constants are read at
@@ -1445,29 +1502,9 @@ __device__ __forceinline__ void split_tile(const StepParams<T> &p, int tile, int
             }
         }
     }
-    if (tid == 0) {
-        long long n = p.nfix >= 0 ? p.nfix : *((volatile long long *)&p.ctl->step);
-        s_n = n;
-        if (!p.imp_only && p.nfix < 0) {
-            // The last CTA to read the step index advances it.  Later kernels
-            // on the stream see the new value; no CTA of this launch reads it
-            // again, so no CTA has to wait for its own stores first.
-            __threadfence();
-            unsigned t = atomicAdd(&p.ctl->ticket, 1u);
-            if (t == (unsigned)ntiles - 1u) {
-                p.ctl->ticket = 0u;
-                p.ctl->step = n + KS;
-            }
-        }
-        if (src)
-            for (int k = 0; k < KS; ++k) {
-                double t = (double)(n + k) * p.dt64;
-                // phases of Eqs. 13 and 14 times their stage lengths dt/2 and dt
-                const double2 e1 = phase_at(p.mOmega, t), e2 = phase_at(p.mOmega, t + 0.5 * p.dt64);
-                sph[2 * k] = make_double2(0.5 * p.dt64 * e1.x, 0.5 * p.dt64 * e1.y);
-                sph[2 * k + 1] = make_double2(p.dt64 * e2.x, p.dt64 * e2.y);
-            }
-    }
+    // The step index is read before the first barrier; after it the last CTA
+    // to have read it advances it (below).
+    const long long n_in = p.nfix >= 0 ? p.nfix : *((volatile long long *)&p.ctl->step);
     // ---- A: tile rows g0 .. g0+R-1 (state), r and theta tables; the row
     // solves read their pivots from global memory (L2), which leaves room for
     // taller tiles
@@ -1541,6 +1578,7 @@ __device__ __forceinline__ void split_tile(const StepParams<T> &p, int tile, int
         }
     }
     for (int idx = tid; idx < NTF * N; idx += NT) sTh[idx] = p.thtab[idx];
+    if constexpr (kPaired<T, S>) pair_th_fill(sTh2, p.thtab, N, tid, NT);
     // Every implicit step of the launch uses K: with more steps per launch K
     // is the full step (the launcher refuses first steps and state outputs).
     for (int lr = tid; lr < R; lr += NT) {
@@ -1548,6 +1586,28 @@ __device__ __forceinline__ void split_tile(const StepParams<T> &p, int tile, int
         s_plan[lr] = (gi >= 0 && gi < Nr) ? K.plan[gi] : 0;
     }
     __syncthreads();
+    if (tid == 0 && !p.imp_only && p.nfix < 0) {
+        // The last CTA to read the step index advances it.  Later kernels
+        // on the stream see the new value; no CTA of this launch reads it
+        // again, so no CTA has to wait for its own stores first.
+        __threadfence();
+        unsigned t = atomicAdd(&p.ctl->ticket, 1u);
+        if (t == (unsigned)ntiles - 1u) {
+            p.ctl->ticket = 0u;
+            p.ctl->step = n_in + KS;
+        }
+    }
+    // Source phases of Eqs. 13 and 14 times their stage lengths dt/2 and dt:
+    // one lane each, in the last warp, which short tiles leave idle in the
+    // implicit stage.  An FP64 sincos takes about 3 us of one warp; taken one
+    // after the other by the thread that starts the tile's copies, the 2 KS of
+    // them held a source tile, and with it the launch, for 6 us a step.
+    if (src && tid >= NT - 32 && tid - (NT - 32) < 2 * KS) {
+        const int q = tid - (NT - 32);
+        const double t = (double)(n_in + (q >> 1)) * p.dt64, len = (q & 1) ? p.dt64 : 0.5 * p.dt64;
+        const double2 e = phase_at(p.mOmega, (q & 1) ? t + 0.5 * p.dt64 : t);
+        sph[q] = make_double2(len * e.x, len * e.y);
+    }
     const int g = tid & (G - 1), tq = tid >> lgG;   // lane in the row group, row of the pass
     const int wq = (tid & ~31) >> lgG;              // first row of the warp's in the pass
     const bool vec = p.vec != 0;
@@ -1583,6 +1643,12 @@ __device__ __forceinline__ void split_tile(const StepParams<T> &p, int tile, int
                     t1g = p.tape + ((size_t)Nr + gi) * N;
                 }
             }
+            if constexpr (kPaired<T, S>) {
+                implicit_row_one<T, S>(Ki, sPhi + lrc * P, sPi + lrc * P, active ? gi : 1,
+                                       sSt + 2 * interior_row(lrc, g0, Nr) * NSF, sTh, sTh2, N, active, in_tile, g, G, vec,
+                                       s_plan[lrc], t1f, t1g);
+                continue;
+            }
             // FP64: the stored segment products spare FP64 arithmetic, the
             // bound of that path; FP32 forms them (cheaper than the loads)
             const c2 *segr = sizeof(T) == 8 ? Ki.seg + ((size_t)(active ? gi : 1) * G + g) * 2 : nullptr;
@@ -1597,27 +1663,21 @@ __device__ __forceinline__ void split_tile(const StepParams<T> &p, int tile, int
                                    active, in_tile, g, G, vec, s_plan[lrc], nullptr, 0, t1f, t1g, segr);
         }
     };
-    // physical sample u = C_{dt/2} s of the extraction row (tile row lx) in
-    // place, or of its copy in (xPhi, xPi); warp 0
-    auto extract_row = [&](int lx, long long slot, bool copy) {
-        if (tid < 32) {
-            c2 *rf = copy ? xPhi : sPhi + lx * P, *rg = copy ? xPi : sPi + lx * P;
-            bool mine = tid < G;
-            bool active = mine && p.i_ext >= 1 && p.i_ext <= Nr - 2;
-            implicit_row_fwd<T, S>(p.half, rf, rg, p.half.piv + (size_t)p.i_ext * N, sSt + 2 * lx * NSF, sTh, N,
-                                     active, mine, tid & (G - 1), G, vec, p.half.plan[p.i_ext]);
-            __syncwarp();
-            if (p.nfix >= 0) {
-                // a step applied to caller buffers: the sample alone, to h_out
-                const double2 h = sample_warp<T>(p, rf);
-                if (tid == 0) *p.h_out = h;
-            } else {
-                extract_warp<T>(p, rf, slot);
-            }
+    // Waveform samples: the tile leaves the extraction row of every state it
+    // forms in p.raw, and one sampling launch per chunk of steps solves and sums
+    // those rows side by side (launch_sample_steps).  Solved here, one row by
+    // one warp in every step, they ended the tile's every step: 17 of a
+    // 1024 x 32 FP64 step's 35 us.
+    const bool ext_row = p.i_ext >= i0 && p.i_ext < i0 + TR && p.i_ext < Nr;
+    const bool ext = !p.imp_only && p.nfix < 0 && ext_row;
+    const int lx = p.i_ext - g0;
+    auto leave_row = [&](long long n) {
+        c2 *dst = p.raw + (size_t)(n % kRawSlots) * 2 * N;
+        for (int j = tid; j < N; j += NT) {
+            dst[j] = sPhi[lx * P + j];
+            dst[N + j] = sPi[lx * P + j];
         }
     };
-    const bool ext = !p.imp_only && (p.nfix < 0 || p.h_out != nullptr) && p.i_ext >= i0 && p.i_ext < i0 + TR &&
-                     p.i_ext < Nr;
     // ---- B and C, once per time step of the launch.  Step k (from 0) runs
     // the implicit stage on tile rows k .. R-1-k and the Lax-Wendroff stages
     // on rows k+1 .. R-2-k, so the output rows KS .. KS+TR-1 are exact after
@@ -1694,18 +1754,9 @@ __device__ __forceinline__ void split_tile(const StepParams<T> &p, int tile, int
                 lw_phase<T, false>(p, sPhi, sPi, sSt, sTh, k + 1, R - 2 - 2 * k, g0, tid, NT, src, ph1, ph2, sync_all);
         }
         __syncthreads();
-        if (k + 1 < KS && ext) {
-            // sample of step n+k+1 from a copy of the extraction row; the row
-            // itself goes on into the next step
-            if (tid < 32) {
-                const int lx = p.i_ext - g0;
-                for (int j = tid; j < N; j += 32) {
-                    xPhi[j] = sPhi[lx * P + j];
-                    xPi[j] = sPi[lx * P + j];
-                }
-            }
-            __syncthreads();
-            extract_row(p.i_ext - g0, s_n + k + 1, true);
+        if (ext) {
+            leave_row(n_in + k + 1);
+            if (k + 1 < KS) __syncthreads();   // the next implicit stage works in place
         }
     }
     // ---- D: store the output rows (tile rows KS .. KS+TR-1)
@@ -1733,10 +1784,19 @@ __device__ __forceinline__ void split_tile(const StepParams<T> &p, int tile, int
         }
     }
     if (p.imp_only) return;
-    // ---- E: physical sample u_{n+KS} = C_{dt/2} s_{n+KS} on the extraction row
-    if (ext) {
+    // ---- E: a step applied to caller buffers writes the sample of its output, to h_out
+    if (p.nfix >= 0 && p.h_out && ext_row) {
         __syncthreads();
-        extract_row(p.i_ext - g0, s_n + KS, false);
+        if (tid < 32) {
+            const bool mine = tid < G;
+            const bool active = mine && p.i_ext >= 1 && p.i_ext <= Nr - 2;
+            c2 *rf = sPhi + lx * P, *rg = sPi + lx * P;
+            implicit_row_one<T, S>(p.half, rf, rg, p.i_ext, sSt + 2 * lx * NSF, sTh, sTh2, N, active, mine, tid & (G - 1), G,
+                                   vec, p.half.plan[p.i_ext]);
+            __syncwarp();
+            const double2 h = sample_warp<T>(p, rf);
+            if (tid == 0) *p.h_out = h;
+        }
     }
 }
 

@@ -74,11 +74,18 @@ enum TField { TF_S2 = 0, TF_C, TF_AM, TF_A0, TF_AP, TF_GTH, TF_GA2, TF_DGA2, NTF
 // Error flags in Ctl::flags.
 enum : unsigned { FLAG_NONFINITE = 1u, FLAG_TIMEOUT = 2u };
 
+// Extraction rows the step kernels leave for the sampling kernel, by step
+// number modulo kRawSlots: a launch samples every step since the last one.
+constexpr int kRawSlots = 128;
+
 struct Ctl {
     long long step;      // index n of the state the next step reads
     unsigned ticket;     // CTAs of the current step that have finished
     unsigned flags;      // FLAG_*
-    long long pad[6];
+    long long sampled;   // last step whose waveform sample is recorded
+    unsigned sticket;    // CTAs of the current sampling launch that have finished
+    unsigned spad;
+    long long pad[4];
 };
 
 template <typename T> struct V2;
@@ -186,6 +193,7 @@ template <typename T> struct StepParams {
     c2 *uout;                // [2][Nr][Nth]
     c2 *mid;                 // literal scheme scratch [2][Nr-1][Nth]
     double2 *wave;           // [cap][1 + Nth]
+    c2 *raw;                 // [kRawSlots][2][Nth]: extraction rows of the internal state
     Ctl *ctl;
     // Applying one step to caller buffers (nfix >= 0): the step index is
     // nfix, the step counter is not touched and the ring buffer is not
@@ -209,13 +217,35 @@ template <typename T> struct StepParams {
 constexpr double kGamma = 0.29289321881345247559915563789515;
 constexpr double kPi = 3.14159265358979323846264338327950;
 
+// Lane segments of the implicit row solves.
+constexpr int kSegNarrow = 4;           // theta elements per thread (Ntheta <= 128)
+constexpr int kSeg = 8;                 // theta elements per thread (Ntheta <= 256)
+constexpr int kSegWide = 32;            // theta elements per thread (Ntheta <= 1024)
+// theta elements per thread of the implicit row solves
+__host__ __device__ inline int implicit_seg(int Nth) { return Nth <= 128 ? kSegNarrow : (Nth <= 256 ? kSeg : kSegWide); }
+// threads per theta row (a power of two, at most a warp)
+__host__ __device__ inline int implicit_group(int Nth)
+{
+    int seg = implicit_seg(Nth);
+    int need = (Nth + seg - 1) / seg;
+    int G = 1;
+    while (G < need) G <<= 1;
+    return G;
+}
+
 // Shared-memory carve-up of the split kernel for R = tile_rows + 2 KS rows
 // of N theta points; every section starts on a 16-byte boundary.  piv holds
 // the tile rows' Thomas pivots; rt holds the step-table entries (SField) of
 // the tile's positions, nodes and half nodes interleaved as in the global
 // table.
+// th2: the paired theta table of the FP32 row solves (teuk_pair.cuh): five
+// fields of 128 pairs, for 128 < Ntheta <= 256.
+__host__ __device__ inline unsigned pair_th_bytes(int N, int tsize)
+{
+    return tsize == 4 && implicit_seg(N) == kSeg ? 5u * 128u * 8u : 0u;
+}
 struct SplitSmem {
-    unsigned phi, pi, piv, rt, th, total;
+    unsigned phi, pi, piv, rt, th, th2, total;
 };
 __host__ __device__ inline unsigned smem_align16(unsigned x) { return (x + 15u) & ~15u; }
 __host__ __device__ inline SplitSmem split_smem_plan(int R, int N, int tsize)
@@ -227,7 +257,8 @@ __host__ __device__ inline SplitSmem split_smem_plan(int R, int N, int tsize)
     s.piv = smem_align16(s.pi + plane);
     s.rt = s.piv;   // no pivot plane: the row solves read the pivots from global memory (L2)
     s.th = smem_align16(s.rt + (unsigned)(2 * R - 1) * NSF * (unsigned)tsize);
-    s.total = smem_align16(s.th + (unsigned)NTF * (unsigned)N * (unsigned)tsize);
+    s.th2 = smem_align16(s.th + (unsigned)NTF * (unsigned)N * (unsigned)tsize);
+    s.total = smem_align16(s.th2 + pair_th_bytes(N, tsize));
     return s;
 }
 
@@ -262,14 +293,15 @@ __host__ __device__ inline PersistSmem persist_smem_plan(int R, int N, int tsize
 // [2R][NSF] and the scan plans of its rows (R + 8 ints, the copy starts on
 // a 16-byte boundary of the global plan array).
 struct PipeSmem {
-    unsigned th, xphi, xpi, buf, pi, piv, st, plan, bsize, total;
+    unsigned th, th2, xphi, xpi, buf, pi, piv, st, plan, bsize, total;
 };
 __host__ __device__ inline PipeSmem pipe_smem_plan(int R, int N, int tsize)
 {
     PipeSmem s;
     const unsigned c2 = 2u * (unsigned)tsize, plane = (unsigned)R * (unsigned)N * c2;
     s.th = 0;
-    s.xphi = smem_align16((unsigned)NTF * (unsigned)N * (unsigned)tsize);
+    s.th2 = smem_align16((unsigned)NTF * (unsigned)N * (unsigned)tsize);
+    s.xphi = smem_align16(s.th2 + pair_th_bytes(N, tsize));
     s.xpi = smem_align16(s.xphi + (unsigned)N * c2);
     s.buf = smem_align16(s.xpi + (unsigned)N * c2);
     s.pi = smem_align16(plane);
@@ -283,7 +315,7 @@ __host__ __device__ inline PipeSmem pipe_smem_plan(int R, int N, int tsize)
 
 // ---------------------------------------------------------------- host side
 struct Layout {
-    size_t rtab64, rtabT, stab, dstab, th64, thT, piv, pivh, plan, planh, seg, segh, patch, patchu, w, ctl, staging,
+    size_t rtab64, rtabT, stab, dstab, th64, thT, piv, pivh, plan, planh, seg, segh, patch, patchu, w, ctl, raw, staging,
         scratch;
     size_t mat, mat_bytes;   // materialised coefficients (FP64 split scheme; 0 bytes otherwise)
     size_t total;
@@ -314,6 +346,14 @@ cudaError_t launch_apply_step(const StepParams<T> &p, int threads, size_t smem, 
 template <typename T>
 cudaError_t launch_sample(const StepParams<T> &p, const typename V2<T>::t *s, int physical, double2 *h_out,
                           cudaStream_t st);
+// Waveform samples of the steps after ctl->sampled up to ctl->step, from the
+// extraction rows the step kernels left in p.raw (pending: at least their
+// number, at most kRawSlots); the batched form does so for the instances of a
+// parameter table (Nmax: their largest Ntheta).
+template <typename T>
+cudaError_t launch_sample_steps(const StepParams<T> &p, int pending, cudaStream_t st);
+template <typename T>
+cudaError_t launch_sample_steps_batch(const StepParams<T> *d_params, int count, int Nmax, int pending, cudaStream_t st);
 template <typename T>
 cudaError_t launch_adjoint_step(const StepParams<T> &p, int tile_rows, const double2 *gseed, double *part,
                                 double *acc, cudaStream_t st);
@@ -387,6 +427,18 @@ template <typename T>
 int split3_blocks_per_sm(int Nth, int threads, size_t smem);
 template <typename T>
 cudaError_t launch_split_step3(const StepParams<T> &p, int threads, size_t smem, cudaStream_t st);
+// The FP32 step kernels on packed pairs (teuk_pair_tile.cuh): ks = 1 .. 3 full
+// steps per launch for 128 < Ntheta <= 256, a multiple of 4 (whole lane
+// segments and bulk-copyable rows).  They take the place of k_split_step / 2 /
+// 3 and of the batched kernel there; first steps, state output and steps on
+// caller buffers stay with k_split_step.
+bool pair_eligible(int Nth);
+size_t pair_smem_bytes(int tile_rows, int Nth, int ks);
+int pair_blocks_per_sm(int ks, size_t smem);
+cudaError_t launch_pair_step(const StepParams<float> &p, int ks, cudaStream_t st);
+int pair_batch_blocks_per_sm(int ks, size_t smem);
+cudaError_t launch_pair_batch(const StepParams<float> *d_params, const int2 *d_tiles, int ntiles, size_t smem, int ks,
+                              cudaStream_t st);
 // Scan levels of every row's implicit solves for the steps dt (p.full) and
 // dt/2 (p.half), written to plan_full / plan_half ([Nr] ints each).
 template <typename T>
@@ -421,20 +473,6 @@ int split_batch_blocks_per_sm(int seg, size_t smem, int ks);
 template <typename T>
 cudaError_t launch_split_batch(const StepParams<T> *d_params, const int2 *d_tiles, int ntiles, int seg, size_t smem,
                                int ks, cudaStream_t st);
-constexpr int kSegNarrow = 4;           // theta elements per thread (Ntheta <= 128)
-constexpr int kSeg = 8;                 // theta elements per thread (Ntheta <= 256)
-constexpr int kSegWide = 32;            // theta elements per thread (Ntheta <= 1024)
-// theta elements per thread of the implicit row solves
-inline int implicit_seg(int Nth) { return Nth <= 128 ? kSegNarrow : (Nth <= 256 ? kSeg : kSegWide); }
-// threads per theta row (a power of two, at most a warp)
-inline int implicit_group(int Nth)
-{
-    int seg = implicit_seg(Nth);
-    int need = (Nth + seg - 1) / seg;
-    int G = 1;
-    while (G < need) G <<= 1;
-    return G;
-}
 inline bool split_batch_available(int seg, int ks) { return ks == 1 || (ks == 2 && seg != kSegWide); }
 
 cudaError_t launch_convert_to(int prec, const double2 *src, void *dst, size_t n, cudaStream_t st);

@@ -210,6 +210,7 @@ __global__ void __maxnreg__(PersistRegs<NC>::v) k_split_persist(const StepParams
                                      tid % G, G, vec, p.half.plan[p.i_ext]);
             __syncwarp();
             extract_warp<T>(p, xPhi, s_n + 1);
+            if (tid == 0) p.ctl->sampled = s_n + 1;
         }
     }
 }

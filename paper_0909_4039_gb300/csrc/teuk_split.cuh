@@ -91,6 +91,55 @@ __global__ void __launch_bounds__(256) k_scan_plans(const StepParams<T> p, int *
     int len = N - j0;
     len = len < 0 ? 0 : (len > S ? S : len);
     if (!active) len = 0;
+    if constexpr (kPaired<T, S>) {
+        // one warp per row; segments of four elements, lane g's at 4 g and at 128 + 4 g
+        for (int h = 0; h < 2; ++h) {
+            const ImpConst<T> &K = h ? p.half : p.full;
+            const c2 *prow = K.piv + (size_t)gr * N;
+            c2 Af[2], Ab[2];
+            for (int q = 0; q < 2; ++q) {
+                const int jq = 128 * q + 4 * g;
+                int n = active ? N - jq : 0;
+                n = n < 0 ? 0 : (n > 4 ? 4 : n);
+                ImpCoef<T, 4> C;
+                c2 w[4], y[4];
+                imp_load<T, 4>(K, prow, prow, prow, p.stab + (size_t)(2 * gr) * NSF, p.thtab, N, n, jq, p.vec != 0, C, w, y);
+                const ScanPlan<T> Q = scan_plan_products<T, 4>(C);
+                Af[q] = Q.Af0;
+                Ab[q] = Q.Ab0;
+            }
+            if (in_grid) {
+                c2 *o = (h ? seg_half : seg_full) + ((size_t)gi * 32 + g) * 4;
+                o[0] = Af[0];
+                o[1] = Ab[0];
+                o[2] = Af[1];
+                o[3] = Ab[1];
+            }
+            // levels over the 64 segments, as scan_plan counts them
+            const T tol2 = ScanTol<T>::v * ScanTol<T>::v;
+            auto big = [&](c2 a) { return fma(a.x, a.x, a.y * a.y) > tol2; };
+            int nf = 0, nb = 0;
+            bool gf = true, gb = true;
+#pragma unroll 1
+            for (int l = 0; l < 6; ++l) {
+                const int d = 1 << l;
+                gf = __any_sync(0xffffffffu, gf && ((g >= d && big(Af[0])) || big(Af[1])));
+                gb = __any_sync(0xffffffffu, gb && (big(Ab[0]) || (g + d < 32 && big(Ab[1]))));
+                if (gf) nf = l + 1;
+                if (gb) nb = l + 1;
+                if (!gf && !gb) break;
+                PC F = pc_pack(Af[0], Af[1]), B = pc_pack(Ab[0], Ab[1]);
+                F = pc_up(F, d);
+                B = pc_down(B, d);
+                if (g >= d) Af[0] = cmul(Af[0], cmk<c2>(p_lo(F.x), p_lo(F.y)));
+                Af[1] = cmul(Af[1], cmk<c2>(p_hi(F.x), p_hi(F.y)));
+                Ab[0] = cmul(Ab[0], cmk<c2>(p_lo(B.x), p_lo(B.y)));
+                if (g + d < 32) Ab[1] = cmul(Ab[1], cmk<c2>(p_hi(B.x), p_hi(B.y)));
+            }
+            if (in_grid && g == 0) (h ? plan_half : plan_full)[gi] = nf | (nb << 8);
+        }
+        return;
+    }
     for (int h = 0; h < 2; ++h) {
         const ImpConst<T> &K = h ? p.half : p.full;
         const c2 *prow = K.piv + (size_t)gr * N;
@@ -146,6 +195,7 @@ __global__ void __launch_bounds__(NTH, (NTH == 256 && sizeof(T) == 4 && S <= 4) 
     const int ntiles = (Nr + TR - 1) / TR;
     const PipeSmem L = pipe_smem_plan(R, N, (int)sizeof(T));
     T *sTh = (T *)(smem_raw + L.th);
+    unsigned long long *sTh2 = (unsigned long long *)(smem_raw + L.th2);
     c2 *xPhi = (c2 *)(smem_raw + L.xphi);
     c2 *xPi = (c2 *)(smem_raw + L.xpi);
     const ImpConst<T> &K = p.full;
@@ -222,6 +272,7 @@ __global__ void __launch_bounds__(NTH, (NTH == 256 && sizeof(T) == 4 && S <= 4) 
         if ((int)blockIdx.x < ntiles) issue((int)blockIdx.x, 0);
     }
     for (int idx = tid; idx < NTF * N; idx += NT) sTh[idx] = p.thtab[idx];
+    if constexpr (kPaired<T, S>) pair_th_fill(sTh2, p.thtab, N, tid, NT);
     __syncthreads();
 
     const int g = tid % G;
@@ -273,8 +324,12 @@ __global__ void __launch_bounds__(NTH, (NTH == 256 && sizeof(T) == 4 && S <= 4) 
                         continue;
                     }
                 }
-                implicit_row_fwd<T, S>(K, sPhi + lrc * P, sPi + lrc * P, K.piv + (size_t)(active ? gi : 1) * N, sSt + 2 * lrc * NSF, sTh, N,
-                                       active, in_tile, g, G, vec, plan);
+                if constexpr (kPaired<T, S>)
+                    implicit_row_one<T, S>(K, sPhi + lrc * P, sPi + lrc * P, active ? gi : 1,
+                                           sSt + 2 * interior_row(lrc, g0, Nr) * NSF, sTh, sTh2, N, active, in_tile, g, G, vec, plan);
+                else
+                    implicit_row_fwd<T, S>(K, sPhi + lrc * P, sPi + lrc * P, K.piv + (size_t)(active ? gi : 1) * N, sSt + 2 * lrc * NSF, sTh, N,
+                                           active, in_tile, g, G, vec, plan);
             }
         };
         // Lax-Wendroff stages of step s on tile rows r0 .. r0+nr-1
@@ -314,10 +369,11 @@ __global__ void __launch_bounds__(NTH, (NTH == 256 && sizeof(T) == 4 && S <= 4) 
                 __syncwarp();
                 const bool mine = tid < G;
                 const bool active = mine && p.i_ext >= 1 && p.i_ext <= Nr - 2;
-                implicit_row_fwd<T, S>(p.half, xPhi, xPi, p.half.piv + (size_t)p.i_ext * N, sSt + 2 * lx * NSF, sTh,
-                                       N, active, mine, tid % G, G, vec, p.half.plan[p.i_ext]);
+                implicit_row_one<T, S>(p.half, xPhi, xPi, p.i_ext, sSt + 2 * lx * NSF, sTh, sTh2, N, active, mine, tid % G, G,
+                                       vec, p.half.plan[p.i_ext]);
                 __syncwarp();
                 extract_warp<T>(p, xPhi, slot);
+                if ((tid & 31) == 0) p.ctl->sampled = slot;
             }
         };
 
@@ -527,14 +583,24 @@ cudaError_t launch_mat_coef(const StepParams<T> &p, cudaStream_t st)
 template <typename T>
 size_t split_smem_bytes(int tile_rows, int Nth)
 {
-    return split_smem_plan(tile_rows + 2, Nth, (int)sizeof(T)).total;
+    size_t sm = split_smem_plan(tile_rows + 2, Nth, (int)sizeof(T)).total;
+    if (sizeof(T) == 4 && pair_eligible(Nth)) {
+        const size_t pm = pair_smem_bytes(tile_rows, Nth, 1);
+        sm = pm > sm ? pm : sm;
+    }
+    return sm;
 }
 
-// Two steps per launch: R = TR + 4 rows plus a copy of the extraction row.
+// Two steps per launch: R = TR + 4 rows.
 template <typename T>
 size_t split2_smem_bytes(int tile_rows, int Nth)
 {
-    return split_smem_plan(tile_rows + 4, Nth, (int)sizeof(T)).total + 2 * (size_t)Nth * sizeof(typename V2<T>::t);
+    if (sizeof(T) == 4 && pair_eligible(Nth)) {
+        // (a first step runs the one-step kernel at the same height)
+        const size_t pm = pair_smem_bytes(tile_rows, Nth, 2), sm = split_smem_bytes<T>(tile_rows, Nth);
+        return pm > sm ? pm : sm;
+    }
+    return split_smem_plan(tile_rows + 4, Nth, (int)sizeof(T)).total;
 }
 
 template <typename T>
@@ -542,6 +608,10 @@ int split_blocks_per_sm(int Nth, int threads, size_t smem)
 {
     const int seg = implicit_seg(Nth);
     auto fn = seg == kSegNarrow ? k_split_step<T, kSegNarrow> : (seg == kSeg ? k_split_step<T, kSeg> : k_split_step<T, kSegWide>);
+    // both kernels run at one height: full steps on pairs, first steps here
+    int cap = 1 << 20;
+    if constexpr (sizeof(T) == 4)
+        if (pair_eligible(Nth)) cap = pair_blocks_per_sm(1, smem);
     if (smem_limit_max((const void *)fn) != cudaSuccess) {
         cudaGetLastError();
         return 0;
@@ -551,12 +621,14 @@ int split_blocks_per_sm(int Nth, int threads, size_t smem)
         cudaGetLastError();
         return 0;
     }
-    return nb;
+    return nb < cap ? nb : cap;
 }
 
 template <typename T>
 cudaError_t launch_split_step(const StepParams<T> &p, int threads, size_t smem, cudaStream_t st)
 {
+    if constexpr (sizeof(T) == 4)
+        if (!p.first && !p.imp_only && p.nfix < 0 && pair_eligible(p.Nth)) return launch_pair_step(p, 1, st);
     const int seg = implicit_seg(p.Nth);
     const int v = seg == kSegNarrow ? 0 : (seg == kSeg ? 1 : 2);
     auto fn = v == 0 ? k_split_step<T, kSegNarrow> : (v == 1 ? k_split_step<T, kSeg> : k_split_step<T, kSegWide>);
@@ -636,6 +708,8 @@ static void (*split2_fn(int Nth))(const StepParams<T>)
 template <typename T>
 int split2_blocks_per_sm(int Nth, int threads, size_t smem)
 {
+    if constexpr (sizeof(T) == 4)
+        if (pair_eligible(Nth)) return pair_blocks_per_sm(2, smem);
     auto fn = split2_fn<T>(Nth);
     if (smem_limit_max((const void *)fn) != cudaSuccess) {
         cudaGetLastError();
@@ -653,6 +727,8 @@ template <typename T>
 cudaError_t launch_split_step2(const StepParams<T> &p, int threads, size_t smem, cudaStream_t st)
 {
     if (p.first || p.imp_only) return cudaErrorInvalidValue;   // two full steps only
+    if constexpr (sizeof(T) == 4)
+        if (pair_eligible(p.Nth)) return launch_pair_step(p, 2, st);
     auto fn = split2_fn<T>(p.Nth);
     cudaError_t e = smem_limit_max((const void *)fn);
     if (e != cudaSuccess) return e;
@@ -672,12 +748,19 @@ static void (*split3_fn(int Nth))(const StepParams<T>)
 template <typename T>
 size_t split3_smem_bytes(int tile_rows, int Nth)
 {
-    return split_smem_plan(tile_rows + 6, Nth, (int)sizeof(T)).total + 2 * (size_t)Nth * sizeof(typename V2<T>::t);
+    if (sizeof(T) == 4 && pair_eligible(Nth)) {
+        // (a first step runs the one-step kernel at the same height)
+        const size_t pm = pair_smem_bytes(tile_rows, Nth, 3), sm = split_smem_bytes<T>(tile_rows, Nth);
+        return pm > sm ? pm : sm;
+    }
+    return split_smem_plan(tile_rows + 6, Nth, (int)sizeof(T)).total;
 }
 
 template <typename T>
 int split3_blocks_per_sm(int Nth, int threads, size_t smem)
 {
+    if constexpr (sizeof(T) == 4)
+        if (pair_eligible(Nth)) return pair_blocks_per_sm(3, smem);
     auto fn = split3_fn<T>(Nth);
     if (smem_limit_max((const void *)fn) != cudaSuccess) {
         cudaGetLastError();
@@ -695,6 +778,8 @@ template <typename T>
 cudaError_t launch_split_step3(const StepParams<T> &p, int threads, size_t smem, cudaStream_t st)
 {
     if (p.first || p.imp_only) return cudaErrorInvalidValue;   // three full steps only
+    if constexpr (sizeof(T) == 4)
+        if (pair_eligible(p.Nth)) return launch_pair_step(p, 3, st);
     auto fn = split3_fn<T>(p.Nth);
     cudaError_t e = smem_limit_max((const void *)fn);
     if (e != cudaSuccess) return e;

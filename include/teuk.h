@@ -196,12 +196,10 @@ int teuk_kernel_config(const teuk_ctx *ctx, int *persistent, int *consumer_threa
                        int *steps_per_launch);
 
 /* Measured tile autotuner.  Ranks the launch configurations that fit on the
- * device (tile heights of the tiled kernel with one or two steps per launch,
- * the pipelined kernel, and tile height x consumer count of the persistent
- * kernel) by a wave-quantisation cost model, times the best four of each
- * kind, and the tiled kernel with three steps per launch at the heights of
- * the four two-step candidates, for
- * trial_steps launches each on this grid (CUDA events on `stream`), in two
+ * device (tile heights of the tiled kernel with one, two or three steps per
+ * launch, the pipelined kernel, and tile height x consumer count of the
+ * persistent kernel) by a wave-quantisation cost model, times the best four
+ * of each kind for trial_steps launches each on this grid (CUDA events on `stream`), in two
  * interleaved rounds, and keeps the fastest per time step (a candidate's
  * better round).  The trials overwrite the
  * state: afterwards the field is zero at step 0 and the waveform ring buffer
@@ -338,7 +336,9 @@ int teuk_apply_step_sample(teuk_ctx *ctx, const void *d_in, void *d_out, int64_t
                            void *stream);
 
 /* One waveform sample into d_h (one complex double, device): E d_s if
- * physical, else E C_{dt/2} d_s; the same FP64 sum the steps write. */
+ * physical, else E C_{dt/2} d_s: up to FP64 rounding (FP64: the adjoint
+ * vector C_{dt/2}^H E^H 1 times d_s's extraction row) the sample the steps
+ * write. */
 int teuk_apply_sample(teuk_ctx *ctx, const void *d_s, int physical, void *d_h, void *stream);
 
 /* Device workspace of teuk_adjoint_step, teuk_adjoint_step_spin and
@@ -346,16 +346,15 @@ int teuk_apply_sample(teuk_ctx *ctx, const void *d_s, int physical, void *d_h, v
  * doubles accumulate the parameter derivatives (see teuk_adjoint_step and
  * teuk_adjoint_step_spin); zero them before a backward sweep.  In FP64 its
  * tail holds the coefficient planes teuk_adjoint_prepare writes (for an
- * Nr x Ntheta grid 17 Nr Ntheta + 8 (2 Nr - 1) Ntheta doubles). */
+ * Nr x Ntheta grid about 17 Nr Ntheta doubles). */
 int teuk_adjoint_workspace_bytes(const teuk_ctx *ctx, size_t *bytes);
 
-/* Fills the workspace's coefficient planes for teuk_adjoint_step_spin (FP64
- * contexts; FP32 contexts form them in place and only record d_ws): the
- * coefficients of the full step's implicit stage and Lax-Wendroff stages
- * (Eqs. 13-14, the implicit reading of S) at every grid element, and their
- * exact spin derivatives, formed by the same device functions the step
- * uses (so the adjoint reads bit for bit the coefficients the forward step
- * forms).  Asynchronous on `stream`.  The
+/* Fills the workspace's coefficient planes for the adjoint steps (FP64
+ * contexts; FP32 contexts form them in place and only record d_ws): at every
+ * grid element the exact spin derivatives of the full step's implicit stage
+ * and Lax-Wendroff stages (Eqs. 13-14, the implicit reading of S) and the
+ * products and scan levels of the transposed solves; the coefficients
+ * themselves are the forward step's own.  Asynchronous on `stream`.  The
  * context remembers d_ws; teuk_adjoint_step_spin with another workspace
  * returns TEUK_E_STATE.  Keep the planes unmodified between the calls;
  * after writing over them (or after reusing the memory), call this again.

@@ -1,7 +1,7 @@
 // teuk_adjoint.cu -- the step's waveform sample as an operator, the Hermitian
 // adjoint of one split-scheme step with the source-parameter derivatives,
 // and deterministic FP64 inner products (gradients of waveform losses).
-#include "teuk_dev.cuh"
+#include "teuk_adjoint.cuh"
 
 namespace teuk {
 namespace {
@@ -19,12 +19,11 @@ __device__ __forceinline__ int tile_of_block(int b, int nt, int i_ext, int tile_
     return b < nt ? b : b - nt;
 }
 
-// h = E u with u = s (physical) or u = C_{dt/2} s on the extraction row; one
-// warp.  The sum is the one the step kernels write to the waveform buffer.
-// The row's planes at (f, g); without h_out the sample goes to the ring buffer, as `step`'s.
+// The physical row u = C_{dt/2} s of the extraction row s (planes f, g), in
+// shared memory; one warp.
 template <typename T, int S>
-__device__ __forceinline__ void sample_row(const StepParams<T> &p, const typename V2<T>::t *f, const typename V2<T>::t *g,
-                                           int physical, double2 *h_out, long long step)
+__device__ __forceinline__ const typename V2<T>::t *physical_row(const StepParams<T> &p, const typename V2<T>::t *f,
+                                                                 const typename V2<T>::t *g)
 {
     typedef typename V2<T>::t c2;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -42,28 +41,31 @@ __device__ __forceinline__ void sample_row(const StepParams<T> &p, const typenam
     if (tid < NSF) xF[tid] = p.stab[(size_t)(2 * i) * NSF + tid];
     for (int k = tid; k < NTF * N; k += 32) xTh[k] = p.thtab[k];
     __syncwarp();
-    if (!physical) {
-        const int G = p.group;
-        const bool mine = tid < G;
-        const bool active = mine && i >= 1 && i <= Nr - 2;
-        implicit_row_one<T, S>(p.half, xPhi, xPi, i, xF, xTh, xTh2, N, active, mine, tid % G, G, p.vec != 0,
-                               p.half.plan[i]);
-        __syncwarp();
-    }
-    if (!h_out) {
-        extract_warp<T>(p, xPhi, step);
-        return;
-    }
-    double2 h = sample_warp<T>(p, xPhi);
-    if (tid == 0) *h_out = h;
+    const int G = p.group;
+    const bool mine = tid < G;
+    const bool active = mine && i >= 1 && i <= Nr - 2;
+    implicit_row_one<T, S>(p.half, xPhi, xPi, i, xF, xTh, xTh2, N, active, mine, tid % G, G, p.vec != 0, p.half.plan[i]);
+    __syncwarp();
+    return xPhi;
 }
 
+// h = E s (physical) or E C_{dt/2} s of the extraction row of s, as the step
+// kernels form it (see seed_dot).
 template <typename T, int S>
 __global__ void __launch_bounds__(32) k_sample(const StepParams<T> p, const typename V2<T>::t *s, int physical,
                                                double2 *h_out)
 {
     const size_t o = (size_t)p.i_ext * p.Nth;
-    sample_row<T, S>(p, s + o, s + (size_t)p.Nr * p.Nth + o, physical, h_out, 0);
+    const typename V2<T>::t *f = s + o, *g = f + (size_t)p.Nr * p.Nth;
+    double2 h;
+    if (physical) {
+        h = sample_warp<T>(p, f);
+    } else if constexpr (sizeof(T) == 8) {
+        h = seed_dot<T>(p, f, g);
+    } else {
+        h = sample_warp<T>(p, physical_row<T, S>(p, f, g));
+    }
+    if (threadIdx.x == 0) *h_out = h;
 }
 
 // CTA (b, instance): the b-th step after ctl->sampled, if it has been taken.
@@ -76,7 +78,7 @@ __device__ __forceinline__ void sample_step(const StepParams<T> &p)
     // (only the last wave_cap samples stay in the ring: two steps of one slot do not race)
     if (n <= n1 && n > n1 - p.wave_cap) {
         const typename V2<T>::t *r = p.raw + (size_t)(n % kRawSlots) * 2 * p.Nth;
-        sample_row<T, S>(p, r, r + p.Nth, 0, nullptr, n);
+        extract_warp<T>(p, physical_row<T, S>(p, r, r + p.Nth), n);
     }
     __syncwarp();
     if (threadIdx.x == 0) {
@@ -102,26 +104,6 @@ __global__ void __launch_bounds__(32) k_sample_steps_batch(const StepParams<T> *
         reinterpret_cast<int *>(&sp)[k] = reinterpret_cast<const int *>(params + blockIdx.y)[k];
     __syncwarp();
     sample_step<T, S>(sp);
-}
-
-// Adds conj(lam) * coef * (unit source) * phase to the amplitude sum cA and
-// conj(lam) * coef * (source) * (rho d r0*/d r0 - i m Omega' t) to the orbit
-// sum cr (rho = (r* - r0*)/sigma_r^2): the derivatives of the source term
-// A F_pref G(r*, theta) e^{-i m Omega t} with respect to A and r0.
-template <typename T>
-__device__ __forceinline__ void source_grad(const StepParams<T> &p, typename V2<T>::t lam, double coef,
-                                            typename V2<T>::t u, double2 ph, double rs, double t, double2 &cA,
-                                            double2 &cr)
-{
-    const double lr = (double)lam.x, li = -(double)lam.y;             // conj(lam)
-    const double ur = (double)u.x * ph.x - (double)u.y * ph.y, ui = (double)u.x * ph.y + (double)u.y * ph.x;
-    const double vr = coef * (lr * ur - li * ui), vi = coef * (lr * ui + li * ur);   // conj(lam) coef U ph
-    cA.x += vr;
-    cA.y += vi;
-    const double fr = p.amp_re * vr - p.amp_im * vi, fi = p.amp_re * vi + p.amp_im * vr;   // times A
-    const double zr = (rs - p.rs0) * p.inv_sig_r2 * p.drs0_dr0, zi = -p.m_dOmega * t;
-    cr.x += fr * zr - fi * zi;
-    cr.y += fr * zi + fi * zr;
 }
 
 // Hermitian adjoint of one split step s_n -> s_{n+1} = LW_n C_h s_n (h = dt;
@@ -371,23 +353,6 @@ __global__ void __launch_bounds__(256, 1) k_adjoint_step(const StepParams<T> p, 
 // spin derivative (dstab, exact forward-mode derivatives of the FP64
 // table generator, r(r*; a) by implicit differentiation of Eq. 2).
 
-// The source term of a stage, S = F ph (ph: the scaled phase), as the
-// forward step forms it, and dS/da: F = SRC sg (SR2 GTH + GA2) through its
-// factors and 1/Sigma^2, the phase through Omega(a) (mdt = m t dOmega/da).
-template <typename T>
-__device__ __forceinline__ void src_da(const T *f, const T *df, T sg, T dsg, T gth, T ga2, T dga2,
-                                       typename V2<T>::t ph, T mdt, typename V2<T>::t &Sv, typename V2<T>::t &dS)
-{
-    typedef typename V2<T>::t c2;
-    const T X = fma(f[SF_SR2], gth, ga2), dX = fma(df[SF_SR2], gth, dga2);
-    const c2 src = cmk<c2>(f[SF_SRE], f[SF_SIM]), dsrc = cmk<c2>(df[SF_SRE], df[SF_SIM]);
-    const c2 F = cscale<c2>(sg * X, src);
-    const c2 dF = cadd(cscale<c2>(sg * X, dsrc), cscale<c2>(fma(dsg, X, sg * dX), src));
-    Sv = cmul(F, ph);
-    // d/da e^{-i m Omega t} = -i m t (dOmega/da) e^{-i m Omega t}
-    dS = cadd(cmul(dF, ph), cmk<c2>(Sv.y * mdt, -Sv.x * mdt));
-}
-
 // Loads the lane's segment of a row (zero past its end).
 template <typename T, int S>
 __device__ __forceinline__ void seg_load(const typename V2<T>::t *row, int j0, int len, bool vec,
@@ -406,13 +371,12 @@ __device__ __forceinline__ void seg_load(const typename V2<T>::t *row, int j0, i
 // exit), and this lane's part of <mu, dC_h u> from the forward stage values
 // (u1f, u1g) = U1 and (u2f, u2g) = U2 of the same row; f, df: the row's
 // step-table entry and its spin derivative.
-template <typename T, int S, bool MAT = false, bool SPIN = true>
+template <typename T, int S, bool SPIN = true>
 __device__ double implicit_row_adj_spin(const ImpConst<T> &K, typename V2<T>::t *lf, typename V2<T>::t *lg,
                                         const typename V2<T>::t *u1f, const typename V2<T>::t *u1g,
                                         const typename V2<T>::t *u2f, const typename V2<T>::t *u2g,
                                         const typename V2<T>::t *prow, const T *f, const T *df, const T *th, int N,
-                                        bool active, bool in_tile, int g, int G, bool vec,
-                                        const AdjPlanes<T> *A = nullptr, int gi = 0)
+                                        bool active, bool in_tile, int g, int G, bool vec)
 {
     typedef typename V2<T>::t c2;
     const c2 zero = cmk<c2>(T(0), T(0));
@@ -424,10 +388,7 @@ __device__ double implicit_row_adj_spin(const ImpConst<T> &K, typename V2<T>::t 
     const T gh = K.gh, c = K.h1g;
     ImpCoef<T, S> C;
     c2 w[S], y[S];   // mu_Phi, mu_Pi
-    if constexpr (MAT)
-        imp_load_mat<T, S>(A->m, lf, lg, prow, gi, N, len, j0, vec, C, w, y);
-    else
-        imp_load<T, S>(K, lf, lg, prow, f, th, N, len, j0, vec, C, w, y);
+    imp_load<T, S>(K, lf, lg, prow, f, th, N, len, j0, vec, C, w, y);
     // multipliers of M^H = U^H L^H and the rows of W^H (qap_{j-1}, conj(dg_j), qam_{j+1})
     c2 fm[S], pm[S], bm[S];
     T qapp[S], qamn[S];
@@ -492,22 +453,7 @@ __device__ double implicit_row_adj_spin(const ImpConst<T> &K, typename V2<T>::t 
     // derivative coefficients dW (dqam, ddg, dqap) and dc_t of the row
     c2 ddg[S], dct[S];
     T dqam[S], dqap[S];
-    if constexpr (MAT) {
-#pragma unroll
-        for (int k = 0; k < S; ++k) {
-            T v[8];
-            if (k < len) {
-                vload<8>(v, A->dimp + ((size_t)gi * N + j0 + k) * 8);
-            } else {
-#pragma unroll
-                for (int q = 0; q < 8; ++q) v[q] = T(0);
-            }
-            ddg[k] = cmk<c2>(v[0], v[1]);
-            dct[k] = cmk<c2>(v[2], v[3]);
-            dqam[k] = v[4];
-            dqap[k] = v[5];
-        }
-    } else {
+    {
         const ImpRow<T> r = imp_row(K, f);
         T fr[8], dfr[8];
         vload<8>(fr, f);
@@ -523,7 +469,7 @@ __device__ double implicit_row_adj_spin(const ImpConst<T> &K, typename V2<T>::t 
                 ddg[k] = dct[k] = zero;
             }
         }
-    }
+        }
     // Q = dW x_Phi + dc_t x_Pi for the stage values
     auto apply_dQ = [&](const c2 (&xf_)[S], const c2 (&xp_)[S], c2 (&out)[S]) {
         c2 vl = shfl_up_c(xf_[S - 1], 1, G), vr = shfl_down_c(xf_[0], 1, G);
@@ -558,6 +504,74 @@ __device__ double implicit_row_adj_spin(const ImpConst<T> &K, typename V2<T>::t 
     return acc;
 }
 
+// The sample's adjoint C_{dt/2}^H E^H 1 on the extraction row, [2][Nth], for
+// the weights as they are; one warp.
+template <int S>
+__global__ void __launch_bounds__(32) k_seed(const StepParams<double> p, double2 *seed)
+{
+    typedef double T;
+    typedef double2 c2;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int N = p.Nth, Nr = p.Nr, i = p.i_ext, tid = threadIdx.x, G = p.group;
+    c2 *xF = (c2 *)smem_raw, *xG = xF + ((N + 1) & ~1);
+    T *f = (T *)(xG + ((N + 1) & ~1)), *th = f + NSF;
+    for (int j = tid; j < N; j += 32) {
+        xF[j] = cmk<c2>((T)p.w[j], T(0));
+        xG[j] = cmk<c2>(T(0), T(0));
+    }
+    if (tid < NSF) f[tid] = p.stab[(size_t)(2 * i) * NSF + tid];
+    for (int k = tid; k < NTF * N; k += 32) th[k] = p.thtab[k];
+    __syncwarp();
+    const bool mine = tid < G, active = mine && i >= 1 && i <= Nr - 2;
+    implicit_row_adj_spin<T, S, false>(p.half, xF, xG, nullptr, nullptr, nullptr, nullptr, p.half.piv + (size_t)i * N, f,
+                                       nullptr, th, N, active, mine, tid % G, G, p.vec != 0);
+    __syncwarp();
+    for (int j = tid; j < N; j += 32) {
+        seed[j] = make_double2((double)xF[j].x, (double)xF[j].y);
+        seed[N + j] = make_double2((double)xG[j].x, (double)xG[j].y);
+    }
+}
+
+// The sample's spin derivative as a vector on the extraction row: d(E C_{dt/2})/da
+// of the unit state blockIdx.x (plane, theta), contracted with 1 and with i.
+template <int S>
+__global__ void __launch_bounds__(32) k_delta(const StepParams<double> p, double2 *delta)
+{
+    typedef double2 c2;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int N = p.Nth, Nr = p.Nr, i = p.i_ext, tid = threadIdx.x, G = p.group;
+    c2 *sF = (c2 *)smem_raw, *sG = sF + N, *aF = sG + N, *aG = aF + N, *xF = aG + N, *xG = xF + N;
+    double *f = (double *)(xG + N), *df = f + NSF, *th = df + NSF;
+    const c2 zero = cmk<c2>(0.0, 0.0);
+    for (int j = tid; j < N; j += 32) {
+        sF[j] = cmk<c2>((int)blockIdx.x == j ? 1.0 : 0.0, 0.0);
+        sG[j] = cmk<c2>((int)blockIdx.x == N + j ? 1.0 : 0.0, 0.0);
+    }
+    if (tid < NSF) {
+        f[tid] = p.stab[(size_t)(2 * i) * NSF + tid];
+        df[tid] = p.dstab[(size_t)(2 * i) * NSF + tid];
+    }
+    for (int k = tid; k < NTF * N; k += 32) th[k] = p.thtab[k];
+    __syncwarp();
+    const bool mine = tid < G, active = mine && i >= 1 && i <= Nr - 2;
+    implicit_row_fwd<double, S>(p.half, sF, sG, p.half.piv + (size_t)i * N, f, th, N, active, mine, tid % G, G, p.vec != 0,
+                                active ? p.half.plan[i] : 0, aF, aG);
+    double d[2];
+    for (int q = 0; q < 2; ++q) {
+        __syncwarp();
+        for (int j = tid; j < N; j += 32) {
+            xF[j] = q ? cmk<c2>(0.0, p.w[j]) : cmk<c2>(p.w[j], 0.0);
+            xG[j] = zero;
+        }
+        __syncwarp();
+        d[q] = implicit_row_adj_spin<double, S>(p.half, xF, xG, aF, aG, sF, sG, p.half.piv + (size_t)i * N, f, df, th, N,
+                                                active, mine, tid % G, G, p.vec != 0);
+        if (!active) d[q] = 0.0;
+        for (int o = 16; o > 0; o >>= 1) d[q] += __shfl_xor_sync(0xffffffffu, d[q], o);
+    }
+    if (tid == 0) delta[blockIdx.x] = make_double2(d[0], d[1]);
+}
+
 // Adjoint step with the spin derivative: lam_n as k_adjoint_step (here
 // through the block form of C_h^H), the source derivatives (amplitude and
 // r0) as k_adjoint_step, and the step's part of dL/da.  p.uin = lam_{n+1},
@@ -565,12 +579,10 @@ __device__ double implicit_row_adj_spin(const ImpConst<T> &K, typename V2<T>::t 
 // part[NPART b + (0 .. 4)] = (Re cA, Im cA, Re cr, Im cr, spin term).
 // Tile rows i0-1 .. i0+TR: lam_{n+1} (lF, lG), the stage values U2 = C_h s_n
 // (vF, vG) and U1 (u1F, u1G), the midpoint adjoints (mF, mG).
-constexpr int kNPart = 6;
-
-template <typename T, int S, bool MAT, bool SPIN>
+template <typename T, int S>
 __global__ void __launch_bounds__(256, 1) k_adjoint_spin(const StepParams<T> p, const typename V2<T>::t *sin,
                                                          const typename V2<T>::t *tape, const double2 *gseed,
-                                                         const AdjPlanes<T> A, double *part)
+                                                         double *part)
 {
     typedef typename V2<T>::t c2;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -603,7 +615,7 @@ __global__ void __launch_bounds__(256, 1) k_adjoint_spin(const StepParams<T> p, 
     T *sDSt = sSt + (2 * R - 1) * NSF;
     T *sTh = sDSt + (2 * R - 1) * NSF;
     unsigned long long *sTh2 = (unsigned long long *)(sTh + NTF * N);   // FP32 rows of 128 < Ntheta <= 256 (teuk_pair.cuh)
-    if constexpr (kPaired<T, S> && SPIN) pair_th_fill(sTh2, p.thtab, N, tid, NT);
+    if constexpr (kPaired<T, S>) pair_th_fill(sTh2, p.thtab, N, tid, NT);
 
     // ---- lam_{n+1} and s_n (with a tape: the forward stage values U2 and U1
     // the forward step recorded) on rows i0-1 .. i0+TR, the step tables,
@@ -617,8 +629,7 @@ __global__ void __launch_bounds__(256, 1) k_adjoint_spin(const StepParams<T> p, 
             const size_t qf = (size_t)gi * N + j, qg = ((size_t)Nr + gi) * N + j;
             a = p.uin[qf];
             b = p.uin[qg];
-            if (!SPIN) {
-            } else if (tape) {
+            if (tape) {
                 sa = tp2[qf];
                 sb = tp2[qg];
                 ua = tp1[qf];
@@ -651,7 +662,7 @@ __global__ void __launch_bounds__(256, 1) k_adjoint_spin(const StepParams<T> p, 
     __syncthreads();
 
     // ---- forward implicit stage on all rows: (vF, vG) <- U2 = C_h s_n, (u1F, u1G) <- U1
-    if (SPIN && !tape) {
+    if (!tape) {
         const int rpp = NT / G;
         for (int base = 0; base < R; base += rpp) {
             if (base + (tid & ~31) / G >= R) continue;   // no row for this warp
@@ -665,10 +676,9 @@ __global__ void __launch_bounds__(256, 1) k_adjoint_spin(const StepParams<T> p, 
                                        sSt + 2 * interior_row(lrc, i0 - 1, Nr) * NSF, sTh, sTh2, N, active, in_tile, g, G,
                                        vec, active ? K.plan[gi] : 0, u1F + lrc * P, u1G + lrc * P);
             else
-                implicit_row_fwd<T, S, MAT>(K, vF + lrc * P, vG + lrc * P, K.piv + (size_t)(active ? gi : 1) * N,
-                                            sSt + 2 * lrc * NSF, sTh, N, active, in_tile, g, G, vec,
-                                            active ? K.plan[gi] : 0, &A.m, active ? gi : 1, u1F + lrc * P,
-                                            u1G + lrc * P);
+                implicit_row_fwd<T, S>(K, vF + lrc * P, vG + lrc * P, K.piv + (size_t)(active ? gi : 1) * N,
+                                       sSt + 2 * lrc * NSF, sTh, N, active, in_tile, g, G, vec, active ? K.plan[gi] : 0,
+                                       u1F + lrc * P, u1G + lrc * P);
         }
     }
     __syncthreads();
@@ -691,22 +701,7 @@ __global__ void __launch_bounds__(256, 1) k_adjoint_spin(const StepParams<T> p, 
     // beta, kap, 1/Sigma^2 and their spin derivatives at tile position e
     // (2 lr: node, 2 k + 1: half node) and theta j
     auto lwc = [&](int e, int j, T S2, T Cc) -> LwDa<T> {
-        if constexpr (MAT) {
-            const size_t o = ((size_t)(2 * (i0 - 1) + e) * N + j) * 4;
-            T v[4], dv[4];
-            vload<4>(v, A.m.lw + o);
-            vload<4>(dv, A.dlw + o);
-            LwDa<T> r;
-            r.beta = v[0];
-            r.kap = cmk<c2>(v[1], v[2]);
-            r.sg = v[3];
-            r.dbeta = dv[0];
-            r.dkap = cmk<c2>(dv[1], dv[2]);
-            r.dsg = dv[3];
-            return r;
-        } else {
-            return lw_coef_da<T>(sSt + e * NSF, sDSt + e * NSF, S2, Cc);
-        }
+        return lw_coef_da<T>(sSt + e * NSF, sDSt + e * NSF, S2, Cc);
     };
 
     // ---- adjoints of the midpoints k = 0 .. R-2, and their spin terms
@@ -735,7 +730,7 @@ __global__ void __launch_bounds__(256, 1) k_adjoint_spin(const StepParams<T> p, 
                     source_grad<T>(p, wG, (double)hdtT, p.patchu[((size_t)pr * 2 + 1) * N + j], ph1,
                                    p.rs_min64 + ((double)gl + 0.5) * p.drs64, t1, cA, cr);
             }
-            if constexpr (SPIN) {
+            {
                 // the forward midpoint from U2, as the step forms it (stored for
                 // the node stage's spin terms), and this midpoint's spin term
                 const LwDa<T> h = lwc(2 * k + 1, j, S2, Cc);
@@ -790,7 +785,7 @@ __global__ void __launch_bounds__(256, 1) k_adjoint_spin(const StepParams<T> p, 
                     source_grad<T>(p, lg, (double)dtT, p.patchu[((size_t)pr * 2) * N + j], ph2,
                                    p.rs_min64 + (double)gi * p.drs64, t2, cA, cr);
             }
-            if constexpr (SPIN) {
+            {
             // spin terms of the node stage: d(Phi') = -dbeta dMf,
             // d(Pi') = dbeta dMg + dkap dMf + dS, dM the forward midpoint difference
             const LwDa<T> nd = lwc(2 * lr, j, S2, Cc);
@@ -823,10 +818,10 @@ __global__ void __launch_bounds__(256, 1) k_adjoint_spin(const StepParams<T> p, 
             const int gi = i0 - 1 + lr;
             const bool active = in_tile && gi >= 1 && gi <= Nr - 2;
             const int lrc = in_tile ? lr : 1;
-            const double d = implicit_row_adj_spin<T, S, MAT, SPIN>(
+            const double d = implicit_row_adj_spin<T, S>(
                 K, lF + lrc * P, lG + lrc * P, u1F + lrc * P, u1G + lrc * P, vF + lrc * P, vG + lrc * P,
                 K.piv + (size_t)(active ? gi : 1) * N, sSt + 2 * lrc * NSF, sDSt + 2 * lrc * NSF, sTh, N, active,
-                in_tile, g, G, vec, &A, active ? gi : 1);
+                in_tile, g, G, vec);
             if (active) spin += d;
         }
     }
@@ -845,8 +840,7 @@ __global__ void __launch_bounds__(256, 1) k_adjoint_spin(const StepParams<T> p, 
                 const double w = p.w[j];
                 xF[j] = cmk<c2>((T)(w * gv.x), (T)(w * gv.y));
                 xG[j] = zero;
-                if (!SPIN) {
-                } else if (tape) {
+                if (tape) {
                     sF[j] = tape[tape_x_off(Nr, N) + j];
                     sG[j] = tape[tape_x_off(Nr, N) + N + j];
                 } else {
@@ -859,11 +853,10 @@ __global__ void __launch_bounds__(256, 1) k_adjoint_spin(const StepParams<T> p, 
                 const bool mine = tid < G;
                 const bool active = mine && p.i_ext >= 1 && p.i_ext <= Nr - 2;
                 // forward C_{dt/2} on the row of s_n: (sF, sG) <- U2, (aF, aG) <- U1
-                if constexpr (SPIN)
-                    implicit_row_one<T, S>(p.half, sF, sG, p.i_ext, sSt + 2 * lx * NSF, sTh, sTh2, N, active, mine, tid % G,
+                implicit_row_one<T, S>(p.half, sF, sG, p.i_ext, sSt + 2 * lx * NSF, sTh, sTh2, N, active, mine, tid % G,
                                            G, vec, active ? p.half.plan[p.i_ext] : 0, aF, aG);
                 __syncwarp();
-                const double d = implicit_row_adj_spin<T, S, false, SPIN>(p.half, xF, xG, aF, aG, sF, sG,
+                const double d = implicit_row_adj_spin<T, S>(p.half, xF, xG, aF, aG, sF, sG,
                                                              p.half.piv + (size_t)p.i_ext * N, sSt + 2 * lx * NSF,
                                                              sDSt + 2 * lx * NSF, sTh, N, active, mine, tid % G, G,
                                                              vec);
@@ -1004,6 +997,27 @@ cudaError_t launch_sample(const StepParams<T> &p, const typename V2<T>::t *s, in
     return cudaGetLastError();
 }
 
+cudaError_t launch_seed(const StepParams<double> &p, double2 *seed, cudaStream_t st)
+{
+    const int seg = implicit_seg(p.Nth);
+    auto fn = seg == kSegNarrow ? k_seed<kSegNarrow> : (seg == kSeg ? k_seed<kSeg> : k_seed<kSegWide>);
+    cudaError_t e = smem_limit_max((const void *)fn);
+    if (e != cudaSuccess) return e;
+    fn<<<1, 32, sample_smem_bytes<double>(p.Nth), st>>>(p, seed);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_delta(const StepParams<double> &p, double2 *delta, cudaStream_t st)
+{
+    const int seg = implicit_seg(p.Nth);
+    auto fn = seg == kSegNarrow ? k_delta<kSegNarrow> : (seg == kSeg ? k_delta<kSeg> : k_delta<kSegWide>);
+    cudaError_t e = smem_limit_max((const void *)fn);
+    if (e != cudaSuccess) return e;
+    const size_t smem = 6 * (size_t)p.Nth * sizeof(double2) + (2 * (size_t)NSF + (size_t)NTF * p.Nth) * sizeof(double);
+    fn<<<2 * p.Nth, 32, smem, st>>>(p, delta);
+    return cudaGetLastError();
+}
+
 template <typename T>
 cudaError_t launch_sample_steps(const StepParams<T> &p, int pending, cudaStream_t st)
 {
@@ -1070,57 +1084,29 @@ size_t adjoint_spin_smem_bytes(int tile_rows, int Nth)
            pair_th_bytes(Nth, (int)sizeof(T));
 }
 
-template <typename T, bool MAT, bool SPIN = true>
-static void (*adjoint_spin_fn(int Nth))(const StepParams<T>, const typename V2<T>::t *, const typename V2<T>::t *,
-                                        const double2 *, const AdjPlanes<T>, double *)
+cudaError_t launch_part_reduce(const double *part, int nblk, double *acc, cudaStream_t st)
 {
-    const int seg = implicit_seg(Nth);
-    return seg == kSegNarrow ? k_adjoint_spin<T, kSegNarrow, MAT, SPIN>
-                             : (seg == kSeg ? k_adjoint_spin<T, kSeg, MAT, SPIN> : k_adjoint_spin<T, kSegWide, MAT, SPIN>);
+    k_part_reduce6<<<1, 32, 0, st>>>(part, nblk, acc);
+    return cudaGetLastError();
 }
 
 template <typename T>
 cudaError_t launch_adjoint_spin(const StepParams<T> &p, int tile_rows, const typename V2<T>::t *sin,
-                                const typename V2<T>::t *tape, const double2 *gseed, const AdjPlanes<T> &A,
-                                double *part, double *acc, cudaStream_t st)
+                                const typename V2<T>::t *tape, const double2 *gseed, double *part, double *acc,
+                                cudaStream_t st)
 {
-    // the planes (FP64) hold the full step's coefficients; a first step
-    // (dt/2) and the FP32 adjoint form their own from the tables
-    auto fn = adjoint_spin_fn<T, false>(p.Nth);
-    if constexpr (sizeof(T) == 8)
-        if (!p.first) fn = adjoint_spin_fn<T, true>(p.Nth);
+    const int seg = implicit_seg(p.Nth);
+    auto fn = seg == kSegNarrow ? k_adjoint_spin<T, kSegNarrow>
+                                : (seg == kSeg ? k_adjoint_spin<T, kSeg> : k_adjoint_spin<T, kSegWide>);
     cudaError_t e = smem_limit_max((const void *)fn);
     if (e != cudaSuccess) return e;
     StepParams<T> q = p;
     q.tile_rows = tile_rows;
     const int grid = adjoint_grid<T>(p.Nr, tile_rows);
-    fn<<<grid, 256, adjoint_spin_smem_bytes<T>(tile_rows, p.Nth), st>>>(q, sin, tape, gseed, A, part);
+    fn<<<grid, 256, adjoint_spin_smem_bytes<T>(tile_rows, p.Nth), st>>>(q, sin, tape, gseed, part);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    k_part_reduce6<<<1, 32, 0, st>>>(part, grid, acc);
-    return cudaGetLastError();
-}
-
-template <typename T>
-cudaError_t launch_adjoint_planes(const StepParams<T> &p, int tile_rows, const double2 *gseed, const AdjPlanes<T> &A,
-                                  double *part, double *acc, cudaStream_t st)
-{
-    if constexpr (sizeof(T) != 8) {
-        return cudaErrorInvalidValue;
-    } else {
-        if (p.first) return cudaErrorInvalidValue;
-        auto fn = adjoint_spin_fn<T, true, false>(p.Nth);
-        cudaError_t e = smem_limit_max((const void *)fn);
-        if (e != cudaSuccess) return e;
-        StepParams<T> q = p;
-        q.tile_rows = tile_rows;
-        const int grid = adjoint_grid<T>(p.Nr, tile_rows);
-        fn<<<grid, 256, adjoint_spin_smem_bytes<T>(tile_rows, p.Nth), st>>>(q, nullptr, nullptr, gseed, A, part);
-        e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
-        k_part_reduce6<<<1, 32, 0, st>>>(part, grid, acc);
-        return cudaGetLastError();
-    }
+    return launch_part_reduce(part, grid, acc, st);
 }
 
 template <typename T>
@@ -1152,13 +1138,9 @@ template cudaError_t launch_adjoint_step<double>(const StepParams<double> &, int
 template size_t adjoint_spin_smem_bytes<float>(int, int);
 template size_t adjoint_spin_smem_bytes<double>(int, int);
 template cudaError_t launch_adjoint_spin<float>(const StepParams<float> &, int, const float2 *, const float2 *,
-                                                const double2 *, const AdjPlanes<float> &, double *, double *,
-                                                cudaStream_t);
+                                                const double2 *, double *, double *, cudaStream_t);
 template cudaError_t launch_adjoint_spin<double>(const StepParams<double> &, int, const double2 *, const double2 *,
-                                                 const double2 *, const AdjPlanes<double> &, double *, double *,
-                                                 cudaStream_t);
-template cudaError_t launch_adjoint_planes<double>(const StepParams<double> &, int, const double2 *,
-                                                   const AdjPlanes<double> &, double *, double *, cudaStream_t);
+                                                 const double2 *, double *, double *, cudaStream_t);
 template cudaError_t launch_dot<float>(const float2 *, const float2 *, const float2 *, size_t, double *, double2 *,
                                        cudaStream_t);
 template cudaError_t launch_dot<double>(const double2 *, const double2 *, const double2 *, size_t, double *,

@@ -55,6 +55,8 @@ struct teuk_ctx {
     // the state output (C_{dt/2} only)
     int tile_rows, threads;
     size_t smem;
+    int one_rows;            // tile height of steps applied to caller buffers (one step per launch)
+    size_t one_smem;
     int persist, nc, grid;
     int pipe;                // the pipelined two-step kernel (grid persistent CTAs)
     size_t persist_smem;
@@ -62,6 +64,7 @@ struct teuk_ctx {
     int wait0;               // teuk_set_wait_limit (< 0: default bound)
     size_t smem2;            // shared memory of the two- or three-step kernel
     const void *adj_ws;      // adjoint workspace whose coefficient planes teuk_adjoint_prepare filled
+    int delta_ok;            // its delta vector is for the present weights
     // graphs, one per starting level
     cudaGraphExec_t graph[2];
     cudaStream_t graph_stream[2];
@@ -98,7 +101,10 @@ Layout make_layout(const teuk_grid_desc &d)
     }
     L.patch = off; off = align256(off + c2 * 2 * N * patch_rows);
     L.patchu = off; off = align256(off + c2 * 2 * N * patch_rows);
+    L.patchd = off;
+    if (!f32 && d.scheme == TEUK_SCHEME_SPLIT) off = align256(off + c2 * 2 * N * patch_rows);
     L.w = off; off = align256(off + sizeof(double) * N);
+    L.seed = off; off = align256(off + 2 * sizeof(double2) * N);
     L.ctl = off; off = align256(off + sizeof(Ctl));
     L.raw = off; off = align256(off + c2 * 2 * N * (size_t)kRawSlots);
     L.staging_elems = 0;
@@ -110,12 +116,12 @@ Layout make_layout(const teuk_grid_desc &d)
     }
     L.scratch = off;
     if (d.scheme == TEUK_SCHEME_LITERAL) off = align256(off + c2 * 2 * (Nr - 1) * N);
-    // FP64 split scheme: materialised coefficients (MatPlanes), three complex
-    // and three real planes [Nr][N], then the Lax-Wendroff planes [2Nr-1][N][4]
+    // FP64 split scheme: the full step's planes (StepPlanes), four complex and
+    // five real ones [Nr][N], then the stencil's [Nr][4][N] pairs
     L.mat = off;
     L.mat_bytes = 0;
     if (!f32 && d.scheme == TEUK_SCHEME_SPLIT) {
-        L.mat_bytes = align256(sizeof(double) * Nr * N * 9) + sizeof(double) * 4 * (2 * Nr - 1) * N;
+        L.mat_bytes = align256(sizeof(double) * Nr * N * kStepPlaneReals) + sizeof(double2) * kLwStencil * Nr * N;
         off = align256(off + L.mat_bytes);
     }
     L.total = off;
@@ -218,22 +224,33 @@ double host_atheta_bound(const teuk_grid_desc &d)
     return lam;
 }
 
-// Launch configurations of the split step and their model cost.
+// Launch configurations of the split step and their model cost, in us per
+// time step.
 //
-// Tiled kernel (256 threads, one tile per CTA): a tile of R = TR + 2 rows
-// costs about 0.6 Rpad + 0.4 R + 4 row-times, where Rpad rounds R up to
-// whole passes of the implicit phase (256 threads / G rows per pass) and the
-// 4 stands for load latency and barriers; k CTAs share an SM, so one wave
-// costs k times that and the grid needs ceil(tiles / (k SMs)) waves, with a
-// 20 % penalty for k = 1 (no second CTA to overlap memory with compute).
+// Tiled kernels (256 threads, one tile per CTA, ks steps per launch): step k
+// of a launch runs the implicit stage on TR + 2 (ks - k) rows and the
+// Lax-Wendroff stages on two rows fewer; a warp takes 32 / G rows of the
+// implicit stage at once.
+//   FP64: the FP64 pipe bounds it.  A scheduler starts one FP64 instruction
+//   per 64 cycles, so a step costs the busiest scheduler's count: per theta
+//   element of a lane's segment 57 (and 48 per segment for the scans) in the
+//   implicit stage, 26 per element in the Lax-Wendroff stages; 1.5 us of
+//   latency a step and 4.5 us a launch and wave come on top.  An SM's tiles
+//   share its pipes, so their counts add up.  (Model against measurement:
+//   16384 x 128, 36 rows, two steps 349 / 365 us; 1024 x 32, 7 rows, three
+//   steps 14 / 17.)
+//   FP32: 0.6 Rpad + 0.4 R row-times a step (Rpad: whole warps of rows), one
+//   row-time 0.188 us for 128 theta points, shared by the k CTAs of an SM,
+//   20 % more for k = 1 (no second CTA to overlap latency with), and 5 us a
+//   launch.  (16384 x 128, 28 rows, two steps 26 / 25 us; 65536 x 256, 36
+//   rows, three steps 206 / 203; 1024 x 32, 7 rows, three steps 3.9 / 5.6.)
+// The model leaves no tile of a grid half empty by accident: it counts waves
+// of the real SM count and occupancy.
 //
-// Persistent kernel (nc consumer threads + a producer warp, one CTA per SM,
-// tiles double-buffered): a CTA computes ceil(tiles / grid) tiles of
-// (0.6 Rpad + 0.4 R) (256 / nc) + 2 row-times each (Rpad in passes of
-// nc / G rows; the 2 for its barriers), plus the first tile's load.  Its
-// consumers move in lockstep between barriers, which costs about a factor
-// of two per row-time against the tiled kernel's two independent CTAs per
-// SM (measured on 16384 x 128 at equal tile height).
+// Pipelined and persistent kernels (see pipe_cand, persist_cand): measured
+// 20 to 100 % behind the tiled ones on every grid tried (16384 x 128 FP32 31
+// against 24.5 us, 1024 x 32 FP64 31.5 against 17.3), so their cost carries a
+// factor that keeps them out of the default choice; the autotuners time them.
 struct TileCand {
     double cost;             // model cost per time step
     int R;                   // tile_rows + 2
@@ -251,89 +268,57 @@ static int sm_count()
     return nsm;
 }
 
-// A tiled-kernel candidate of height TR (false if it does not fit).
-static bool tiled_cand(const teuk_ctx *c, int TR, int nsm, TileCand *out)
-{
-    const int N = (int)c->d.Ntheta;
-    const bool f32 = c->d.precision == TEUK_FP32;
-    const int threads = 256, R = TR + 2;
-    size_t sm = f32 ? split_smem_bytes<float>(TR, N) : split_smem_bytes<double>(TR, N);
-    if (sm > 227 * 1024) return false;
-    int k = f32 ? split_blocks_per_sm<float>(N, threads, sm) : split_blocks_per_sm<double>(N, threads, sm);
-    if (k < 1) return false;
-    const long long Nr = c->d.Nr;
-    long long tiles = (Nr + TR - 1) / TR;
-    long long waves = (tiles + (long long)k * nsm - 1) / ((long long)k * nsm);
-    int rpp = threads / implicit_group(N);
-    int rpad = ((R + rpp - 1) / rpp) * rpp;
-    double rows = 0.6 * rpad + 0.4 * R + 4.0;
-    out->cost = (double)waves * k * rows * (k == 1 ? 1.2 : 1.0);
-    out->R = R;
-    out->persist = 0;
-    out->nc = 0;
-    out->grid = (int)tiles;
-    out->ks = 1;
-    out->pipe = 0;
-    out->smem = sm;
-    return true;
-}
+// us of one row-time of the FP32 kernels (see above).
+static double row_time(int N) { return 0.188 * N / 128.0; }
 
-// A two-steps-per-launch candidate of height TR: per step, half of a tile
-// whose first step covers TR + 4 rows (implicit) and TR + 2 (LW) and whose
-// second covers TR + 2 and TR, with one load latency per two steps.
-static bool tiled2_cand(const teuk_ctx *c, int TR, int nsm, TileCand *out)
+// A tiled candidate of height TR with ks = 1, 2 or 3 steps per launch (false
+// if it does not fit).
+static bool tiled_cand(const teuk_ctx *c, int TR, int ks, int nsm, TileCand *out)
 {
     const int N = (int)c->d.Ntheta;
     const bool f32 = c->d.precision == TEUK_FP32;
     const int threads = 256;
-    size_t sm = f32 ? split2_smem_bytes<float>(TR, N) : split2_smem_bytes<double>(TR, N);
+    if (TR > kMaxTileRows - (ks == 3 ? 6 : 0)) return false;
+    size_t sm;
+    if (ks == 1) sm = f32 ? split_smem_bytes<float>(TR, N) : split_smem_bytes<double>(TR, N);
+    else if (ks == 2) sm = f32 ? split2_smem_bytes<float>(TR, N) : split2_smem_bytes<double>(TR, N);
+    else sm = f32 ? split3_smem_bytes<float>(TR, N) : split3_smem_bytes<double>(TR, N);
     if (sm > 227 * 1024) return false;
-    int k = f32 ? split2_blocks_per_sm<float>(N, threads, sm) : split2_blocks_per_sm<double>(N, threads, sm);
+    int k;
+    if (ks == 1) k = f32 ? split_blocks_per_sm<float>(N, threads, sm) : split_blocks_per_sm<double>(N, threads, sm);
+    else if (ks == 2) k = f32 ? split2_blocks_per_sm<float>(N, threads, sm) : split2_blocks_per_sm<double>(N, threads, sm);
+    else k = f32 ? split3_blocks_per_sm<float>(N, threads, sm) : split3_blocks_per_sm<double>(N, threads, sm);
     if (k < 1) return false;
     const long long Nr = c->d.Nr;
-    long long tiles = (Nr + TR - 1) / TR;
-    long long waves = (tiles + (long long)k * nsm - 1) / ((long long)k * nsm);
-    int rpp = threads / implicit_group(N);
-    auto rpad = [&](int r) { return ((r + rpp - 1) / rpp) * rpp; };
-    double rows = 0.6 * (rpad(TR + 4) + rpad(TR + 2)) + 0.4 * (2.0 * TR + 6.0) + 4.0;
-    out->cost = 0.5 * (double)waves * k * rows * (k == 1 ? 1.2 : 1.0);
+    const long long tiles = (Nr + TR - 1) / TR, per = (tiles + nsm - 1) / nsm, waves = (per + k - 1) / k;
+    const int S = implicit_seg(N), rpw = 32 / implicit_group(N);
+    auto up = [](int a, int b) { return (a + b - 1) / b; };
+    double cost = 0.0;   // us per launch
+    if (f32) {
+        double rows = 0.0;
+        for (int q = 0; q < ks; ++q) {
+            const int ri = TR + 2 * (ks - q);
+            rows += 0.6 * up(ri, rpw) * rpw + 0.4 * (ri - 2);
+        }
+        const long long co = per < k ? per : k;   // CTAs that share an SM
+        cost = 5.0 + waves * co * rows * row_time(N) * (co == 1 ? 1.2 : 1.0);
+    } else {
+        double pipe = 0.0;   // cycles of the busiest scheduler for one tile
+        for (int q = 0; q < ks; ++q) {
+            const int ri = TR + 2 * (ks - q), rl = ri - 2;
+            pipe += 64.0 * up(up(ri, rpw), 4) * (57.0 * S + 48.0);
+            const int nseg = N <= threads ? threads / N : 1, sl = up(rl, nseg);
+            const int warps = N <= threads ? up(N * up(rl, sl), 32) : 8 * up(N, threads);
+            pipe += 64.0 * up(warps, 4) * 26.0 * sl;
+        }
+        cost = per * pipe / 2070.0 + waves * (4.5 + 1.5 * ks);
+    }
+    out->cost = cost / ks;
     out->R = TR + 2;
     out->persist = 0;
     out->nc = 0;
     out->grid = (int)tiles;
-    out->ks = 2;
-    out->pipe = 0;
-    out->smem = sm;
-    return true;
-}
-
-// A three-steps-per-launch candidate of height TR: per step, a third of a
-// tile whose steps cover TR + 6, TR + 4 and TR + 2 rows (implicit) and
-// TR + 4, TR + 2 and TR (LW).  The model leaves it out of the default
-// choice (tile_candidates); the autotuners time it at the heights of the
-// model-best two-step candidates.
-static bool tiled3_cand(const teuk_ctx *c, int TR, int nsm, TileCand *out)
-{
-    const int N = (int)c->d.Ntheta;
-    const bool f32 = c->d.precision == TEUK_FP32;
-    const int threads = 256;
-    if (TR > kMaxTileRows - 6) return false;
-    size_t sm = f32 ? split3_smem_bytes<float>(TR, N) : split3_smem_bytes<double>(TR, N);
-    if (sm > 227 * 1024) return false;
-    int k = f32 ? split3_blocks_per_sm<float>(N, threads, sm) : split3_blocks_per_sm<double>(N, threads, sm);
-    if (k < 1) return false;
-    const long long Nr = c->d.Nr;
-    long long tiles = (Nr + TR - 1) / TR;
-    long long waves = (tiles + (long long)k * nsm - 1) / ((long long)k * nsm);
-    int rpp = threads / implicit_group(N);
-    auto rpad = [&](int r) { return ((r + rpp - 1) / rpp) * rpp; };
-    double rows = 0.6 * (rpad(TR + 6) + rpad(TR + 4) + rpad(TR + 2)) + 0.4 * (3.0 * TR + 9.0) + 4.0;
-    out->cost = (double)waves * k * rows * (k == 1 ? 1.2 : 1.0) / 3.0;
-    out->R = TR + 2;
-    out->persist = 0;
-    out->nc = 0;
-    out->grid = (int)tiles;
-    out->ks = 3;
+    out->ks = ks;
     out->pipe = 0;
     out->smem = sm;
     return true;
@@ -360,7 +345,7 @@ static bool pipe_cand(const teuk_ctx *c, int TR, int threads, int nsm, TileCand 
     auto rpad = [&](int r) { return ((r + rpp - 1) / rpp) * rpp; };
     double rows = (0.6 * (rpad(TR + 4) + rpad(TR + 2)) + 0.4 * (2.0 * TR + 6.0)) * 256.0 / threads + 1.0;
     const int warps = k * threads / 32;
-    out->cost = 0.5 * (double)per * k * rows * (warps < 16 ? 1.2 : 1.0) + 2.0;
+    out->cost = 1.5 * (f32 ? 1.0 : 8.0) * row_time(N) * (0.5 * (double)per * k * rows * (warps < 16 ? 1.2 : 1.0) + 2.0) + 5.0;
     out->R = TR + 2;
     out->persist = 0;
     out->nc = threads;
@@ -391,7 +376,7 @@ static bool persist_cand(const teuk_ctx *c, int TR, int nc, int nsm, TileCand *o
     int rpp = nc / implicit_group(N);
     int rpad = ((R + rpp - 1) / rpp) * rpp;
     double rows = (0.6 * rpad + 0.4 * R) * 256.0 / nc + 2.0;
-    out->cost = 2.0 * (double)per * k * rows + 4.0;
+    out->cost = 1.5 * row_time(N) * (2.0 * (double)per * k * rows + 4.0) + 5.0;
     out->R = R;
     out->persist = 1;
     out->nc = nc;
@@ -410,21 +395,15 @@ int tile_candidates(teuk_ctx *c, TileCand *out, int maxn)
     int n = 0;
     // one-row tiles are the only ones that fit for the widest FP64 rows
     for (int TR = 1; TR <= kMaxTileRows && n < maxn; ++TR) {
-        if (tiled_cand(c, TR, nsm, &out[n])) ++n;
-        if (n < maxn && c->d.scheme == TEUK_SCHEME_SPLIT && tiled2_cand(c, TR, nsm, &out[n])) ++n;
+        for (int ks = 1; ks <= 3; ++ks)
+            if (n < maxn && tiled_cand(c, TR, ks, nsm, &out[n])) ++n;
         for (int th : {256, 512})
             if (n < maxn && c->d.scheme == TEUK_SCHEME_SPLIT && pipe_cand(c, TR, th, nsm, &out[n])) ++n;
         for (int nc : {384, 480})
             if (n < maxn && persist_cand(c, TR, nc, nsm, &out[n])) ++n;
         if (TR >= Nr) break;
     }
-    // insertion sort by cost
-    for (int a = 1; a < n; ++a)
-        for (int b = a; b > 0 && out[b].cost < out[b - 1].cost; --b) {
-            TileCand t = out[b];
-            out[b] = out[b - 1];
-            out[b - 1] = t;
-        }
+    std::stable_sort(out, out + n, [](const TileCand &a, const TileCand &b) { return a.cost < b.cost; });
     return n;
 }
 
@@ -434,7 +413,7 @@ static bool apply_cand(teuk_ctx *c, const TileCand &k)
 {
     const int TR = k.R - 2;
     TileCand t;
-    if (!tiled_cand(c, TR, sm_count(), &t)) return false;
+    if (!tiled_cand(c, TR, 1, sm_count(), &t)) return false;
     c->tile_rows = TR;
     c->threads = 256;
     c->smem = t.smem;
@@ -450,8 +429,14 @@ static bool apply_cand(teuk_ctx *c, const TileCand &k)
 
 int choose_tiles(teuk_ctx *c)
 {
-    std::vector<TileCand> cand(1024);
+    std::vector<TileCand> cand(2048);
     int n = tile_candidates(c, cand.data(), (int)cand.size());
+    for (int k = 0; k < n; ++k)
+        if (cand[k].ks == 1 && !cand[k].persist) {
+            c->one_rows = cand[k].R - 2;
+            c->one_smem = cand[k].smem;
+            break;
+        }
     for (int k = 0; k < n; ++k)
         if (apply_cand(c, cand[k])) return TEUK_OK;
     return set_err(c, TEUK_E_CUDA, "no tile of the split kernel fits on this device");
@@ -506,13 +491,17 @@ StepParams<T> make_params(const teuk_ctx *c, int in_level)
     {
         const size_t pl = (size_t)d.Nr * (size_t)d.Ntheta;   // elements per plane
         const char *m = c->coef + c->L.mat;
+        const size_t t = pl * sizeof(T);
         p.mat.fk = (const c2 *)m;
-        p.mat.dg = (const c2 *)(m + 2 * pl * sizeof(T));
-        p.mat.ct = (const c2 *)(m + 4 * pl * sizeof(T));
-        p.mat.sub = (const T *)(m + 6 * pl * sizeof(T));
-        p.mat.qam = (const T *)(m + 7 * pl * sizeof(T));
-        p.mat.qap = (const T *)(m + 8 * pl * sizeof(T));
-        p.mat.lw = (const T *)(m + ((9 * pl * sizeof(T) + 255) & ~(size_t)255));
+        p.mat.d1 = (const c2 *)(m + 2 * t);
+        p.mat.d2 = (const c2 *)(m + 4 * t);
+        p.mat.pf = (const c2 *)(m + 6 * t);
+        p.mat.sub = (const T *)(m + 8 * t);
+        p.mat.w1l = (const T *)(m + 9 * t);
+        p.mat.w1u = (const T *)(m + 10 * t);
+        p.mat.w2l = (const T *)(m + 11 * t);
+        p.mat.w2u = (const T *)(m + 12 * t);
+        p.mat.lw = (const c2 *)(m + ((kStepPlaneReals * t + 255) & ~(size_t)255));
     }
     p.thtab = (const T *)(c->coef + c->L.thT);
     p.patch = (const c2 *)(c->coef + c->L.patch);
@@ -520,6 +509,7 @@ StepParams<T> make_params(const teuk_ctx *c, int in_level)
     p.h_out = nullptr;
     p.tape = nullptr;
     p.patchu = (const c2 *)(c->coef + c->L.patchu);
+    p.patchd = (const double2 *)(c->coef + c->L.patchd);
     p.unit_p0 = c->unit_p0;
     p.unit_np = c->unit_np;
     p.amp_re = c->amp_re;
@@ -531,6 +521,7 @@ StepParams<T> make_params(const teuk_ctx *c, int in_level)
     p.drs0_dr0 = c->drs0_dr0;
     p.m_dOmega = c->m_dOmega;
     p.w = (const double *)(c->coef + c->L.w);
+    p.seed = (const double2 *)(c->coef + c->L.seed);
     p.uin = (const c2 *)(c->state + (size_t)in_level * c->level_bytes);
     p.uout = (c2 *)(c->state + (size_t)(1 - in_level) * c->level_bytes);
     p.mid = (c2 *)(c->coef + c->L.scratch);
@@ -561,7 +552,14 @@ cudaError_t compute_plans(teuk_ctx *c, cudaStream_t st)
     cudaError_t e = launch_scan_plans<double>(p, pf, ph, (double2 *)sf, (double2 *)sh, st);
     if (e != cudaSuccess) return e;
     // the FP64 path's materialised coefficients come from the same tables
-    return launch_mat_coef<double>(p, st);
+    return launch_step_planes<double>(p, st);
+}
+
+// The sample's adjoint vector for the weights as they are (FP64 split scheme).
+cudaError_t compute_seed(teuk_ctx *c, cudaStream_t st)
+{
+    if (c->d.scheme != TEUK_SCHEME_SPLIT || c->d.precision == TEUK_FP32) return cudaSuccess;
+    return launch_seed(make_params<double>(c, 0), (double2 *)(c->coef + c->L.seed), st);
 }
 
 cudaError_t launch_one(teuk_ctx *c, int in_level, cudaStream_t st)
@@ -767,6 +765,7 @@ int teuk_init_grid(const teuk_grid_desc *desc, void *d_state, void *d_coef, void
         if ((e = cudaMemsetAsync(c->wave, 0, sizeof(double2) * (size_t)(d.Ntheta + 1) * (size_t)wave_capacity, st)) != cudaSuccess) { r2 = cuda_err(c, e, "zero wave"); break; }
         if ((e = launch_coef_tables(d, drs, dt, c->coef, c->L, st)) != cudaSuccess) { r2 = cuda_err(c, e, "coefficient kernels"); break; }
         if ((e = compute_plans(c, st)) != cudaSuccess) { r2 = cuda_err(c, e, "scan plans"); break; }
+        if ((e = compute_seed(c, st)) != cudaSuccess) { r2 = cuda_err(c, e, "sample adjoint"); break; }
         if ((e = launch_set_ctl(c->coef, c->L, 0, 1, st)) != cudaSuccess) { r2 = cuda_err(c, e, "control block"); break; }
         if ((e = extract_current(c, st)) != cudaSuccess) { r2 = cuda_err(c, e, "extract"); break; }
         if ((e = cudaStreamSynchronize(st)) != cudaSuccess) { r2 = cuda_err(c, e, "init sync"); break; }
@@ -841,6 +840,10 @@ int teuk_set_source(teuk_ctx *c, double amp_re, double amp_im, double r0, double
     c->m_dOmega = kepler ? (double)d.m * (-1.5 * sqrt(r0) * Om * Om / sqrt(d.M)) : 0.0;
     // and dOmega/da = -M / (r0^(3/2) + a M^(1/2))^2 = -Omega^2 for the Kepler frequency
     c->m_dOmega_da = kepler ? (double)d.m * (-Om * Om) : 0.0;
+    if (d.precision == TEUK_FP64 && d.scheme == TEUK_SCHEME_SPLIT && c->patch_np > 0) {
+        CK(launch_patch_da(make_params<double>(c, 0), st), "source derivative");
+        CK(cudaStreamSynchronize(st), "source sync");
+    }
     return TEUK_OK;
 }
 
@@ -859,8 +862,10 @@ int teuk_set_weights(teuk_ctx *c, const double *w)
     } else {
         CK(launch_coef_tables(c->d, c->drs, c->dt, c->coef, c->L, 0), "default weights");
         CK(compute_plans(c, 0), "scan plans");
-        CK(cudaDeviceSynchronize(), "weights sync");
     }
+    CK(compute_seed(c, 0), "sample adjoint");
+    c->delta_ok = 0;
+    CK(cudaDeviceSynchronize(), "weights sync");
     return TEUK_OK;
 }
 
@@ -1090,26 +1095,18 @@ static int autotune_impl(teuk_ctx *c, int trial_steps, void *flush, size_t flush
         if (tile_rows_out) *tile_rows_out = c->tile_rows;
         return TEUK_OK;
     }
-    std::vector<TileCand> all(1024);
+    std::vector<TileCand> all(2048);
     int n = tile_candidates(c, all.data(), (int)all.size());
     // the best few of each kernel by the model
     std::vector<TileCand> cand;
-    for (int kind = 0; kind < 4; ++kind) {   // tiled, tiled two steps per launch, persistent, pipelined
+    for (int kind = 0; kind < 5; ++kind) {   // tiled with one, two, three steps per launch, persistent, pipelined
         int taken = 0;
         for (int k = 0; k < n && taken < 4; ++k) {
-            const int kk = all[k].pipe ? 3 : (all[k].persist ? 2 : (all[k].ks == 2 ? 1 : 0));
+            const int kk = all[k].pipe ? 4 : (all[k].persist ? 3 : all[k].ks - 1);
             if (kk == kind) {
                 cand.push_back(all[k]);
                 ++taken;
             }
-        }
-    }
-    // three steps per launch at the heights of the two-step candidates
-    {
-        const size_t n2 = cand.size();
-        for (size_t k = 0; k < n2; ++k) {
-            TileCand t3;
-            if (cand[k].ks == 2 && !cand[k].pipe && tiled3_cand(c, cand[k].R - 2, sm_count(), &t3)) cand.push_back(t3);
         }
     }
     if (cand.empty()) return set_err(c, TEUK_E_CUDA, "no tile of the split kernel fits on this device");
@@ -1193,7 +1190,7 @@ int teuk_set_tiling(teuk_ctx *c, int tile_rows)
     if (c->d.scheme != TEUK_SCHEME_SPLIT) return TEUK_OK;
     if (tile_rows < 1 || tile_rows > 254) return set_err(c, TEUK_E_INVAL, "tile_rows out of range [1, 254]");
     TileCand t;
-    if (!tiled_cand(c, tile_rows, sm_count(), &t)) return set_err(c, TEUK_E_INVAL, "tile does not fit in shared memory");
+    if (!tiled_cand(c, tile_rows, 1, sm_count(), &t)) return set_err(c, TEUK_E_INVAL, "tile does not fit in shared memory");
     drop_graphs(c);
     apply_cand(c, t);
     return TEUK_OK;
@@ -1210,10 +1207,10 @@ int teuk_set_tiling_steps(teuk_ctx *c, int tile_rows, int steps_per_launch)
     const int trmax = kMaxTileRows - 2 * steps_per_launch;
     if (tile_rows < 1 || tile_rows > trmax) return set_err(c, TEUK_E_INVAL, "tile_rows out of range [1, %d]", trmax);
     TileCand t;
-    if (!(steps_per_launch == 3 ? tiled3_cand(c, tile_rows, sm_count(), &t) : tiled2_cand(c, tile_rows, sm_count(), &t)))
+    if (!tiled_cand(c, tile_rows, steps_per_launch, sm_count(), &t))
         return set_err(c, TEUK_E_INVAL, "tile does not fit in shared memory");
     TileCand tt;
-    if (!tiled_cand(c, tile_rows, sm_count(), &tt)) return set_err(c, TEUK_E_INVAL, "tile does not fit in shared memory");
+    if (!tiled_cand(c, tile_rows, 1, sm_count(), &tt)) return set_err(c, TEUK_E_INVAL, "tile does not fit in shared memory");
     drop_graphs(c);
     apply_cand(c, t);
     return TEUK_OK;
@@ -1230,7 +1227,7 @@ int teuk_set_pipelined(teuk_ctx *c, int tile_rows, int threads)
         return set_err(c, TEUK_E_INVAL, "pipelined kernel unavailable: rows must be 16-byte multiples and two tile "
                                         "buffers must fit in shared memory");
     TileCand tt;
-    if (!tiled_cand(c, tile_rows, sm_count(), &tt)) return set_err(c, TEUK_E_INVAL, "tile does not fit in shared memory");
+    if (!tiled_cand(c, tile_rows, 1, sm_count(), &tt)) return set_err(c, TEUK_E_INVAL, "tile does not fit in shared memory");
     drop_graphs(c);
     apply_cand(c, t);
     return TEUK_OK;
@@ -1252,7 +1249,7 @@ int teuk_set_persistent(teuk_ctx *c, int tile_rows, int consumer_threads)
         return set_err(c, TEUK_E_INVAL, "persistent kernel unavailable for this grid: %s", why);
     }
     TileCand tt;
-    if (!tiled_cand(c, tile_rows, sm_count(), &tt)) return set_err(c, TEUK_E_INVAL, "tile does not fit in shared memory");
+    if (!tiled_cand(c, tile_rows, 1, sm_count(), &tt)) return set_err(c, TEUK_E_INVAL, "tile does not fit in shared memory");
     drop_graphs(c);
     apply_cand(c, t);
     return TEUK_OK;
@@ -1327,8 +1324,8 @@ int adjoint_tile_rows(const teuk_ctx *c)
     return best;
 }
 
-// Tile height of the adjoint step with the spin derivative: twice the
-// shared memory per row (eight state planes), at most about 200 KB per tile.
+// Tile height of k_adjoint_spin (one CTA per SM): ten state planes, at most
+// about 200 KB per tile.
 int adjoint_spin_tile_rows(const teuk_ctx *c)
 {
     const int N = (int)c->d.Ntheta;
@@ -1343,65 +1340,68 @@ int adjoint_spin_tile_rows(const teuk_ctx *c)
     return best;
 }
 
+// Tile height of k_adjoint_f64 (one CTA per SM): the fewest FP64 instructions
+// of the busiest scheduler, counted as for tiled_cand (an element takes about
+// 93 in the transposed row solve with its spin term, 57 without, 56 or 26 in
+// the stencil, 57 more where the stage values are recomputed), and 5 us of
+// latency a tile.
+int adjoint_f64_tile_rows(const teuk_ctx *c, bool spin)
+{
+    const int N = (int)c->d.Ntheta, S = implicit_seg(N), rpw = 32 / implicit_group(N), nsm = sm_count();
+    auto up = [](long long a, long long b) { return (a + b - 1) / b; };
+    int best = 1;
+    double bc = 1e300;
+    for (int tr = 1; tr <= kMaxTileRows && adjoint_f64_smem_bytes(tr, N, spin) <= 226 * 1024; ++tr) {
+        double pipe = 64.0 * up(up(tr, rpw), 4) * ((spin ? 93.0 : 57.0) * S + 48.0);
+        if (spin) pipe += 64.0 * up(up(tr + 2, rpw), 4) * (57.0 * S + 48.0);
+        const long long nseg = N <= 256 ? 256 / N : 1, sl = up(tr, nseg);
+        const long long warps = N <= 256 ? up(N * up(tr, sl), 32) : 8 * up(N, 256);
+        pipe += 64.0 * up(warps, 4) * (spin ? 56.0 : 26.0) * sl;
+        const double cost = up(up(c->d.Nr, tr), nsm) * (pipe / 2070.0 + 5.0);
+        if (cost < bc) {
+            bc = cost;
+            best = tr;
+        }
+        if (tr >= c->d.Nr) break;
+    }
+    return best;
+}
+
 // The adjoint workspace: accumulators (8 doubles), per-CTA parts, the
-// dot product's parts (512 doubles), then the coefficient planes of the
-// spin adjoint from a 256-byte boundary.
+// dot product's parts (512 doubles), then the planes of the FP64 step from a
+// 256-byte boundary.
 size_t adjoint_small_doubles(const teuk_ctx *c)
 {
-    const int tr = adjoint_tile_rows(c), trs = adjoint_spin_tile_rows(c);
-    const int grid = (int)((c->d.Nr + tr - 1) / tr), grids = (int)((c->d.Nr + trs - 1) / trs);
-    const int gmax = grid > grids ? grid : grids;
+    auto grid = [&](int tr) { return (c->d.Nr + tr - 1) / tr; };
+    int64_t gmax = std::max(grid(adjoint_tile_rows(c)), grid(adjoint_spin_tile_rows(c)));
+    if (c->d.precision == TEUK_FP64)
+        gmax = std::max(gmax, std::max(grid(adjoint_f64_tile_rows(c, true)), grid(adjoint_f64_tile_rows(c, false))));
     return 8 + 6 * (size_t)gmax + 2 * 256;
 }
 size_t adjoint_planes_offset(const teuk_ctx *c) { return (sizeof(double) * adjoint_small_doubles(c) + 255) & ~(size_t)255; }
 // FP64 only: the FP32 adjoint forms its coefficients in place, which costs
 // it less than reading them (the FP64 step is bound by the FP64 pipe, the
 // FP32 step is not)
-AdjPlaneLayout adjoint_planes_layout(const teuk_ctx *c)
+size_t adjoint_ws_bytes(const teuk_ctx *c)
 {
-    if (c->d.precision == TEUK_FP32) {
-        AdjPlaneLayout L = {};
-        return L;
-    }
-    return adj_plane_layout(c->d.Nr, c->d.Ntheta, sizeof(double));
+    const size_t planes = c->d.precision == TEUK_FP32
+                              ? 0
+                              : adj_plane_layout(c->d.Nr, c->d.Ntheta, implicit_group((int)c->d.Ntheta)).total;
+    return adjoint_planes_offset(c) + planes;
 }
-size_t adjoint_ws_bytes(const teuk_ctx *c) { return adjoint_planes_offset(c) + adjoint_planes_layout(c).total; }
 
-template <typename T>
-AdjPlanes<T> adjoint_planes(const teuk_ctx *c, const void *ws)
+AdjPlanes adjoint_planes(const teuk_ctx *c, const void *ws)
 {
-    typedef typename V2<T>::t c2;
     const char *b = (const char *)ws + adjoint_planes_offset(c);
-    const AdjPlaneLayout L = adjoint_planes_layout(c);
-    AdjPlanes<T> A;
-    A.m.fk = (const c2 *)(b + L.off[0]);
-    A.m.dg = (const c2 *)(b + L.off[1]);
-    A.m.ct = (const c2 *)(b + L.off[2]);
-    A.m.sub = (const T *)(b + L.off[3]);
-    A.m.qam = (const T *)(b + L.off[4]);
-    A.m.qap = (const T *)(b + L.off[5]);
-    A.m.lw = (const T *)(b + L.off[6]);
-    A.dlw = (const T *)(b + L.off[7]);
-    A.dimp = (const T *)(b + L.off[8]);
+    const AdjPlaneLayout L = adj_plane_layout(c->d.Nr, c->d.Ntheta, implicit_group((int)c->d.Ntheta));
+    AdjPlanes A;
+    A.pb = (const double2 *)(b + L.off[0]);
+    A.af = (const double2 *)(b + L.off[1]);
+    A.dlw = (const double2 *)(b + L.off[2]);
+    A.dimp = (const double2 *)(b + L.off[3]);
+    A.delta = (const double2 *)(b + L.off[4]);
+    A.plan = (const int *)(b + L.off[5]);
     return A;
-}
-
-template <typename T>
-cudaError_t fill_adjoint_planes(const teuk_ctx *c, void *ws, cudaStream_t st)
-{
-    typedef typename V2<T>::t c2;
-    const AdjPlanes<T> A = adjoint_planes<T>(c, ws);
-    MatOut<T> o;
-    o.fk = (c2 *)A.m.fk;
-    o.dg = (c2 *)A.m.dg;
-    o.ct = (c2 *)A.m.ct;
-    o.sub = (T *)A.m.sub;
-    o.qam = (T *)A.m.qam;
-    o.qap = (T *)A.m.qap;
-    o.lw = (T *)A.m.lw;
-    o.dlw = (T *)A.dlw;
-    o.dimp = (T *)A.dimp;
-    return launch_mat_coef_to<T>(make_params<T>(c, 0), o, st);
 }
 
 }  // namespace
@@ -1423,7 +1423,8 @@ static int apply_step(teuk_ctx *c, const void *d_in, void *d_out, int64_t n, int
         p.first = first ? 1 : 0;
         p.nfix = n;
         p.h_out = (double2 *)d_h;
-        e = launch_apply_step<float>(p, c->threads, c->smem, st);
+        p.tile_rows = c->one_rows;
+        e = launch_apply_step<float>(p, c->threads, c->one_smem, st);
     } else {
         StepParams<double> p = make_params<double>(c, 0);
         p.uin = (const double2 *)d_in;
@@ -1431,7 +1432,8 @@ static int apply_step(teuk_ctx *c, const void *d_in, void *d_out, int64_t n, int
         p.first = first ? 1 : 0;
         p.nfix = n;
         p.h_out = (double2 *)d_h;
-        e = launch_apply_step<double>(p, c->threads, c->smem, st);
+        p.tile_rows = c->one_rows;
+        e = launch_apply_step<double>(p, c->threads, c->one_smem, st);
     }
     if (e != cudaSuccess) return cuda_err(c, e, "apply step");
     return TEUK_OK;
@@ -1478,8 +1480,14 @@ int teuk_adjoint_prepare(teuk_ctx *c, void *d_ws, void *stream)
     if (c->d.scheme != TEUK_SCHEME_SPLIT) return set_err(c, TEUK_E_INVAL, "the adjoint needs the split scheme");
     if (!d_ws || ((uintptr_t)d_ws & 255)) return set_err(c, TEUK_E_INVAL, "need a 256-byte aligned workspace");
     cudaStream_t st = (cudaStream_t)stream;
-    cudaError_t e = c->d.precision == TEUK_FP32 ? cudaSuccess : fill_adjoint_planes<double>(c, d_ws, st);
-    if (e != cudaSuccess) return cuda_err(c, e, "adjoint planes");
+    if (c->d.precision == TEUK_FP64) {
+        const StepParams<double> p = make_params<double>(c, 0);
+        const AdjPlanes A = adjoint_planes(c, d_ws);
+        cudaError_t e = launch_adjoint_f64_planes(p, A, st);
+        if (e == cudaSuccess) e = launch_delta(p, (double2 *)A.delta, st);
+        if (e != cudaSuccess) return cuda_err(c, e, "adjoint planes");
+        c->delta_ok = 1;
+    }
     c->adj_ws = d_ws;
     return TEUK_OK;
 }
@@ -1511,8 +1519,8 @@ int teuk_adjoint_step(teuk_ctx *c, const void *d_lam_in, void *d_lam_out, int64_
         // full steps with a prepared workspace read the coefficient planes
         // (the FP64 pipe bounds this step)
         if (!first && d_ws == c->adj_ws)
-            e = launch_adjoint_planes<double>(p, adjoint_spin_tile_rows(c), (const double2 *)d_gseed,
-                                              adjoint_planes<double>(c, d_ws), part, acc, st);
+            e = launch_adjoint_f64(p, adjoint_f64_tile_rows(c, false), false, nullptr, nullptr, (const double2 *)d_gseed,
+                                   adjoint_planes(c, d_ws), part, acc, st);
         else
             e = launch_adjoint_step<double>(p, tr, (const double2 *)d_gseed, part, acc, st);
     }
@@ -1535,16 +1543,28 @@ static int adjoint_spin(teuk_ctx *c, const void *d_lam_in, void *d_lam_out, cons
         p.uout = (float2 *)d_lam_out;
         p.first = first ? 1 : 0;
         p.nfix = n;
-        e = launch_adjoint_spin<float>(p, tr, (const float2 *)d_s, (const float2 *)d_tape, (const double2 *)d_gseed,
-                                       adjoint_planes<float>(c, d_ws), part, acc, st);
+        e = launch_adjoint_spin<float>(p, tr, (const float2 *)d_s, (const float2 *)d_tape, (const double2 *)d_gseed, part,
+                                       acc, st);
     } else {
         StepParams<double> p = make_params<double>(c, 0);
         p.uin = (const double2 *)d_lam_in;
         p.uout = (double2 *)d_lam_out;
         p.first = first ? 1 : 0;
         p.nfix = n;
-        e = launch_adjoint_spin<double>(p, tr, (const double2 *)d_s, (const double2 *)d_tape,
-                                        (const double2 *)d_gseed, adjoint_planes<double>(c, d_ws), part, acc, st);
+        if (first) {
+            e = launch_adjoint_spin<double>(p, tr, (const double2 *)d_s, (const double2 *)d_tape, (const double2 *)d_gseed,
+                                            part, acc, st);
+        } else {
+            const AdjPlanes A = adjoint_planes(c, d_ws);
+            e = cudaSuccess;
+            if (!c->delta_ok) {   // the weights have changed since teuk_adjoint_prepare
+                e = launch_delta(p, (double2 *)A.delta, st);
+                if (e == cudaSuccess) c->delta_ok = 1;
+            }
+            if (e == cudaSuccess)
+                e = launch_adjoint_f64(p, adjoint_f64_tile_rows(c, true), true, (const double2 *)d_s, (const double2 *)d_tape,
+                                       (const double2 *)d_gseed, A, part, acc, st);
+        }
     }
     if (e != cudaSuccess) return cuda_err(c, e, "adjoint step (spin)");
     return TEUK_OK;
@@ -1585,7 +1605,8 @@ int teuk_apply_step_tape(teuk_ctx *c, const void *d_in, void *d_out, int64_t n, 
         p.nfix = n;
         p.h_out = (double2 *)d_h;
         p.tape = (float2 *)d_tape;
-        e = launch_apply_step<float>(p, c->threads, c->smem, st);
+        p.tile_rows = c->one_rows;
+        e = launch_apply_step<float>(p, c->threads, c->one_smem, st);
     } else {
         StepParams<double> p = make_params<double>(c, 0);
         p.uin = (const double2 *)d_in;
@@ -1594,7 +1615,8 @@ int teuk_apply_step_tape(teuk_ctx *c, const void *d_in, void *d_out, int64_t n, 
         p.nfix = n;
         p.h_out = (double2 *)d_h;
         p.tape = (double2 *)d_tape;
-        e = launch_apply_step<double>(p, c->threads, c->smem, st);
+        p.tile_rows = c->one_rows;
+        e = launch_apply_step<double>(p, c->threads, c->one_smem, st);
     }
     if (e != cudaSuccess) return cuda_err(c, e, "apply step (tape)");
     return TEUK_OK;

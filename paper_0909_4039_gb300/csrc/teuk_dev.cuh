@@ -676,47 +676,6 @@ __device__ __forceinline__ void imp_load(const ImpConst<T> &K, const typename V2
                  C.fk[k]);
 }
 
-// The same segment with the coefficients read from the materialised planes
-// (row gi of the full step's tables; FP64 state), bit for bit what imp_load
-// forms.
-template <typename T, int S>
-__device__ __forceinline__ void imp_load_mat(const MatPlanes<T> &M, const typename V2<T>::t *phi,
-                                             const typename V2<T>::t *pi, const typename V2<T>::t *prow, int gi,
-                                             int N, int len, int j0, bool vec, ImpCoef<T, S> &C,
-                                             typename V2<T>::t (&w)[S], typename V2<T>::t (&y)[S])
-{
-    typedef typename V2<T>::t c2;
-    const c2 zero = cmk<c2>(T(0), T(0));
-    const c2 one = cmk<c2>(T(1), T(0));
-    const size_t o = (size_t)gi * N + j0;
-    if (vec && len == S) {
-        vload<S>(C.e, prow + j0);
-        vload<S>(w, phi + j0);
-        vload<S>(y, pi + j0);
-        vload<S>(C.fk, M.fk + o);
-        vload<S>(C.dg, M.dg + o);
-        vload<S>(C.ct, M.ct + o);
-        vload<S>(C.sub, M.sub + o);
-        vload<S>(C.qam, M.qam + o);
-        vload<S>(C.qap, M.qap + o);
-    } else {
-#pragma unroll
-        for (int k = 0; k < S; ++k) {
-            const bool real = k < len;
-            const size_t q = real ? o + k : 0;
-            C.e[k] = real ? prow[j0 + k] : one;
-            w[k] = real ? phi[j0 + k] : zero;
-            y[k] = real ? pi[j0 + k] : zero;
-            C.fk[k] = real ? M.fk[q] : zero;
-            C.dg[k] = real ? M.dg[q] : zero;
-            C.ct[k] = real ? M.ct[q] : zero;
-            C.sub[k] = real ? M.sub[q] : T(0);
-            C.qam[k] = real ? M.qam[q] : T(0);
-            C.qap[k] = real ? M.qap[q] : T(0);
-        }
-    }
-}
-
 // Scan plan of the LU solve from the row's stored levels: the segment maps'
 // multiplicative parts are prod(-e_j sub_j) forward and prod(-fk_j)
 // backward (formed only when a level uses them).
@@ -859,9 +818,8 @@ __device__ __forceinline__ void apply_W(const ImpCoef<T, S> &C, const typename V
 template <typename T, int S, bool MAT = false>
 __device__ void implicit_row_fwd(const ImpConst<T> &K0, typename V2<T>::t *phi, typename V2<T>::t *pi,
                                  const typename V2<T>::t *prow, const T *f, const T *th, int N, bool active,
-                                 bool in_tile, int g, int G, bool vec, int plan, const MatPlanes<T> *mat = nullptr,
-                                 int gi = 0, typename V2<T>::t *u1phi = nullptr, typename V2<T>::t *u1pi = nullptr,
-                                 const typename V2<T>::t *seg = nullptr)
+                                 bool in_tile, int g, int G, bool vec, int plan, typename V2<T>::t *u1phi = nullptr,
+                                 typename V2<T>::t *u1pi = nullptr, const typename V2<T>::t *seg = nullptr)
 {
     typedef typename V2<T>::t c2;
     const ImpConst<T> K = K0;   // the step's constants, read once from the parameters
@@ -872,10 +830,7 @@ __device__ void implicit_row_fwd(const ImpConst<T> &K0, typename V2<T>::t *phi, 
     if (!active) len = 0;
     ImpCoef<T, S> C;
     c2 w[S], y[S], v[S];
-    if constexpr (MAT)
-        imp_load_mat<T, S>(*mat, phi, pi, prow, gi, N, len, j0, vec, C, w, y);
-    else
-        imp_load<T, S>(K, phi, pi, prow, f, th, N, len, j0, vec, C, w, y);
+    imp_load<T, S>(K, phi, pi, prow, f, th, N, len, j0, vec, C, w, y);
     const ScanPlan<T> P = scan_plan_lu<T, S>(C, active ? plan : 0, seg);
     {
         c2 Wu[S];
@@ -906,6 +861,157 @@ __device__ void implicit_row_fwd(const ImpConst<T> &K0, typename V2<T>::t *phi, 
     seg_solve_lu<T, S>(v, C, P, g, G);             // U2_Pi
 #pragma unroll
     for (int k = 0; k < S; ++k) w[k] = caxpy(K.gh, v[k], w[k]);
+    if (in_tile) row_store<T, S>(phi, pi, w, v, j0, lenw, vec);
+}
+
+// The full implicit step of an FP64 row on the materialised planes (row gi):
+// the map of implicit_row_fwd with fewer FP64 instructions, which is what it
+// costs (see StepPlanes).  Against it: W and c_t arrive multiplied by the
+// constants they meet, the second stage's W and c_t as one operator (8
+// instructions an element for 14), and a lane adds the incoming value times
+// the stored products pf to its own solution (4 an element) where
+// seg_solve_lu runs the recurrence a second time (6).
+template <typename T, int S>
+__device__ __forceinline__ void implicit_row_mat(const ImpConst<T> &K0, const StepPlanes<T> &M, typename V2<T>::t *phi,
+                                                 typename V2<T>::t *pi, int gi, int N, bool active, bool in_tile, int g,
+                                                 int G, bool vec, int plan, typename V2<T>::t *u1phi = nullptr,
+                                                 typename V2<T>::t *u1pi = nullptr)
+{
+    typedef typename V2<T>::t c2;
+    const c2 zero = cmk<c2>(T(0), T(0)), one = cmk<c2>(T(1), T(0));
+    const int j0 = g * S;
+    int len = N - j0;
+    len = len < 0 ? 0 : (len > S ? S : len);
+    const int lenw = len;
+    if (!active) {
+        len = 0;
+        gi = 1;
+    }
+    const size_t o = (size_t)gi * N + j0;
+    const bool whole = vec && len == S;
+    // a plane's segment (pad past the row's end and for rows that are not active)
+    auto cseg = [&](const c2 *src, c2 pad, c2(&r)[S]) {
+        if (whole) {
+            vload<S>(r, src);
+        } else {
+#pragma unroll
+            for (int k = 0; k < S; ++k) r[k] = k < len ? src[k] : pad;
+        }
+    };
+    auto rseg = [&](const T *src, T(&r)[S]) {
+        if (whole) {
+            vload<S>(r, src);
+        } else {
+#pragma unroll
+            for (int k = 0; k < S; ++k) r[k] = k < len ? src[k] : T(0);
+        }
+    };
+    c2 e[S], fk[S], pf[S];
+    T sub[S];
+    cseg(K0.piv + o, one, e);
+    cseg(M.fk + o, zero, fk);
+    cseg(M.pf + o, zero, pf);
+    rseg(M.sub + o, sub);
+    const int nf = plan & 0xff, nb = (plan >> 8) & 0xff;
+    const int nfw = (int)__reduce_max_sync(0xffffffffu, (unsigned)nf), nbw = (int)__reduce_max_sync(0xffffffffu, (unsigned)nb);
+    c2 Ab = zero;
+    if (nbw > 0) Ab = (K0.seg + ((size_t)gi * G + g) * 2)[1];
+    // acc - (wl x_{j-1} + d x_j + wu x_{j+1}) for the lane's segment
+    auto minus_tri = [&](const T(&wl)[S], const c2(&d)[S], const T(&wu)[S], const c2(&x)[S], c2(&acc)[S]) {
+        const c2 xl = shfl_up_c(x[S - 1], 1, G), xr = shfl_down_c(x[0], 1, G);
+#pragma unroll
+        for (int k = 0; k < S; ++k) {
+            const c2 xm = k ? x[k ? k - 1 : 0] : xl, xp = (k + 1 < S) ? x[(k + 1) < S ? k + 1 : S - 1] : xr;
+            acc[k] = cfnma(d[k], x[k], caxpy(-wu[k], xp, caxpy(-wl[k], xm, acc[k])));
+        }
+    };
+    // r <- M^{-1} r
+    auto solve = [&](c2(&r)[S]) {
+        r[0] = cmul(e[0], r[0]);
+#pragma unroll
+        for (int k = 1; k < S; ++k) r[k] = cmul(e[k], caxpy(-sub[k], r[k - 1], r[k]));
+        c2 B = r[S - 1], A = pf[S - 1];
+#pragma unroll 1
+        for (int l = 0; l < nfw; ++l) {
+            const int d = 1 << l;
+            const c2 Bo = shfl_up_c(B, d, G);
+            c2 Ao = one;
+            if (l + 1 < nfw) Ao = shfl_up_c(A, d, G);
+            if (l < nf && g >= d) {
+                B = cfma(A, Bo, B);
+                if (l + 1 < nf) A = cmul(A, Ao);
+            }
+        }
+        // lane 0's incoming value meets pf = 0 (first row of the operator)
+        const c2 z = shfl_up_c(B, 1, G);
+#pragma unroll
+        for (int k = 0; k < S; ++k) r[k] = cfma(pf[k], z, r[k]);
+        B = r[S - 1];
+#pragma unroll
+        for (int k = S - 2; k >= 0; --k) B = cfnma(fk[k], B, r[k]);
+        A = Ab;
+#pragma unroll 1
+        for (int l = 0; l < nbw; ++l) {
+            const int d = 1 << l;
+            const c2 Bo = shfl_down_c(B, d, G);
+            c2 Ao = one;
+            if (l + 1 < nbw) Ao = shfl_down_c(A, d, G);
+            if (l < nb && g + d < G) {
+                B = cfma(A, Bo, B);
+                if (l + 1 < nb) A = cmul(A, Ao);
+            }
+        }
+        // the last lane's incoming value meets fk = 0 (last row, or padding)
+        c2 x = shfl_down_c(B, 1, G);
+#pragma unroll
+        for (int k = S - 1; k >= 0; --k) {
+            x = cfnma(fk[k], x, r[k]);
+            r[k] = x;
+        }
+    };
+    c2 w[S], y[S], v[S];
+    cseg(phi + j0, zero, w);
+    cseg(pi + j0, zero, y);
+    const T gh = K0.gh, h1g = K0.h1g;
+    {
+        // t = -gh W u_Phi; stage 1's right side u_Pi + t, the second's first part u_Pi + t / gamma
+        c2 d[S];
+        T wl[S], wu[S];
+        cseg(M.d1 + o, zero, d);
+        rseg(M.w1l + o, wl);
+        rseg(M.w1u + o, wu);
+#pragma unroll
+        for (int k = 0; k < S; ++k) v[k] = zero;
+        minus_tri(wl, d, wu, w, v);
+        const T ig = T(1.0 / kGamma);
+#pragma unroll
+        for (int k = 0; k < S; ++k) {
+            const c2 t = v[k];
+            v[k] = caxpy(ig, t, y[k]);
+            y[k] = cadd(y[k], t);
+        }
+    }
+    solve(y);                                      // U1_Pi
+    if (u1phi && in_tile) {
+        // the first stage value U1 (U1_Phi = u_Phi + gh U1_Pi), for the adjoint's spin term
+        c2 t[S];
+#pragma unroll
+        for (int k = 0; k < S; ++k) t[k] = caxpy(gh, y[k], w[k]);
+        row_store<T, S>(u1phi, u1pi, t, y, j0, lenw, vec);
+    }
+    {
+        c2 d[S];
+        T wl[S], wu[S];
+        cseg(M.d2 + o, zero, d);
+        rseg(M.w2l + o, wl);
+        rseg(M.w2u + o, wu);
+        minus_tri(wl, d, wu, y, v);                // stage 2 right side
+#pragma unroll
+        for (int k = 0; k < S; ++k) w[k] = caxpy(h1g, y[k], w[k]);   // u_Phi + (1 - gamma) h U1_Pi
+    }
+    solve(v);                                      // U2_Pi
+#pragma unroll
+    for (int k = 0; k < S; ++k) w[k] = caxpy(gh, v[k], w[k]);
     if (in_tile) row_store<T, S>(phi, pi, w, v, j0, lenw, vec);
 }
 
@@ -963,7 +1069,7 @@ __device__ __forceinline__ void implicit_row_one(const ImpConst<T> &K, typename 
         implicit_pair(K, A, B, th2, g, vec);
     } else {
         implicit_row_fwd<T, S>(K, phi, pi, K.piv + (size_t)gi * N, f, th, N, active, in_tile, g, G, vec,
-                               plan, nullptr, 0, u1f, u1g);
+                               plan, u1f, u1g);
     }
 }
 
@@ -1192,7 +1298,7 @@ __device__ __forceinline__ void imp_da(const ImpRow<T> &r, const T (&fr)[8], con
     dct = cmk<c2>(fma(dsg, fr[SF_CTR], sg * ctr), fma(dsg, fma(fr[SF_CTC], cc, fr[SF_CTI]), sg * cti));
 }
 
-template <typename T, bool INTERIOR, bool MAT = false, bool SRC = true>
+template <typename T, bool INTERIOR, bool SRC = true>
 __device__ void lw_segment(const StepParams<T> &p, typename V2<T>::t *sPhi, typename V2<T>::t *sPi,
                            const T *sSt, const T *sTh, int j, int ra, int rb,
                            typename V2<T>::t pf, typename V2<T>::t pg, typename V2<T>::t nf,
@@ -1213,19 +1319,8 @@ __device__ void lw_segment(const StepParams<T> &p, typename V2<T>::t *sPhi, type
     // beta and kap at tile position e (2 lr: node, 2 k + 1: half node), and
     // 1/Sigma^2 there when the source needs it
     auto coef = [&](int e, T &beta, c2 &kap, T &sg, bool need_sg) {
-        if constexpr (MAT) {
-            T v[4];
-            vload<4>(v, p.mat.lw + ((size_t)(2 * g0 + e) * N + j) * 4);
-            beta = v[0];
-            kap = cmk<c2>(v[1], v[2]);
-            if (need_sg) {
-                const T *f = sSt + e * NSF;
-                const T rs = rsq_(fma(-f[SF_AD], S2, f[SF_R2]));
-                sg = rs * rs;
-            }
-        } else {
-            lw_coef<T>(sSt + e * NSF, S2, C, beta, kap, &sg);
-        }
+        (void)need_sg;
+        lw_coef<T>(sSt + e * NSF, S2, C, beta, kap, &sg);
     };
     // source at tile position e times the scaled phase ph (zero outside the
     // patch rows): F = SRC sg (SR2 GTH + GA2)
@@ -1297,6 +1392,68 @@ __device__ void lw_segment(const StepParams<T> &p, typename V2<T>::t *sPhi, type
     }
 }
 
+// Both Lax-Wendroff stages of FP64 tile rows [ra, rb) in theta column j from
+// the stencil planes, in place (pf, pg, nf, ng as in lw_segment).  Eq. 13 put
+// into Eq. 14 is, with beta, kap at the node and beta_-+, kap_-+ at the half
+// nodes below and above it and d_-+ the differences to the neighbouring rows,
+//   Phi' = Phi + Am d_- Phi - Ap d_+ Phi
+//   Pi'  = Pi - Bm d_- Pi + Bp d_+ Pi + Cm d_- Phi + Cp d_+ Phi
+//          + beta (S_+ - S_-) + S,
+//   Am = beta (1/2 + beta_-), Ap = beta (1/2 - beta_+),
+//   Bm = beta (1/2 - beta_-), Bp = beta (1/2 + beta_+),
+//   Cm = beta kap_- - kap (1/2 + beta_-), Cp = beta kap_+ + kap (1/2 - beta_+)
+// (S: the source at the node and the half nodes, from the source patch): 16
+// FP64 multiply-adds and 8 additions an element for the two stages' 32
+// instructions, and no half row to repeat at a segment's start.  In
+// differences, the rounding of the coefficients meets the differences only
+// (with the stencil's weights summed into a middle one, 24 multiply-adds,
+// 1024 x 32 was 1.7 times as far from 64 bits after 200 steps).  Pairs of a
+// plane: (Am, Ap), (Bm, Bp), Cm, Cp; beta = Am + Bm.
+template <typename T, bool INTERIOR>
+__device__ __forceinline__ void lw_segment_mat(const StepParams<T> &p, typename V2<T>::t *sPhi, typename V2<T>::t *sPi, int j,
+                                               int ra, int rb, typename V2<T>::t pf, typename V2<T>::t pg,
+                                               typename V2<T>::t nf, typename V2<T>::t ng, int g0, typename V2<T>::t ph1,
+                                               typename V2<T>::t ph2, bool src)
+{
+    typedef typename V2<T>::t c2;
+    const int N = p.Nth, P = p.pitch, Nr = p.Nr;
+    const c2 zero = cmk<c2>(T(0), T(0));
+    c2 fa = pf, ga = pg, fb = sPhi[ra * P + j], gb = sPi[ra * P + j];
+#pragma unroll 2
+    for (int lr = ra; lr < rb; ++lr) {
+        const int gi = g0 + lr;
+        if (!INTERIOR && gi >= Nr) break;
+        c2 fc = nf, gc = ng;
+        if (lr + 1 < rb) {
+            fc = sPhi[(lr + 1) * P + j];
+            gc = sPi[(lr + 1) * P + j];
+        }
+        c2 f = zero, g = zero;
+        if (INTERIOR || (gi >= 1 && gi <= Nr - 2)) {
+            const c2 *q = p.mat.lw + (size_t)gi * kLwStencil * N + j;
+            const c2 a = q[0], b = q[N], cm = q[2 * N], cp = q[3 * N];
+            const c2 dm = csub(fa, fb), dp = csub(fc, fb);
+            f = caxpy(-a.y, dp, caxpy(a.x, dm, fb));
+            g = caxpy(b.y, csub(gc, gb), caxpy(-b.x, csub(ga, gb), gb));
+            g = cfma(cp, dp, cfma(cm, dm, g));
+            if (src) {
+                const int pr = gi - p.patch_p0;
+                auto F = [&](int r, int pos) {
+                    return r >= 0 && r < p.patch_np ? p.patch[((size_t)r * 2 + pos) * N + j] : zero;
+                };
+                if (pr >= 0 && pr <= p.patch_np)
+                    g = cfma(F(pr, 0), ph2, cfma(cscale<c2>(a.x + b.x, csub(F(pr, 1), F(pr - 1, 1))), ph1, g));
+            }
+        }
+        sPhi[lr * P + j] = f;
+        sPi[lr * P + j] = g;
+        fa = fb;
+        ga = gb;
+        fb = fc;
+        gb = gc;
+    }
+}
+
 __device__ __forceinline__ double2 phase_at(double mOmega, double t)
 {
     double ph = mOmega * t;
@@ -1342,13 +1499,20 @@ __device__ __forceinline__ void lw_phase(const StepParams<T> &p, typename V2<T>:
             ng = sPi[rb * P + j];
         }
         bar();
-        if (work) lw_segment<T, INTERIOR, MAT, SRC>(p, sPhi, sPi, sSt, sTh, j, ra, rb, pf, pg, nf, ng, g0, ph1, ph2, src);
+        if constexpr (MAT) {
+            if (work) lw_segment_mat<T, INTERIOR>(p, sPhi, sPi, j, ra, rb, pf, pg, nf, ng, g0, ph1, ph2, src);
+        } else {
+            if (work) lw_segment<T, INTERIOR, SRC>(p, sPhi, sPi, sSt, sTh, j, ra, rb, pf, pg, nf, ng, g0, ph1, ph2, src);
+        }
     } else {
         // each thread owns whole columns: rows r0-1 and r0+nr are read before any write
         for (int j = ctid; j < N; j += NC) {
             c2 pf = sPhi[(r0 - 1) * P + j], pg = sPi[(r0 - 1) * P + j];
             c2 nf = sPhi[(r0 + nr) * P + j], ng = sPi[(r0 + nr) * P + j];
-            lw_segment<T, INTERIOR, MAT, SRC>(p, sPhi, sPi, sSt, sTh, j, r0, r0 + nr, pf, pg, nf, ng, g0, ph1, ph2, src);
+            if constexpr (MAT)
+                lw_segment_mat<T, INTERIOR>(p, sPhi, sPi, j, r0, r0 + nr, pf, pg, nf, ng, g0, ph1, ph2, src);
+            else
+                lw_segment<T, INTERIOR, SRC>(p, sPhi, sPi, sSt, sTh, j, r0, r0 + nr, pf, pg, nf, ng, g0, ph1, ph2, src);
         }
     }
 }
@@ -1422,6 +1586,27 @@ __device__ double2 sample_warp(const StepParams<T> &p, const typename V2<T>::t *
         sim += __shfl_xor_sync(0xffffffffu, sim, o);
     }
     return make_double2(sre, sim);
+}
+
+// h = E C_{dt/2} s = sum conj(seed) s over the extraction row (planes f, g) of
+// an internal FP64 state, one warp: the sample is linear in s, and against the
+// row solve (15 us by one warp) this costs two products an element.  (FP32
+// solves the row: a seed rounded to FP32 put the amplitude's derivative
+// further from 64 bits.)
+template <typename T>
+__device__ __forceinline__ double2 seed_dot(const StepParams<T> &p, const typename V2<T>::t *f, const typename V2<T>::t *g)
+{
+    double2 h = make_double2(0.0, 0.0);
+    for (int j = threadIdx.x & 31; j < p.Nth; j += 32) {
+        const double2 a = p.seed[j], b = p.seed[p.Nth + j];
+        h = cfma(make_double2(a.x, -a.y), make_double2((double)f[j].x, (double)f[j].y), h);
+        h = cfma(make_double2(b.x, -b.y), make_double2((double)g[j].x, (double)g[j].y), h);
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+        h.x += __shfl_xor_sync(0xffffffffu, h.x, o);
+        h.y += __shfl_xor_sync(0xffffffffu, h.y, o);
+    }
+    return h;
 }
 
 // FP64 extraction of one row held anywhere (shared or global); one warp.
@@ -1649,18 +1834,18 @@ __device__ __forceinline__ void split_tile(const StepParams<T> &p, int tile, int
                                        s_plan[lrc], t1f, t1g);
                 continue;
             }
-            // FP64: the stored segment products spare FP64 arithmetic, the
-            // bound of that path; FP32 forms them (cheaper than the loads)
+            // FP64 (first steps): the stored segment products spare FP64 arithmetic,
+            // the bound of that path; FP32 forms them (cheaper than the loads)
             const c2 *segr = sizeof(T) == 8 ? Ki.seg + ((size_t)(active ? gi : 1) * G + g) * 2 : nullptr;
             if constexpr (sizeof(T) == 8) {
                 if (use_mat) {
-                    implicit_row_fwd<T, S, true>(Ki, sPhi + lrc * P, sPi + lrc * P, Ki.piv + (size_t)(active ? gi : 1) * N, nullptr, nullptr,
-                                                 N, active, in_tile, g, G, vec, s_plan[lrc], &p.mat, gi, t1f, t1g, segr);
+                    implicit_row_mat<T, S>(Ki, p.mat, sPhi + lrc * P, sPi + lrc * P, gi, N, active, in_tile, g, G, vec,
+                                           s_plan[lrc], t1f, t1g);
                     continue;
                 }
             }
             implicit_row_fwd<T, S>(Ki, sPhi + lrc * P, sPi + lrc * P, Ki.piv + (size_t)(active ? gi : 1) * N, sSt + 2 * lrc * NSF, sTh, N,
-                                   active, in_tile, g, G, vec, s_plan[lrc], nullptr, 0, t1f, t1g, segr);
+                                   active, in_tile, g, G, vec, s_plan[lrc], t1f, t1g, segr);
         }
     };
     // Waveform samples: the tile leaves the extraction row of every state it
@@ -1788,13 +1973,17 @@ __device__ __forceinline__ void split_tile(const StepParams<T> &p, int tile, int
     if (p.nfix >= 0 && p.h_out && ext_row) {
         __syncthreads();
         if (tid < 32) {
-            const bool mine = tid < G;
-            const bool active = mine && p.i_ext >= 1 && p.i_ext <= Nr - 2;
-            c2 *rf = sPhi + lx * P, *rg = sPi + lx * P;
-            implicit_row_one<T, S>(p.half, rf, rg, p.i_ext, sSt + 2 * lx * NSF, sTh, sTh2, N, active, mine, tid & (G - 1), G,
-                                   vec, p.half.plan[p.i_ext]);
-            __syncwarp();
-            const double2 h = sample_warp<T>(p, rf);
+            double2 h;
+            if constexpr (sizeof(T) == 8) {
+                h = seed_dot<T>(p, sPhi + lx * P, sPi + lx * P);
+            } else {
+                const bool mine = tid < G, active = mine && p.i_ext >= 1 && p.i_ext <= Nr - 2;
+                c2 *rf = sPhi + lx * P, *rg = sPi + lx * P;
+                implicit_row_one<T, S>(p.half, rf, rg, p.i_ext, sSt + 2 * lx * NSF, sTh, sTh2, N, active, mine, tid & (G - 1),
+                                       G, vec, p.half.plan[p.i_ext]);
+                __syncwarp();
+                h = sample_warp<T>(p, rf);
+            }
             if (tid == 0) *p.h_out = h;
         }
     }

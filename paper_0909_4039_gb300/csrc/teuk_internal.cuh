@@ -105,27 +105,57 @@ template <typename T> struct ImpConst {
     const c2 *seg;
 };
 
-// Materialised coefficients of the FP64 path: the implicit step of length
-// dt ([Nr][Nth] per element, as imp_elem forms them) and the Lax-Wendroff
-// stages ([2Nr-1][Nth][4]: c_p b, c_p K, 1/Sigma^2 per position and theta).
-// The FP64 pipe is the bound of the FP64 step, so what the step can read
-// instead of recompute it reads.
-template <typename T> struct MatPlanes {
+// Materialised coefficients of the FP64 full step, per grid element.  The
+// FP64 pipe bounds that step: a scheduler starts one FP64 instruction per 64
+// cycles whatever else it does, so every product the step can read it reads,
+// and the planes hold the coefficients in the form that takes the fewest
+// instructions.
+// Implicit stage (implicit_row_mat), [Nr][Nth]: the LU multipliers fk and sub,
+// W times gamma h (d1, w1l, w1u), the second stage's operator 2 gamma (1 -
+// gamma) h^2 W + (1 - gamma) h c_t (d2, w2l, w2u), and pf: the products
+// prod(-e_i sub_i) from the start of the lane segment to the element.
+// Lax-Wendroff stages (lw_segment_mat): both stages as one three-point
+// stencil, [Nr][kLwStencil][Nth] pairs.
+template <typename T> struct StepPlanes {
     typedef typename V2<T>::t c2;
-    const c2 *fk, *dg, *ct;
-    const T *sub, *qam, *qap;
-    const T *lw;
+    const c2 *fk, *d1, *d2, *pf;
+    const T *sub, *w1l, *w1u, *w2l, *w2u;
+    const c2 *lw;
+};
+constexpr int kStepPlaneReals = 13;     // reals per element of the implicit planes
+constexpr int kLwStencil = 4;           // pairs per element of the stencil planes
+
+// What the FP64 adjoint step reads besides the StepPlanes, in its workspace
+// (teuk_adjoint_f64.cu): pb, the products prod(-conj(e_i) sub_{i+1}) from an
+// element to the end of its lane segment, [Nr][Nth]; af, the segments'
+// products of the transposed forward multipliers, [Nr][G]; plan, the scan
+// levels of the transposed solves, [Nr]; the spin derivatives of the stencil
+// (dlw, as StepPlanes::lw) and of the implicit operator (dimp, [Nr][3][Nth] pairs: dW's diagonal, dc_t, dW's off-diagonals);
+// delta, the sample's spin derivative on the extraction row, [2][Nth].
+struct AdjPlanes {
+    const double2 *pb, *af, *dlw, *dimp, *delta;
+    const int *plan;
 };
 
-// The coefficient planes of the adjoint step with the spin derivative, in
-// its workspace (either precision): the full step's MatPlanes, the spin
-// derivatives of the Lax-Wendroff coefficients (dlw, [2Nr-1][Nth][4]:
-// d(c_p b), d(c_p K), d(1/Sigma^2)) and of the implicit operator (dimp,
-// [Nr][Nth][8]: dW's diagonal (2), dc_t (2), dW's off-diagonals, 0, 0).
-template <typename T> struct AdjPlanes {
-    MatPlanes<T> m;
-    const T *dlw, *dimp;
+// Byte layout from offset 0 of their region: pb, af, dlw, dimp, delta, plan.
+struct AdjPlaneLayout {
+    size_t off[6];
+    size_t total;
 };
+inline AdjPlaneLayout adj_plane_layout(long long Nr, long long Nth, int G)
+{
+    const size_t pl = (size_t)Nr * (size_t)Nth, c2 = sizeof(double2);
+    const size_t sz[6] = {pl * c2, (size_t)Nr * (size_t)G * c2, kLwStencil * pl * c2, 3 * pl * c2, 2 * (size_t)Nth * c2,
+                          (size_t)Nr * sizeof(int)};
+    AdjPlaneLayout L;
+    size_t o = 0;
+    for (int k = 0; k < 6; ++k) {
+        L.off[k] = o;
+        o = (o + sz[k] + 255) & ~(size_t)255;
+    }
+    L.total = o;
+    return L;
+}
 
 // One applied step's tape record, in elements of the state's complex type:
 // the first stage value U1 and the implicit stage's output U2 = C_h s_n of
@@ -133,34 +163,6 @@ template <typename T> struct AdjPlanes {
 __host__ __device__ inline size_t tape_u2_off(long long Nr, long long Nth) { return 2 * (size_t)Nr * (size_t)Nth; }
 __host__ __device__ inline size_t tape_x_off(long long Nr, long long Nth) { return 4 * (size_t)Nr * (size_t)Nth; }
 __host__ __device__ inline size_t tape_elems(long long Nr, long long Nth) { return 4 * (size_t)Nr * (size_t)Nth + 2 * (size_t)Nth; }
-
-// Where the generator of k_mat_coef writes (dlw, dimp NULL: no derivatives).
-template <typename T> struct MatOut {
-    typedef typename V2<T>::t c2;
-    c2 *fk, *dg, *ct;
-    T *sub, *qam, *qap, *lw, *dlw, *dimp;
-};
-
-// Byte layout of those planes from offset 0 of their region: plane offsets
-// (fk, dg, ct, sub, qam, qap, lw, dlw, dimp) and the total.
-struct AdjPlaneLayout {
-    size_t off[9];
-    size_t total;
-};
-inline AdjPlaneLayout adj_plane_layout(long long Nr, long long Nth, size_t tsize)
-{
-    const size_t pl = (size_t)Nr * (size_t)Nth, pos = (size_t)(2 * Nr - 1) * (size_t)Nth;
-    const size_t sz[9] = {2 * pl * tsize, 2 * pl * tsize, 2 * pl * tsize, pl * tsize, pl * tsize, pl * tsize,
-                          4 * pos * tsize, 4 * pos * tsize, 8 * pl * tsize};
-    AdjPlaneLayout L;
-    size_t o = 0;
-    for (int k = 0; k < 9; ++k) {
-        L.off[k] = o;
-        o = (o + sz[k] + 255) & ~(size_t)255;
-    }
-    L.total = o;
-    return L;
-}
 
 // Everything a step kernel needs, passed by value.
 template <typename T> struct StepParams {
@@ -184,11 +186,12 @@ template <typename T> struct StepParams {
     const T *rtab;           // [2Nr-1][NRF]
     const T *stab;           // step table [2Nr-1][NSF]
     const T *dstab;          // its derivative with respect to the spin a at fixed r* and theta
-    MatPlanes<T> mat;        // materialised coefficients (mat_on)
+    StepPlanes<T> mat;       // materialised coefficients (mat_on)
     int mat_on;              // 1: full steps read them (FP64 state)
     const T *thtab;          // [NTF][Nth]
     const c2 *patch;         // [np][2][Nth]
     const double *w;         // [Nth]
+    const double2 *seed;     // [2][Nth]: C_{dt/2}^H E^H 1 on the extraction row (FP64 state)
     const c2 *uin;           // [2][Nr][Nth]
     c2 *uout;                // [2][Nr][Nth]
     c2 *mid;                 // literal scheme scratch [2][Nr-1][Nth]
@@ -208,6 +211,7 @@ template <typename T> struct StepParams {
     // [np][2][Nth] (same rows as patch), the amplitude, the r* grid and the
     // orbit's r0*, 1/sigma_r^2, d r0*/d r0 and m dOmega/d r0.
     const c2 *patchu;
+    const double2 *patchd;   // FP64 split scheme: d patch / da, same rows
     int unit_p0, unit_np;    // rows of the unit-amplitude patch (np = 0: none)
     double amp_re, amp_im, rs_min64, drs64, rs0, inv_sig_r2, drs0_dr0, m_dOmega;
     double m_dOmega_da;      // m dOmega/da of the orbit (spin derivative of the source phase)
@@ -315,7 +319,7 @@ __host__ __device__ inline PipeSmem pipe_smem_plan(int R, int N, int tsize)
 
 // ---------------------------------------------------------------- host side
 struct Layout {
-    size_t rtab64, rtabT, stab, dstab, th64, thT, piv, pivh, plan, planh, seg, segh, patch, patchu, w, ctl, raw, staging,
+    size_t rtab64, rtabT, stab, dstab, th64, thT, piv, pivh, plan, planh, seg, segh, patch, patchu, patchd, w, seed, ctl, raw, staging,
         scratch;
     size_t mat, mat_bytes;   // materialised coefficients (FP64 split scheme; 0 bytes otherwise)
     size_t total;
@@ -364,20 +368,24 @@ size_t adjoint_smem_bytes(int tile_rows, int Nth);
 // term).
 template <typename T>
 size_t adjoint_spin_smem_bytes(int tile_rows, int Nth);
-// A: the context's adjoint planes (read for the full steps; a first step,
-// of length dt/2, forms its coefficients from the tables).  tape: the
-// forward step's record (tape_* above) whose stage values replace their
-// recomputation from sin (NULL: recompute).
+// tape: the forward step's record (tape_* above) whose stage values replace
+// their recomputation from sin (NULL: recompute).  FP32, and FP64 first steps.
 template <typename T>
 cudaError_t launch_adjoint_spin(const StepParams<T> &p, int tile_rows, const typename V2<T>::t *sin,
-                                const typename V2<T>::t *tape, const double2 *gseed, const AdjPlanes<T> &A,
-                                double *part, double *acc, cudaStream_t st);
-// The adjoint step without the spin term through the FP64 coefficient
-// planes (the same lam_n and source sums as launch_adjoint_step up to
-// rounding; full steps of FP64 contexts only).
-template <typename T>
-cudaError_t launch_adjoint_planes(const StepParams<T> &p, int tile_rows, const double2 *gseed, const AdjPlanes<T> &A,
-                                  double *part, double *acc, cudaStream_t st);
+                                const typename V2<T>::t *tape, const double2 *gseed, double *part, double *acc,
+                                cudaStream_t st);
+// FP64 full steps on the planes, with or without the spin term (the same lam_n
+// and sums up to rounding), and what fills the planes but delta.
+size_t adjoint_f64_smem_bytes(int tile_rows, int Nth, bool spin);
+cudaError_t launch_adjoint_f64(const StepParams<double> &p, int tile_rows, bool spin, const double2 *sin, const double2 *tape,
+                               const double2 *gseed, const AdjPlanes &A, double *part, double *acc, cudaStream_t st);
+cudaError_t launch_adjoint_f64_planes(const StepParams<double> &p, const AdjPlanes &A, cudaStream_t st);
+// The sample's adjoint vector (p.seed) and its spin derivative, for the
+// weights as they are.
+cudaError_t launch_seed(const StepParams<double> &p, double2 *seed, cudaStream_t st);
+cudaError_t launch_delta(const StepParams<double> &p, double2 *delta, cudaStream_t st);
+// The spin derivative of the source patch into p.patchd (p.patch_np rows).
+cudaError_t launch_patch_da(const StepParams<double> &p, cudaStream_t st);
 template <typename T>
 int adjoint_grid(int Nr, int tile_rows);
 template <typename T>
@@ -454,13 +462,9 @@ template <typename T>
 int pipe_blocks_per_sm(int Nth, int threads, size_t smem);
 template <typename T>
 cudaError_t launch_split_pipe(const StepParams<T> &p, int threads, int grid, size_t smem, cudaStream_t st);
-// Materialised coefficients of the FP64 path into p.mat (no-op unless p.mat_on).
+// The FP64 full step's planes into p.mat (no-op unless p.mat_on).
 template <typename T>
-cudaError_t launch_mat_coef(const StepParams<T> &p, cudaStream_t st);
-// The same planes, plus the spin derivatives where o.dlw / o.dimp are set,
-// into o (either precision).
-template <typename T>
-cudaError_t launch_mat_coef_to(const StepParams<T> &p, const MatOut<T> &o, cudaStream_t st);
+cudaError_t launch_step_planes(const StepParams<T> &p, cudaStream_t st);
 // Largest tile height of the split kernels (rows of the per-tile plan copy).
 constexpr int kMaxTileRows = 254;
 // Batched split step: one CTA of 256 threads per entry of the tile list

@@ -319,8 +319,8 @@ __global__ void __launch_bounds__(NTH, (NTH == 256 && sizeof(T) == 4 && S <= 4) 
                 const int plan = active ? sPl[gi - q.a0] : 0;
                 if constexpr (sizeof(T) == 8) {
                     if (p.mat_on) {
-                        implicit_row_fwd<T, S, true>(K, sPhi + lrc * P, sPi + lrc * P, K.piv + (size_t)(active ? gi : 1) * N, nullptr, nullptr,
-                                                     N, active, in_tile, g, G, vec, plan, &p.mat, gi);
+                        implicit_row_mat<T, S>(K, p.mat, sPhi + lrc * P, sPi + lrc * P, gi, N, active, in_tile, g, G, vec,
+                                               plan);
                         continue;
                     }
                 }
@@ -429,79 +429,59 @@ __global__ void __launch_bounds__(NTH, (NTH == 256 && sizeof(T) == 4 && S <= 4) 
     if (tid == 0) bulk_wait_read();   // the last stores have read their rows before the CTA exits
 }
 
-// Materialised coefficients (MatPlanes): thread (e, j) of the grid covers
-// step-table position e (node 2i or half node 2i+1) and theta j, forming
-// exactly what the kernels would form in place (imp_row, imp_sg, imp_elem
-// for the full step at nodes; lw_coef at every position), and where asked
-// their spin derivatives (lw_coef_da, imp_da) for the adjoint.
-template <typename T>
-__global__ void __launch_bounds__(256) k_mat_coef(const StepParams<T> p, const MatOut<T> o)
+// The FP64 full step's planes (StepPlanes), a thread per grid element.
+template <typename T, int S>
+__global__ void __launch_bounds__(256) k_step_planes(const StepParams<T> p)
 {
     typedef typename V2<T>::t c2;
     const int N = p.Nth, Nr = p.Nr;
     const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= (long long)(2 * Nr - 1) * N) return;
-    const int e = (int)(idx / N), j = (int)(idx - (long long)e * N);
-    const T *f = p.stab + (size_t)e * NSF;
-    const T S2 = p.thtab[TF_S2 * N + j], C = p.thtab[TF_C * N + j];
-    T beta, sg;
-    c2 kap;
-    lw_coef<T>(f, S2, C, beta, kap, &sg);
-    T *lo = o.lw + ((size_t)e * N + j) * 4;
-    lo[0] = beta;
-    lo[1] = kap.x;
-    lo[2] = kap.y;
-    lo[3] = sg;
-    if (o.dlw) {
-        const LwDa<T> d = lw_coef_da<T>(f, p.dstab + (size_t)e * NSF, S2, C);
-        T *dl = o.dlw + ((size_t)e * N + j) * 4;
-        dl[0] = d.dbeta;
-        dl[1] = d.dkap.x;
-        dl[2] = d.dkap.y;
-        dl[3] = d.dsg;
-    }
-    if (e & 1) return;
-    const int i = e >> 1;
-    const size_t q = (size_t)i * N + j;
+    if (idx >= (long long)Nr * N) return;
+    const int i = (int)(idx / N), j = (int)(idx - (long long)i * N);
+    const size_t q = (size_t)idx;
     const c2 zero = cmk<c2>(T(0), T(0));
+    const StepPlanes<T> &M = p.mat;
+    c2 *lw = (c2 *)M.lw + (size_t)i * kLwStencil * N + j;
     if (i < 1 || i > Nr - 2) {
-        // boundary rows: the step treats them as inactive and reads nothing here
-        o.fk[q] = zero;
-        o.dg[q] = zero;
-        o.ct[q] = zero;
-        o.sub[q] = o.qam[q] = o.qap[q] = T(0);
-        if (o.dimp)
-            for (int k = 0; k < 8; ++k) o.dimp[q * 8 + k] = T(0);
+        // boundary rows: the step reads nothing here
+        ((c2 *)M.fk)[q] = ((c2 *)M.d1)[q] = ((c2 *)M.d2)[q] = ((c2 *)M.pf)[q] = zero;
+        ((T *)M.sub)[q] = ((T *)M.w1l)[q] = ((T *)M.w1u)[q] = ((T *)M.w2l)[q] = ((T *)M.w2u)[q] = T(0);
+        for (int k = 0; k < kLwStencil; ++k) lw[k * N] = zero;
         return;
     }
-    const ImpRow<T> r = imp_row(p.full, f);
-    const T am = p.thtab[TF_AM * N + j], a0 = p.thtab[TF_A0 * N + j], ap = p.thtab[TF_AP * N + j];
-    c2 vct, vdg, vfk;
-    T vqam, vqap, vsub;
-    imp_elem(p.full, r, imp_sg(r, S2), C, am, a0, ap, p.full.piv[q], vct, vdg, vqam, vqap, vsub, vfk);
-    o.fk[q] = vfk;
-    o.dg[q] = vdg;
-    o.ct[q] = vct;
-    o.sub[q] = vsub;
-    o.qam[q] = vqam;
-    o.qap[q] = vqap;
-    if (o.dimp) {
-        T fr[8], dfr[8];
-        vload<8>(fr, f);
-        vload<8>(dfr, p.dstab + (size_t)e * NSF);
-        c2 ddg, dct;
-        T dqam, dqap;
-        imp_da<T>(r, fr, dfr, S2, C, am, a0, ap, ddg, dct, dqam, dqap);
-        T *dq = o.dimp + q * 8;
-        dq[0] = ddg.x;
-        dq[1] = ddg.y;
-        dq[2] = dct.x;
-        dq[3] = dct.y;
-        dq[4] = dqam;
-        dq[5] = dqap;
-        dq[6] = T(0);
-        dq[7] = T(0);
+    const ImpConst<T> &K = p.full;
+    const T *f = p.stab + (size_t)(2 * i) * NSF;
+    const ImpRow<T> r = imp_row(K, f);
+    auto elem = [&](int jj, c2 &ct, c2 &dg, T &qam, T &qap, T &sub, c2 &fk) {
+        const T *th = p.thtab + jj;
+        imp_elem(K, r, imp_sg(r, th[TF_S2 * N]), th[TF_C * N], th[TF_AM * N], th[TF_A0 * N], th[TF_AP * N],
+                 K.piv[(size_t)i * N + jj], ct, dg, qam, qap, sub, fk);
+    };
+    c2 ct, dg, fk, P = cmk<c2>(T(1), T(0));
+    T qam, qap, sub;
+    for (int jj = j - j % S; jj <= j; ++jj) {
+        elem(jj, ct, dg, qam, qap, sub, fk);
+        P = cmul(cscale<c2>(-sub, K.piv[(size_t)i * N + jj]), P);
     }
+    ((c2 *)M.fk)[q] = fk;
+    ((c2 *)M.pf)[q] = P;
+    ((T *)M.sub)[q] = sub;
+    ((c2 *)M.d1)[q] = cscale<c2>(K.gh, dg);
+    ((T *)M.w1l)[q] = K.gh * qam;
+    ((T *)M.w1u)[q] = K.gh * qap;
+    ((c2 *)M.d2)[q] = caxpy(K.g2h1, dg, ct);   // ct carries (1 - gamma) h
+    ((T *)M.w2l)[q] = K.g2h1 * qam;
+    ((T *)M.w2u)[q] = K.g2h1 * qap;
+    const T S2 = p.thtab[TF_S2 * N + j], C = p.thtab[TF_C * N + j], half = T(0.5);
+    T b, bm, bp;
+    c2 k, km, kp;
+    lw_coef<T>(f, S2, C, b, k);
+    lw_coef<T>(f - NSF, S2, C, bm, km);
+    lw_coef<T>(f + NSF, S2, C, bp, kp);
+    lw[0] = cmk<c2>(b * (half + bm), b * (half - bp));
+    lw[N] = cmk<c2>(b * (half - bm), b * (half + bp));
+    lw[2 * N] = caxpy(-(half + bm), k, cscale<c2>(b, km));
+    lw[3 * N] = caxpy(half - bp, k, cscale<c2>(b, kp));
 }
 
 }  // namespace
@@ -556,28 +536,15 @@ cudaError_t launch_split_pipe(const StepParams<T> &p, int threads, int grid, siz
 }
 
 template <typename T>
-cudaError_t launch_mat_coef_to(const StepParams<T> &p, const MatOut<T> &o, cudaStream_t st)
+cudaError_t launch_step_planes(const StepParams<T> &p, cudaStream_t st)
 {
-    const long long n = (long long)(2 * p.Nr - 1) * p.Nth;
-    k_mat_coef<T><<<(unsigned)((n + 255) / 256), 256, 0, st>>>(p, o);
-    return cudaGetLastError();
-}
-
-template <typename T>
-cudaError_t launch_mat_coef(const StepParams<T> &p, cudaStream_t st)
-{
-    typedef typename V2<T>::t c2;
     if (!p.mat_on) return cudaSuccess;
-    MatOut<T> o;
-    o.fk = (c2 *)p.mat.fk;
-    o.dg = (c2 *)p.mat.dg;
-    o.ct = (c2 *)p.mat.ct;
-    o.sub = (T *)p.mat.sub;
-    o.qam = (T *)p.mat.qam;
-    o.qap = (T *)p.mat.qap;
-    o.lw = (T *)p.mat.lw;
-    o.dlw = o.dimp = nullptr;
-    return launch_mat_coef_to<T>(p, o, st);
+    const int seg = implicit_seg(p.Nth);
+    auto fn = seg == kSegNarrow ? k_step_planes<T, kSegNarrow>
+                                : (seg == kSeg ? k_step_planes<T, kSeg> : k_step_planes<T, kSegWide>);
+    const long long n = (long long)p.Nr * p.Nth;
+    fn<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(p);
+    return cudaGetLastError();
 }
 
 template <typename T>

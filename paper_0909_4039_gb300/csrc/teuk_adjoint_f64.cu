@@ -396,6 +396,9 @@ __global__ void __launch_bounds__(256, 1)
         __syncthreads();
         if (work) march(j, ra, rb, fm, gm, nf, ng);
     } else {
+        // the march writes its columns in place; the source derivatives above
+        // read whatever columns their elements fall on
+        __syncthreads();
         for (int j = tid; j < N; j += NT) march(j, 1, top, lF[j], lG[j], lF[top * N + j], lG[top * N + j]);
     }
     __syncthreads();

@@ -20,27 +20,28 @@ __device__ __forceinline__ int tile_of_block(int b, int nt, int i_ext, int tile_
 }
 
 // The physical row u = C_{dt/2} s of the extraction row s (planes f, g), in
-// shared memory; one warp.
+// shared memory: all threads load, warp 0 solves (the row is warp 0's).
 template <typename T, int S>
 __device__ __forceinline__ const typename V2<T>::t *physical_row(const StepParams<T> &p, const typename V2<T>::t *f,
                                                                  const typename V2<T>::t *g)
 {
     typedef typename V2<T>::t c2;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int N = p.Nth, Nr = p.Nr, i = p.i_ext, tid = threadIdx.x;
+    const int N = p.Nth, Nr = p.Nr, i = p.i_ext, tid = threadIdx.x, NT = blockDim.x;
     c2 *xPhi = (c2 *)smem_raw;
     c2 *xPi = xPhi + ((N + 1) & ~1);
     T *xF = (T *)(xPi + ((N + 1) & ~1));
     unsigned long long *xTh2 = (unsigned long long *)(xF + NSF);
     T *xTh = (T *)(xTh2 + pair_th_bytes(N, (int)sizeof(T)) / 8);
-    if constexpr (kPaired<T, S>) pair_th_fill(xTh2, p.thtab, N, tid, 32);
-    for (int j = tid; j < N; j += 32) {
+    if constexpr (kPaired<T, S>) pair_th_fill(xTh2, p.thtab, N, tid, NT);
+    for (int j = tid; j < N; j += NT) {
         xPhi[j] = f[j];
         xPi[j] = g[j];
     }
-    if (tid < NSF) xF[tid] = p.stab[(size_t)(2 * i) * NSF + tid];
-    for (int k = tid; k < NTF * N; k += 32) xTh[k] = p.thtab[k];
-    __syncwarp();
+    if (tid >= NT - 32 && tid - (NT - 32) < NSF) xF[tid - (NT - 32)] = p.stab[(size_t)(2 * i) * NSF + tid - (NT - 32)];
+    for (int k = tid; k < NTF * N; k += NT) xTh[k] = p.thtab[k];
+    __syncthreads();
+    if (tid >= 32) return xPhi;
     const int G = p.group;
     const bool mine = tid < G;
     const bool active = mine && i >= 1 && i <= Nr - 2;
@@ -68,6 +69,11 @@ __global__ void __launch_bounds__(32) k_sample(const StepParams<T> p, const type
     if (threadIdx.x == 0) *h_out = h;
 }
 
+// Threads of a sampling CTA: one warp has the row to solve, and four load its
+// tables (7 Ntheta entries one after the other held a lone warp for 10 of the
+// 22 us that a launch of 64 x 16 rows of 128 took).
+constexpr int kSampleThreads = 128;
+
 // CTA (b, instance): the b-th step after ctl->sampled, if it has been taken.
 // The last CTA of an instance moves ctl->sampled on.
 template <typename T, int S>
@@ -78,9 +84,10 @@ __device__ __forceinline__ void sample_step(const StepParams<T> &p)
     // (only the last wave_cap samples stay in the ring: two steps of one slot do not race)
     if (n <= n1 && n > n1 - p.wave_cap) {
         const typename V2<T>::t *r = p.raw + (size_t)(n % kRawSlots) * 2 * p.Nth;
-        extract_warp<T>(p, physical_row<T, S>(p, r, r + p.Nth), n);
+        const typename V2<T>::t *row = physical_row<T, S>(p, r, r + p.Nth);
+        if (threadIdx.x < 32) extract_warp<T>(p, row, n);
     }
-    __syncwarp();
+    __syncthreads();   // (all threads have read the counters)
     if (threadIdx.x == 0) {
         __threadfence();
         if (atomicAdd(&p.ctl->sticket, 1u) == gridDim.x - 1u) {
@@ -91,18 +98,20 @@ __device__ __forceinline__ void sample_step(const StepParams<T> &p)
 }
 
 template <typename T, int S>
-__global__ void __launch_bounds__(32) k_sample_steps(const StepParams<T> p)
+__global__ void __launch_bounds__(kSampleThreads) k_sample_steps(const StepParams<T> p)
 {
+    launch_turn();
     sample_step<T, S>(p);
 }
 
 template <typename T, int S>
-__global__ void __launch_bounds__(32) k_sample_steps_batch(const StepParams<T> *params)
+__global__ void __launch_bounds__(kSampleThreads) k_sample_steps_batch(const StepParams<T> *params)
 {
+    launch_turn();
     __shared__ __align__(16) StepParams<T> sp;
-    for (int k = threadIdx.x; k < (int)(sizeof(StepParams<T>) / 4); k += 32)
+    for (int k = threadIdx.x; k < (int)(sizeof(StepParams<T>) / 4); k += kSampleThreads)
         reinterpret_cast<int *>(&sp)[k] = reinterpret_cast<const int *>(params + blockIdx.y)[k];
-    __syncwarp();
+    __syncthreads();
     sample_step<T, S>(sp);
 }
 
@@ -121,6 +130,7 @@ __global__ void __launch_bounds__(32) k_sample_steps_batch(const StepParams<T> *
 template <typename T, int S>
 __global__ void __launch_bounds__(256, 1) k_adjoint_step(const StepParams<T> p, const double2 *gseed, double *part)
 {
+    launch_turn();
     typedef typename V2<T>::t c2;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ double s_red[8][4];
@@ -584,6 +594,7 @@ __global__ void __launch_bounds__(256, 1) k_adjoint_spin(const StepParams<T> p, 
                                                          const typename V2<T>::t *tape, const double2 *gseed,
                                                          double *part)
 {
+    launch_turn();
     typedef typename V2<T>::t c2;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ double s_red[8][kNPart];
@@ -898,6 +909,7 @@ __global__ void __launch_bounds__(256, 1) k_adjoint_spin(const StepParams<T> p, 
 // acc[c] += sum over the nblk CTAs of part[kNPart b + c], c < kNPart, in a fixed order.
 __global__ void __launch_bounds__(32) k_part_reduce6(const double *part, int nblk, double *acc)
 {
+    launch_turn();
     const int lane = threadIdx.x;
     double v[kNPart] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
     for (int b = lane; b < nblk; b += 32)
@@ -911,6 +923,7 @@ __global__ void __launch_bounds__(32) k_part_reduce6(const double *part, int nbl
 // acc[c] += sum over the nblk CTAs of part[4 b + c], in a fixed order.
 __global__ void __launch_bounds__(32) k_part_reduce(const double *part, int nblk, double *acc)
 {
+    launch_turn();
     const int lane = threadIdx.x;
     double v[4] = {0.0, 0.0, 0.0, 0.0};
     for (int b = lane; b < nblk; b += 32)
@@ -1027,8 +1040,7 @@ cudaError_t launch_sample_steps(const StepParams<T> &p, int pending, cudaStream_
                                 : (seg == kSeg ? k_sample_steps<T, kSeg> : k_sample_steps<T, kSegWide>);
     cudaError_t e = smem_limit_max((const void *)fn);
     if (e != cudaSuccess) return e;
-    fn<<<pending, 32, sample_smem_bytes<T>(p.Nth), st>>>(p);
-    return cudaGetLastError();
+    return launch_dep(fn, dim3((unsigned)pending), kSampleThreads, sample_smem_bytes<T>(p.Nth), st, p);
 }
 
 template <typename T>
@@ -1040,8 +1052,7 @@ cudaError_t launch_sample_steps_batch(const StepParams<T> *d_params, int count, 
                                 : (seg == kSeg ? k_sample_steps_batch<T, kSeg> : k_sample_steps_batch<T, kSegWide>);
     cudaError_t e = smem_limit_max((const void *)fn);
     if (e != cudaSuccess) return e;
-    fn<<<dim3((unsigned)pending, (unsigned)count), 32, sample_smem_bytes<T>(Nmax), st>>>(d_params);
-    return cudaGetLastError();
+    return launch_dep(fn, dim3((unsigned)pending, (unsigned)count), kSampleThreads, sample_smem_bytes<T>(Nmax), st, d_params);
 }
 
 template <typename T>
@@ -1069,11 +1080,9 @@ cudaError_t launch_adjoint_step(const StepParams<T> &p, int tile_rows, const dou
     StepParams<T> q = p;
     q.tile_rows = tile_rows;
     const int grid = adjoint_grid<T>(p.Nr, tile_rows);
-    fn<<<grid, 256, adjoint_smem_bytes<T>(tile_rows, p.Nth), st>>>(q, gseed, part);
-    e = cudaGetLastError();
+    e = launch_dep(fn, dim3((unsigned)grid), 256, adjoint_smem_bytes<T>(tile_rows, p.Nth), st, q, gseed, part);
     if (e != cudaSuccess) return e;
-    k_part_reduce<<<1, 32, 0, st>>>(part, grid, acc);
-    return cudaGetLastError();
+    return launch_dep(k_part_reduce, dim3(1), 32, 0, st, part, grid, acc);
 }
 
 template <typename T>
@@ -1086,8 +1095,7 @@ size_t adjoint_spin_smem_bytes(int tile_rows, int Nth)
 
 cudaError_t launch_part_reduce(const double *part, int nblk, double *acc, cudaStream_t st)
 {
-    k_part_reduce6<<<1, 32, 0, st>>>(part, nblk, acc);
-    return cudaGetLastError();
+    return launch_dep(k_part_reduce6, dim3(1), 32, 0, st, part, nblk, acc);
 }
 
 template <typename T>
@@ -1103,8 +1111,7 @@ cudaError_t launch_adjoint_spin(const StepParams<T> &p, int tile_rows, const typ
     StepParams<T> q = p;
     q.tile_rows = tile_rows;
     const int grid = adjoint_grid<T>(p.Nr, tile_rows);
-    fn<<<grid, 256, adjoint_spin_smem_bytes<T>(tile_rows, p.Nth), st>>>(q, sin, tape, gseed, part);
-    e = cudaGetLastError();
+    e = launch_dep(fn, dim3((unsigned)grid), 256, adjoint_spin_smem_bytes<T>(tile_rows, p.Nth), st, q, sin, tape, gseed, part);
     if (e != cudaSuccess) return e;
     return launch_part_reduce(part, grid, acc, st);
 }

@@ -205,6 +205,7 @@ __global__ void __launch_bounds__(256, 1)
     k_adjoint_f64(const StepParams<double> p, const double2 *sin, const double2 *tape, const double2 *gseed,
                   const AdjPlanes A, double *part)
 {
+    launch_turn();
     typedef double2 c2;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ double s_red[8][kNPart];
@@ -579,8 +580,7 @@ cudaError_t launch_adjoint_f64(const StepParams<double> &p, int tile_rows, bool 
     StepParams<double> q = p;
     q.tile_rows = tile_rows;
     const int grid = (p.Nr + tile_rows - 1) / tile_rows;
-    fn<<<grid, 256, adjoint_f64_smem_bytes(tile_rows, p.Nth, spin), st>>>(q, sin, tape, gseed, A, part);
-    e = cudaGetLastError();
+    e = launch_dep(fn, dim3((unsigned)grid), 256, adjoint_f64_smem_bytes(tile_rows, p.Nth, spin), st, q, sin, tape, gseed, A, part);
     if (e != cudaSuccess) return e;
     return launch_part_reduce(part, grid, acc, st);
 }

@@ -959,7 +959,7 @@ int teuk_step(teuk_ctx *c, int64_t nsteps, void *stream)
     }
     const bool split = c->d.scheme == TEUK_SCHEME_SPLIT;
     // the pipelined and persistent kernels sample their own steps: what is left
-    // from before them comes first (as before a graph, whose chunk is its own)
+    // from before them comes first
     auto flush = [&]() -> cudaError_t {
         if (!split || pending == 0) return cudaSuccess;
         const int n = pending;
@@ -971,7 +971,7 @@ int teuk_step(teuk_ctx *c, int64_t nsteps, void *stream)
     // steps per captured graph: a multiple of ks over an even number of launches
     const int chunk = ks == 3 ? 3 * kGraphChunk / 2 : kGraphChunk;
     bool use_graph = st != nullptr && c->d.scheme == TEUK_SCHEME_SPLIT && left >= 2 * chunk;
-    if (use_graph || c->pipe || c->persist) CK(flush(), "samples");
+    if (c->pipe || c->persist) CK(flush(), "samples");
     if (use_graph) {
         int g = c->cur;
         if (c->graph[g] && c->graph_stream[g] != st) {
@@ -989,7 +989,6 @@ int teuk_step(teuk_ctx *c, int64_t nsteps, void *stream)
                 done += k;
                 lev ^= 1;
             }
-            if (le == cudaSuccess) le = sample_steps(c, chunk, st);
             cudaError_t ee = cudaStreamEndCapture(st, &graph);
             if (le != cudaSuccess) return cuda_err(c, le, "captured launch");
             if (ee != cudaSuccess) return cuda_err(c, ee, "end capture");
@@ -1002,12 +1001,15 @@ int teuk_step(teuk_ctx *c, int64_t nsteps, void *stream)
             c->graph_stream[g] = st;
         }
         while (left >= chunk) {
+            if (pending + chunk > kRawSlots) CK(flush(), "samples");
             CK(cudaGraphLaunch(c->graph[g], st), "graph launch");
             left -= chunk;
+            pending += chunk;
         }
     }
     while (left > 0) {
         int k = 1;
+        if (pending + ks > kRawSlots) CK(flush(), "samples");
         if (left >= ks) {
             CK(launch_unit(c, c->cur, st, &k), "step launch");
         } else {
@@ -1016,7 +1018,6 @@ int teuk_step(teuk_ctx *c, int64_t nsteps, void *stream)
         c->cur ^= 1;
         left -= k;
         pending += k;
-        if (pending + ks > kRawSlots) CK(flush(), "samples");
     }
     CK(flush(), "samples");
     c->step += nsteps;
@@ -1851,8 +1852,6 @@ int batch_step_impl(teuk_batch *b, int64_t nsteps, cudaStream_t st)
         if (r != TEUK_OK) return r;
     }
     if (st != nullptr && left >= 2 * kGraphChunk) {
-        if (pending > 0) BCK(samples(pending), "samples");
-        pending = 0;
         if (b->graph && b->graph_stream != st) {
             cudaGraphExecDestroy(b->graph);
             b->graph = nullptr;
@@ -1863,7 +1862,6 @@ int batch_step_impl(teuk_batch *b, int64_t nsteps, cudaStream_t st)
             cudaError_t le = cudaSuccess;
             // kGraphChunk / ks launches: an even count, so the level parity is unchanged
             for (int k = 0; k < kGraphChunk / b->ks && le == cudaSuccess; ++k) le = batch_launch(b, k & 1, b->ks, st);
-            if (le == cudaSuccess) le = samples(kGraphChunk);
             cudaError_t ee = cudaStreamEndCapture(st, &graph);
             if (le != cudaSuccess) return bcuda_err(b, le, "captured batched launch");
             if (ee != cudaSuccess) return bcuda_err(b, ee, "end capture");
@@ -1876,21 +1874,26 @@ int batch_step_impl(teuk_batch *b, int64_t nsteps, cudaStream_t st)
             b->graph_stream = st;
         }
         while (left >= kGraphChunk) {
+            if (pending + kGraphChunk > kRawSlots) {
+                BCK(samples(pending), "samples");
+                pending = 0;
+            }
             BCK(cudaGraphLaunch(b->graph, st), "graph launch");
             left -= kGraphChunk;
+            pending += kGraphChunk;
         }
     }
     // each launch (one or two steps) flips every instance's level once
     int64_t launches = 0;
     for (; left > 0; ++launches) {
         const int k = left >= b->ks ? b->ks : 1;
-        BCK(batch_launch(b, (int)(launches & 1), k, st), "batched step");
-        left -= k;
-        pending += k;
-        if (left == 0 || pending + b->ks > kRawSlots) {
+        if (pending + k > kRawSlots) {
             BCK(samples(pending), "samples");
             pending = 0;
         }
+        BCK(batch_launch(b, (int)(launches & 1), k, st), "batched step");
+        left -= k;
+        pending += k;
     }
     if (pending > 0) BCK(samples(pending), "samples");
     for (teuk_ctx *c : b->c) {

@@ -1634,6 +1634,17 @@ __device__ void extract_warp(const StepParams<T> &p, const typename V2<T>::t *ro
     for (int j = lane; j < N; j += 32) dst[1 + j] = make_double2((double)row[j].x, (double)row[j].y);
 }
 
+// Programmatic dependent launches (launch_dep): a kernel waits for all that the
+// stream holds before it, then lets the next launch's CTAs take the SMs its own
+// CTAs leave.  Nothing is read or written before the wait, so the order of
+// memory on the stream is that of plain launches; what it spares is the gap
+// between two launches, in which the next one's CTAs are set up.
+__device__ __forceinline__ void launch_turn()
+{
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 // Fused step of the split scheme (merged Strang composition): the tile's
 // input is s_n (or the physical state u_n when p.first), the output is
 //   s_{n+1} = LW_n C_h s_n,   h = dt (h = dt/2 when p.first),
@@ -1655,6 +1666,7 @@ __device__ __forceinline__ void split_tile(const StepParams<T> &p, int tile, int
     constexpr int kMaxChunks = 8;
     static_assert(KS >= 1 && KS <= 3, "one to three steps per launch");
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ long long s_n;   // step index of the input state
     __shared__ double2 sph[2 * KS];
     __shared__ __align__(8) unsigned long long s_mbar[kMaxChunks];
     __shared__ int s_plan[kMaxTileRows + 6];   // stored scan levels of the tile rows
@@ -1687,9 +1699,37 @@ __device__ __forceinline__ void split_tile(const StepParams<T> &p, int tile, int
             }
         }
     }
-    // The step index is read before the first barrier; after it the last CTA
-    // to have read it advances it (below).
-    const long long n_in = p.nfix >= 0 ? p.nfix : *((volatile long long *)&p.ctl->step);
+    // The last warp reads the step index while thread 0 starts the copies.
+    if (tid >= NT - 32) {
+        const int q = tid - (NT - 32);
+        const long long n = p.nfix >= 0 ? p.nfix : *((volatile long long *)&p.ctl->step);
+        __syncwarp();
+        if (q == 0) {
+            s_n = n;
+            if (!p.imp_only && p.nfix < 0) {
+                // The last CTA to read the step index advances it.  Later kernels
+                // on the stream see the new value; no CTA of this launch reads it
+                // again, so no CTA has to wait for its own stores first.
+                __threadfence();
+                unsigned t = atomicAdd(&p.ctl->ticket, 1u);
+                if (t == (unsigned)ntiles - 1u) {
+                    p.ctl->ticket = 0u;
+                    p.ctl->step = n + KS;
+                }
+            }
+        }
+        // Source phases of Eqs. 13 and 14 times their stage lengths dt/2 and dt,
+        // one lane each.  An FP64 sincos takes about 3 us of one warp; taken one
+        // after the other by the thread that starts the tile's copies, the 2 KS
+        // of them held a source tile, and with it the launch, for 6 us a step.
+        // (Done here and not after the tables' barrier: with the row solve's
+        // registers live there, the batch's tiles took 1 % longer.)
+        if (src && q < 2 * KS) {
+            const double t = (double)(n + (q >> 1)) * p.dt64, len = (q & 1) ? p.dt64 : 0.5 * p.dt64;
+            const double2 e = phase_at(p.mOmega, (q & 1) ? t + 0.5 * p.dt64 : t);
+            sph[q] = make_double2(len * e.x, len * e.y);
+        }
+    }
     // ---- A: tile rows g0 .. g0+R-1 (state), r and theta tables; the row
     // solves read their pivots from global memory (L2), which leaves room for
     // taller tiles
@@ -1771,28 +1811,6 @@ __device__ __forceinline__ void split_tile(const StepParams<T> &p, int tile, int
         s_plan[lr] = (gi >= 0 && gi < Nr) ? K.plan[gi] : 0;
     }
     __syncthreads();
-    if (tid == 0 && !p.imp_only && p.nfix < 0) {
-        // The last CTA to read the step index advances it.  Later kernels
-        // on the stream see the new value; no CTA of this launch reads it
-        // again, so no CTA has to wait for its own stores first.
-        __threadfence();
-        unsigned t = atomicAdd(&p.ctl->ticket, 1u);
-        if (t == (unsigned)ntiles - 1u) {
-            p.ctl->ticket = 0u;
-            p.ctl->step = n_in + KS;
-        }
-    }
-    // Source phases of Eqs. 13 and 14 times their stage lengths dt/2 and dt:
-    // one lane each, in the last warp, which short tiles leave idle in the
-    // implicit stage.  An FP64 sincos takes about 3 us of one warp; taken one
-    // after the other by the thread that starts the tile's copies, the 2 KS of
-    // them held a source tile, and with it the launch, for 6 us a step.
-    if (src && tid >= NT - 32 && tid - (NT - 32) < 2 * KS) {
-        const int q = tid - (NT - 32);
-        const double t = (double)(n_in + (q >> 1)) * p.dt64, len = (q & 1) ? p.dt64 : 0.5 * p.dt64;
-        const double2 e = phase_at(p.mOmega, (q & 1) ? t + 0.5 * p.dt64 : t);
-        sph[q] = make_double2(len * e.x, len * e.y);
-    }
     const int g = tid & (G - 1), tq = tid >> lgG;   // lane in the row group, row of the pass
     const int wq = (tid & ~31) >> lgG;              // first row of the warp's in the pass
     const bool vec = p.vec != 0;
@@ -1940,7 +1958,7 @@ __device__ __forceinline__ void split_tile(const StepParams<T> &p, int tile, int
         }
         __syncthreads();
         if (ext) {
-            leave_row(n_in + k + 1);
+            leave_row(s_n + k + 1);
             if (k + 1 < KS) __syncthreads();   // the next implicit stage works in place
         }
     }
@@ -1969,22 +1987,26 @@ __device__ __forceinline__ void split_tile(const StepParams<T> &p, int tile, int
         }
     }
     if (p.imp_only) return;
-    // ---- E: a step applied to caller buffers writes the sample of its output, to h_out
-    if (p.nfix >= 0 && p.h_out && ext_row) {
-        __syncthreads();
-        if (tid < 32) {
-            double2 h;
-            if constexpr (sizeof(T) == 8) {
-                h = seed_dot<T>(p, sPhi + lx * P, sPi + lx * P);
-            } else {
-                const bool mine = tid < G, active = mine && p.i_ext >= 1 && p.i_ext <= Nr - 2;
-                c2 *rf = sPhi + lx * P, *rg = sPi + lx * P;
-                implicit_row_one<T, S>(p.half, rf, rg, p.i_ext, sSt + 2 * lx * NSF, sTh, sTh2, N, active, mine, tid & (G - 1),
-                                       G, vec, p.half.plan[p.i_ext]);
-                __syncwarp();
-                h = sample_warp<T>(p, rf);
+    // ---- E: a step applied to caller buffers writes the sample of its output,
+    // to h_out.  (Such steps run one per launch; compiled into the multi-step
+    // kernels too, this second row solve cost the batch's tiles 1 %.)
+    if constexpr (KS == 1) {
+        if (p.nfix >= 0 && p.h_out && ext_row) {
+            __syncthreads();
+            if (tid < 32) {
+                double2 h;
+                if constexpr (sizeof(T) == 8) {
+                    h = seed_dot<T>(p, sPhi + lx * P, sPi + lx * P);
+                } else {
+                    const bool mine = tid < G, active = mine && p.i_ext >= 1 && p.i_ext <= Nr - 2;
+                    c2 *rf = sPhi + lx * P, *rg = sPi + lx * P;
+                    implicit_row_one<T, S>(p.half, rf, rg, p.i_ext, sSt + 2 * lx * NSF, sTh, sTh2, N, active, mine,
+                                           tid & (G - 1), G, vec, p.half.plan[p.i_ext]);
+                    __syncwarp();
+                    h = sample_warp<T>(p, rf);
+                }
+                if (tid == 0) *p.h_out = h;
             }
-            if (tid == 0) *p.h_out = h;
         }
     }
 }
@@ -1995,6 +2017,23 @@ __device__ __forceinline__ void mbar_arrive(unsigned long long *m)
 }
 
 }  // namespace
+
+// Launches a kernel that begins with launch_turn().
+template <typename... P, typename... A>
+static inline cudaError_t launch_dep(void (*fn)(P...), dim3 grid, unsigned threads, size_t smem, cudaStream_t st, A &&...args)
+{
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, fn, std::forward<A>(args)...);
+}
 
 // Raise a kernel's dynamic shared-memory limit to the device maximum, once
 // per kernel and device.  Occupancy queries and launches never lower it, so

@@ -36,8 +36,8 @@ cudaError_t launch_pair_step(const StepParams<float> &p, int ks, cudaStream_t st
     auto fn = pair_fn(ks);
     cudaError_t e = smem_limit_max((const void *)fn);
     if (e != cudaSuccess) return e;
-    fn<<<(p.Nr + p.tile_rows - 1) / p.tile_rows, 256, pair_smem_bytes(p.tile_rows, p.Nth, ks), st>>>(p);
-    return cudaGetLastError();
+    return launch_dep(fn, dim3((unsigned)((p.Nr + p.tile_rows - 1) / p.tile_rows)), 256,
+                      pair_smem_bytes(p.tile_rows, p.Nth, ks), st, p);
 }
 
 cudaError_t launch_pair_batch(const StepParams<float> *d_params, const int2 *d_tiles, int ntiles, size_t smem, int ks,
@@ -47,8 +47,7 @@ cudaError_t launch_pair_batch(const StepParams<float> *d_params, const int2 *d_t
     cudaError_t e = smem_limit_max((const void *)fn);
     if (e != cudaSuccess) return e;
     if (ntiles < 1) return cudaSuccess;
-    fn<<<ntiles, 256, smem, st>>>(d_params, d_tiles);
-    return cudaGetLastError();
+    return launch_dep(fn, dim3((unsigned)ntiles), 256, smem, st, d_params, d_tiles);
 }
 
 }  // namespace teuk

@@ -454,6 +454,7 @@ __device__ __forceinline__ void pair_tile(const StepParams<float> &p, int tile, 
 template <int KS>
 __global__ void __launch_bounds__(256, 1) k_pair_step(const StepParams<float> p)
 {
+    launch_turn();
     pair_tile<KS>(p, (int)blockIdx.x, (int)gridDim.x);
 }
 
@@ -462,6 +463,7 @@ template <int KS>
 __global__ void __launch_bounds__(256, 1) k_pair_batch(const StepParams<float> *params, const int2 *tiles)
 {
     __shared__ __align__(16) StepParams<float> sp;
+    launch_turn();
     const int2 e = tiles[blockIdx.x];
     if (threadIdx.x < sizeof(StepParams<float>) / 4)
         reinterpret_cast<int *>(&sp)[threadIdx.x] = reinterpret_cast<const int *>(params + e.x)[threadIdx.x];

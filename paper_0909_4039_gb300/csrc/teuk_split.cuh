@@ -34,6 +34,7 @@ namespace {
 template <typename T, int S>
 __global__ void __launch_bounds__(256, (sizeof(T) == 4 && S <= 4) ? 2 : 1) k_split_step(const StepParams<T> p)
 {
+    launch_turn();
     split_tile<T, S, 1>(p, (int)blockIdx.x, (int)gridDim.x);
 }
 
@@ -41,6 +42,7 @@ __global__ void __launch_bounds__(256, (sizeof(T) == 4 && S <= 4) ? 2 : 1) k_spl
 template <typename T, int S>
 __global__ void __launch_bounds__(256, (sizeof(T) == 4 && S <= 4) ? 2 : 1) k_split_step2(const StepParams<T> p)
 {
+    launch_turn();
     split_tile<T, S, 2>(p, (int)blockIdx.x, (int)gridDim.x);
 }
 
@@ -49,6 +51,7 @@ __global__ void __launch_bounds__(256, (sizeof(T) == 4 && S <= 4) ? 2 : 1) k_spl
 template <typename T, int S>
 __global__ void __launch_bounds__(256, (sizeof(T) == 4 && S <= 4) ? 2 : 1) k_split_step3(const StepParams<T> p)
 {
+    launch_turn();
     split_tile<T, S, 3>(p, (int)blockIdx.x, (int)gridDim.x);
 }
 
@@ -64,6 +67,7 @@ __global__ void __launch_bounds__(256, (sizeof(T) == 4 && S <= 4) ? 2 : 1)
 {
     __shared__ __align__(16) StepParams<T> sp;
     static_assert(sizeof(StepParams<T>) % 4 == 0 && sizeof(StepParams<T>) <= 4 * 256, "parameter copy");
+    launch_turn();
     const int2 e = tiles[blockIdx.x];
     if (threadIdx.x < sizeof(StepParams<T>) / 4)
         reinterpret_cast<int *>(&sp)[threadIdx.x] = reinterpret_cast<const int *>(params + e.x)[threadIdx.x];
@@ -602,8 +606,7 @@ cudaError_t launch_split_step(const StepParams<T> &p, int threads, size_t smem, 
     cudaError_t e = smem_limit_max((const void *)fn);
     if (e != cudaSuccess) return e;
     int grid = (p.Nr + p.tile_rows - 1) / p.tile_rows;
-    fn<<<grid, threads, smem, st>>>(p);
-    return cudaGetLastError();
+    return launch_dep(fn, dim3((unsigned)grid), (unsigned)threads, smem, st, p);
 }
 
 template <typename T>
@@ -641,8 +644,7 @@ cudaError_t launch_split_batch(const StepParams<T> *d_params, const int2 *d_tile
     cudaError_t e = smem_limit_max((const void *)fn);
     if (e != cudaSuccess) return e;
     if (ntiles < 1) return cudaSuccess;
-    fn<<<ntiles, 256, smem, st>>>(d_params, d_tiles);
-    return cudaGetLastError();
+    return launch_dep(fn, dim3((unsigned)ntiles), 256, smem, st, d_params, d_tiles);
 }
 
 template <typename T>
@@ -700,8 +702,7 @@ cudaError_t launch_split_step2(const StepParams<T> &p, int threads, size_t smem,
     cudaError_t e = smem_limit_max((const void *)fn);
     if (e != cudaSuccess) return e;
     int grid = (p.Nr + p.tile_rows - 1) / p.tile_rows;
-    fn<<<grid, threads, smem, st>>>(p);
-    return cudaGetLastError();
+    return launch_dep(fn, dim3((unsigned)grid), (unsigned)threads, smem, st, p);
 }
 
 template <typename T>
@@ -751,8 +752,7 @@ cudaError_t launch_split_step3(const StepParams<T> &p, int threads, size_t smem,
     cudaError_t e = smem_limit_max((const void *)fn);
     if (e != cudaSuccess) return e;
     int grid = (p.Nr + p.tile_rows - 1) / p.tile_rows;
-    fn<<<grid, threads, smem, st>>>(p);
-    return cudaGetLastError();
+    return launch_dep(fn, dim3((unsigned)grid), (unsigned)threads, smem, st, p);
 }
 
 }  // namespace teuk

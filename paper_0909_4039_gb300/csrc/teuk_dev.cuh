@@ -1645,22 +1645,34 @@ __device__ __forceinline__ void launch_turn()
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
+// The parameters of a batch tile's instance, with the tile's height (256 threads).
+template <typename T>
+__device__ __forceinline__ void batch_params(StepParams<T> &sp, const StepParams<T> *params, int2 e)
+{
+    static_assert(sizeof(StepParams<T>) % 4 == 0 && sizeof(StepParams<T>) <= 4 * 256, "parameter copy");
+    const int *src = reinterpret_cast<const int *>(params + (e.x & ((1 << kTileShift) - 1)));
+    if (threadIdx.x < sizeof(StepParams<T>) / 4)
+        reinterpret_cast<int *>(&sp)[threadIdx.x] =
+            threadIdx.x == offsetof(StepParams<T>, tile_rows) / 4 ? (int)((unsigned)e.x >> kTileShift) : src[threadIdx.x];
+    __syncthreads();
+}
+
 // Fused step of the split scheme (merged Strang composition): the tile's
 // input is s_n (or the physical state u_n when p.first), the output is
 //   s_{n+1} = LW_n C_h s_n,   h = dt (h = dt/2 when p.first),
 // and the physical sample u_{n+1} = C_{dt/2} s_{n+1} is taken on the
 // extraction row.  With p.imp_only the kernel only applies C_{dt/2} to the
 // tile rows (used to output the physical state).
-// The work of one CTA: tile number `tile` of the grid described by p, whose
-// step takes `ntiles` CTAs (the last of them to start advances the step
+// The work of one CTA: the tile of p.tile_rows rows from row i0 of the grid
+// described by p, whose step takes `ntiles` CTAs (the last of them to start advances the step
 // index), for KS = 1, 2 or 3 time steps per launch.  The tile holds its TR
 // output rows plus KS halo rows on either side (R = TR + 2 KS; tile row lr is
 // global row g0 + lr, g0 = i0 - KS).  Step k (from 0) updates rows
 // k + 1 .. R - 2 - k, so the last one updates the TR output rows; the state
 // read and written per step falls to 1/KS at the cost of recomputing the
 // extra halo rows.  The result is bitwise that of KS single steps.
-template <typename T, int S, int KS>
-__device__ __forceinline__ void split_tile(const StepParams<T> &p, int tile, int ntiles)
+template <typename T, int S, int KS, bool OWN = false>
+__device__ __forceinline__ void split_tile(const StepParams<T> &p, int i0, int ntiles)
 {
     typedef typename V2<T>::t c2;
     constexpr int kMaxChunks = 8;
@@ -1672,7 +1684,7 @@ __device__ __forceinline__ void split_tile(const StepParams<T> &p, int tile, int
     __shared__ int s_plan[kMaxTileRows + 6];   // stored scan levels of the tile rows
     const int Nr = p.Nr, N = p.Nth, TR = p.tile_rows, R = TR + 2 * KS, P = p.pitch;
     const int tid = threadIdx.x, NT = blockDim.x;
-    const int i0 = tile * TR, g0 = i0 - KS;
+    const int g0 = i0 - KS;
     const int G = p.group;
 
     const SplitSmem plan = split_smem_plan(R, N, (int)sizeof(T));
@@ -1870,7 +1882,8 @@ __device__ __forceinline__ void split_tile(const StepParams<T> &p, int tile, int
     // forms in p.raw, and one sampling launch per chunk of steps solves and sums
     // those rows side by side (launch_sample_steps).  Solved here, one row by
     // one warp in every step, they ended the tile's every step: 17 of a
-    // 1024 x 32 FP64 step's 35 us.
+    // 1024 x 32 FP64 step's 35 us.  OWN: the tile samples its steps all the
+    // same (kOwnSamples).
     const bool ext_row = p.i_ext >= i0 && p.i_ext < i0 + TR && p.i_ext < Nr;
     const bool ext = !p.imp_only && p.nfix < 0 && ext_row;
     const int lx = p.i_ext - g0;
@@ -1879,6 +1892,16 @@ __device__ __forceinline__ void split_tile(const StepParams<T> &p, int tile, int
         for (int j = tid; j < N; j += NT) {
             dst[j] = sPhi[lx * P + j];
             dst[N + j] = sPi[lx * P + j];
+        }
+    };
+    auto own_sample = [&](c2 *rf, c2 *rg, long long n) {
+        if (tid < 32) {
+            const bool mine = tid < G, active = mine && p.i_ext >= 1 && p.i_ext <= Nr - 2;
+            implicit_row_one<T, S>(p.half, rf, rg, p.i_ext, sSt + 2 * lx * NSF, sTh, sTh2, N, active, mine, tid & (G - 1), G,
+                                   vec, p.half.plan[p.i_ext]);
+            __syncwarp();
+            extract_warp<T>(p, rf, n);
+            if (tid == 0) p.ctl->sampled = n;
         }
     };
     // ---- B and C, once per time step of the launch.  Step k (from 0) runs
@@ -1957,7 +1980,19 @@ __device__ __forceinline__ void split_tile(const StepParams<T> &p, int tile, int
                 lw_phase<T, false>(p, sPhi, sPi, sSt, sTh, k + 1, R - 2 - 2 * k, g0, tid, NT, src, ph1, ph2, sync_all);
         }
         __syncthreads();
-        if (ext) {
+        if constexpr (OWN) {
+            if (ext && k + 1 < KS) {
+                // from a copy: the row itself goes on into the next step
+                c2 *xPhi = (c2 *)(smem_raw + plan.total), *xPi = xPhi + N;
+                if (tid < 32)
+                    for (int j = tid; j < N; j += 32) {
+                        xPhi[j] = sPhi[lx * P + j];
+                        xPi[j] = sPi[lx * P + j];
+                    }
+                __syncthreads();
+                own_sample(xPhi, xPi, s_n + k + 1);
+            }
+        } else if (ext) {
             leave_row(s_n + k + 1);
             if (k + 1 < KS) __syncthreads();   // the next implicit stage works in place
         }
@@ -1990,7 +2025,12 @@ __device__ __forceinline__ void split_tile(const StepParams<T> &p, int tile, int
     // ---- E: a step applied to caller buffers writes the sample of its output,
     // to h_out.  (Such steps run one per launch; compiled into the multi-step
     // kernels too, this second row solve cost the batch's tiles 1 %.)
-    if constexpr (KS == 1) {
+    if constexpr (OWN) {
+        if (ext) {
+            __syncthreads();
+            own_sample(sPhi + lx * P, sPi + lx * P, s_n + KS);
+        }
+    } else if constexpr (KS == 1) {
         if (p.nfix >= 0 && p.h_out && ext_row) {
             __syncthreads();
             if (tid < 32) {

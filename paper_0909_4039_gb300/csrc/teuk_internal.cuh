@@ -169,6 +169,7 @@ template <typename T> struct StepParams {
     typedef typename V2<T>::t c2;
     int Nr, Nth;
     int tile_rows;           // output rows per CTA (split kernel)
+    int ntiles;              // batches: tiles of the instance
     int pitch;               // shared-memory row pitch in complex elements
     int group;               // threads per theta row in the implicit phase
     int first;               // 1: implicit step dt/2 (input is a physical state)
@@ -223,6 +224,14 @@ constexpr double kPi = 3.14159265358979323846264338327950;
 
 // Lane segments of the implicit row solves.
 constexpr int kSegNarrow = 4;           // theta elements per thread (Ntheta <= 128)
+// Whether a batch's tiles sample their own steps: FP32 rows of up to 128 theta
+// points (seg: the segment).  Two CTAs share an SM there and hundreds of tiles
+// are left to run while one warp solves a row; leaving the rows to a sampling
+// launch took 1.6 % longer (16 uneven instances, 130 steps: 15.64 against
+// 15.39 ms).  A lone state's launch, of few tiles, ends with that warp.
+constexpr bool own_samples(size_t real_bytes, int seg) { return real_bytes == 4 && seg == kSegNarrow; }
+// A batch's tile list: entry (instance | height << kTileShift, first row).
+constexpr int kTileShift = 23;
 constexpr int kSeg = 8;                 // theta elements per thread (Ntheta <= 256)
 constexpr int kSegWide = 32;            // theta elements per thread (Ntheta <= 1024)
 // theta elements per thread of the implicit row solves

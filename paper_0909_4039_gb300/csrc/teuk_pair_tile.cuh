@@ -89,7 +89,7 @@ __device__ __forceinline__ int lw_pair_field(int q)
 // The work of one CTA, as split_tile's for full steps of a context (no first
 // step, no state output, no caller buffers).
 template <int KS>
-__device__ __forceinline__ void pair_tile(const StepParams<float> &p, int tile, int ntiles)
+__device__ __forceinline__ void pair_tile(const StepParams<float> &p, int i0, int ntiles)
 {
     constexpr int kMaxChunks = 8;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -99,7 +99,7 @@ __device__ __forceinline__ void pair_tile(const StepParams<float> &p, int tile, 
     const int Nr = p.Nr, N = p.Nth, TR = p.tile_rows, R = TR + 2 * KS;
     constexpr int NP = 128, NL = 32;                 // pairs of a row, lanes
     const int tid = threadIdx.x, NT = blockDim.x, lane = tid & 31;
-    const int i0 = tile * TR, g0 = i0 - KS;
+    const int g0 = i0 - KS;
     const PairSmem L = pair_smem_plan(R, N);
     unsigned char *sPhi = smem_raw + L.phi, *sPi = smem_raw + L.pi;
     constexpr unsigned bb = NP * 16u;                // bytes of a row of pairs
@@ -455,7 +455,7 @@ template <int KS>
 __global__ void __launch_bounds__(256, 1) k_pair_step(const StepParams<float> p)
 {
     launch_turn();
-    pair_tile<KS>(p, (int)blockIdx.x, (int)gridDim.x);
+    pair_tile<KS>(p, (int)blockIdx.x * p.tile_rows, (int)gridDim.x);
 }
 
 // Batched form, as k_split_batch: entry blockIdx.x of the tile list.
@@ -465,10 +465,8 @@ __global__ void __launch_bounds__(256, 1) k_pair_batch(const StepParams<float> *
     __shared__ __align__(16) StepParams<float> sp;
     launch_turn();
     const int2 e = tiles[blockIdx.x];
-    if (threadIdx.x < sizeof(StepParams<float>) / 4)
-        reinterpret_cast<int *>(&sp)[threadIdx.x] = reinterpret_cast<const int *>(params + e.x)[threadIdx.x];
-    __syncthreads();
-    pair_tile<KS>(sp, e.y, (sp.Nr + sp.tile_rows - 1) / sp.tile_rows);
+    batch_params(sp, params, e);
+    pair_tile<KS>(sp, e.y, sp.ntiles);
 }
 
 }  // namespace

@@ -35,7 +35,7 @@ template <typename T, int S>
 __global__ void __launch_bounds__(256, (sizeof(T) == 4 && S <= 4) ? 2 : 1) k_split_step(const StepParams<T> p)
 {
     launch_turn();
-    split_tile<T, S, 1>(p, (int)blockIdx.x, (int)gridDim.x);
+    split_tile<T, S, 1>(p, (int)blockIdx.x * p.tile_rows, (int)gridDim.x);
 }
 
 // Two time steps per launch (temporal blocking): see split_tile.
@@ -43,7 +43,7 @@ template <typename T, int S>
 __global__ void __launch_bounds__(256, (sizeof(T) == 4 && S <= 4) ? 2 : 1) k_split_step2(const StepParams<T> p)
 {
     launch_turn();
-    split_tile<T, S, 2>(p, (int)blockIdx.x, (int)gridDim.x);
+    split_tile<T, S, 2>(p, (int)blockIdx.x * p.tile_rows, (int)gridDim.x);
 }
 
 // Three time steps per launch: the tile carries three halo rows on either
@@ -52,12 +52,12 @@ template <typename T, int S>
 __global__ void __launch_bounds__(256, (sizeof(T) == 4 && S <= 4) ? 2 : 1) k_split_step3(const StepParams<T> p)
 {
     launch_turn();
-    split_tile<T, S, 3>(p, (int)blockIdx.x, (int)gridDim.x);
+    split_tile<T, S, 3>(p, (int)blockIdx.x * p.tile_rows, (int)gridDim.x);
 }
 
 // Batched split step: every CTA takes entry blockIdx.x of the tile list,
-// (instance, tile), stages that instance's parameters in shared memory and
-// computes the tile.  One launch advances every instance of the batch by one
+// (instance, height, first row), stages that instance's parameters in shared
+// memory and computes the tile.  One launch advances every instance of the batch by one
 // step; the instances may differ in every parameter (grid, spin, mode,
 // source, tile height) as long as they share the state precision and the
 // theta segment S.  KS = 2: two time steps per launch, as k_split_step2.
@@ -66,13 +66,10 @@ __global__ void __launch_bounds__(256, (sizeof(T) == 4 && S <= 4) ? 2 : 1)
     k_split_batch(const StepParams<T> *params, const int2 *tiles)
 {
     __shared__ __align__(16) StepParams<T> sp;
-    static_assert(sizeof(StepParams<T>) % 4 == 0 && sizeof(StepParams<T>) <= 4 * 256, "parameter copy");
     launch_turn();
     const int2 e = tiles[blockIdx.x];
-    if (threadIdx.x < sizeof(StepParams<T>) / 4)
-        reinterpret_cast<int *>(&sp)[threadIdx.x] = reinterpret_cast<const int *>(params + e.x)[threadIdx.x];
-    __syncthreads();
-    split_tile<T, S, KS>(sp, e.y, (sp.Nr + sp.tile_rows - 1) / sp.tile_rows);
+    batch_params(sp, params, e);
+    split_tile<T, S, KS, own_samples(sizeof(T), S)>(sp, e.y, sp.ntiles);
 }
 
 // Stored scan plans: the levels scan_plan chooses for every row of the

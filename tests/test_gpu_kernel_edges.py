@@ -1,11 +1,22 @@
 """Edges of the step and adjoint kernels' ranges: the sizes at which a lane,
-tile or ring of samples is partly filled, against identities, independent
-forward differences and the general paths."""
+tile, tile list or ring of samples is partly filled, against the oracle,
+identities, independent forward differences and the general paths."""
+import numpy as np
 import pytest
 
+from paper_0909_4039_gb300 import inputs
 from tests import test_gpu_adjoint as adj
+from tests._common import gpu_stepper, oracle_problem, rel_l2
 
 pytestmark = pytest.mark.gpu
+
+FP64_TOL = 1e-12
+FP32_TOL = 1e-4
+
+
+def _w(Nr, Nth, m=2, r0=8.0):
+    return inputs.Workload("edge", s=-2, m=m, a=0.7, Nr=Nr, Ntheta=Nth, rs_min=-60.0, rs_max=240.0, steps=0, r0=r0,
+                           amp=0.8 - 0.3j, sig_r=0.9, sig_th=0.3, rs_ext=150.0)
 
 
 @pytest.mark.parametrize("Nth", [129, 200, 256, 257, 300])
@@ -17,3 +28,110 @@ def test_adjoint_step_fp64_wide_rows(Nth):
     against recomputed."""
     adj.test_one_step_spin_term_against_step_differences(False, 2, Nth)
     adj.test_tape_step_and_adjoint_equal_recompute(False, 2, Nth, "fp64")
+
+
+@pytest.mark.parametrize("precision,Nth", [("fp64", 127), ("fp64", 129), ("fp64", 200), ("fp64", 257),
+                                            ("fp32", 129), ("fp32", 132), ("fp32", 200), ("fp32", 256)])
+def test_row_segments_against_oracle_and_tile_shapes(precision, Nth):
+    """Row segments that are partly filled (FP64 planes; FP32 packed pairs for
+    128 < Ntheta <= 256 in multiples of 4, and 129 beside them) against the
+    oracle, in tiles that end within the grid; every tile height and number
+    of steps per launch gives the same bits."""
+    from oracle import oracle as O
+    w = _w(310, Nth)
+    u0, n, got = inputs.random_state(w.Nr, Nth, seed=5), 7, []
+    for tr, ks in [(None, None), (1, 1), (5, 2), (6, 3), (9, 1)]:
+        st = gpu_stepper(w, precision, wave_capacity=n + 1)
+        if tr is not None:
+            st.set_tiling(tr, ks)
+        st.set_state(u0, 0)
+        st.step(n)
+        got.append((st.get_state(), st.waveform(0, n + 1)))
+        st.close()
+    uo, ho = O.run(oracle_problem(w), u0, n)
+    tol = FP64_TOL if precision == "fp64" else FP32_TOL
+    assert rel_l2(got[0][0], uo) <= tol and rel_l2(got[0][1], ho) <= tol
+    for u, h in got[1:]:
+        assert np.array_equal(u, got[0][0]) and np.array_equal(h, got[0][1])
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32"])
+@pytest.mark.parametrize("ks", [1, 2, 3])
+def test_samples_of_long_calls_and_short_rings(precision, ks):
+    """Waveform samples are the same from one call (graph replays, several
+    sampling launches, a remainder), from calls of one to a few steps, and from
+    a ring shorter than the call."""
+    w = _w(90, 24)
+    u0, n = inputs.random_state(w.Nr, 24, seed=9), 331
+    def run(cap, calls):
+        st = gpu_stepper(w, precision, wave_capacity=cap)
+        st.set_tiling(16, ks)
+        st.set_state(u0, 0)
+        for k in calls:
+            st.step(k)
+        h = st.waveform(max(0, n + 1 - cap), min(cap, n + 1), rows=True)
+        u = st.get_state()
+        st.close()
+        return u, np.asarray(h[0]), np.asarray(h[1])
+    one, many, short = run(n + 1, [n]), run(n + 1, [1, 129, 2, 3, 4] * 2 + [53]), run(50, [n])
+    # (noise on this coarse grid grows past FP32's range in some rows of the state)
+    assert np.isfinite(one[1]).all() and np.isfinite(one[2]).all()
+    assert all(np.array_equal(a, b, equal_nan=True) for a, b in zip(one, many))
+    assert np.array_equal(short[0], one[0], equal_nan=True)
+    assert np.array_equal(short[1], one[1][-50:]) and np.array_equal(short[2], one[2][-50:])
+
+
+@pytest.mark.parametrize("precision,Nr,Nth,tr", [("fp32", 4000, 100, 12), ("fp32", 4000, 128, 12), ("fp32", 2000, 200, 12),
+                                                 ("fp64", 4500, 64, 28)])
+def test_batch_of_many_tiles_ends_in_half_tiles(precision, Nr, Nth, tr):
+    """A batch of more than two waves of tiles takes its last rows in tiles of
+    half the height: more tiles than rows / height, the same bits as alone."""
+    from paper_0909_4039_gb300 import teuk
+    ws = [_w(Nr, Nth, m, r0) for m, r0 in ((2, 8.0), (1, 60.0))]
+    u0, n, alone = [inputs.random_state(Nr, Nth, seed=20 + k) for k in range(2)], 5, []
+    for w, u in zip(ws, u0):
+        st = gpu_stepper(w, precision, wave_capacity=n + 1)
+        st.set_state(u, 0)
+        st.step(n)
+        alone.append((st.get_state(), st.waveform(0, n + 1)))
+        st.close()
+    sts = [gpu_stepper(w, precision, wave_capacity=n + 1) for w in ws]
+    b = teuk.Batch(sts)
+    b.set_tiling([tr, tr])
+    assert b.tiling()["total_tiles"] > 2 * -(-Nr // tr)
+    for st, u in zip(sts, u0):
+        st.set_state(u, 0)
+    b.step(n)
+    b.synchronize()
+    for st, (u, h) in zip(sts, alone):
+        assert np.array_equal(st.get_state(), u) and np.array_equal(st.waveform(0, n + 1), h)
+    b.close()
+    for st in sts:
+        st.close()
+
+
+@pytest.mark.parametrize("precision,ks", [("fp64", 1), ("fp32", 3)])
+def test_steps_under_stream_capture(precision, ks):
+    """Steps captured into the caller's graph (dependent launches become graph
+    edges) and replayed once give the state and samples of plain steps."""
+    import torch
+    w = _w(200, 32)
+    u0, n = inputs.random_state(w.Nr, 32, seed=3), 7
+    res = []
+    for captured in (False, True):
+        st = gpu_stepper(w, precision, wave_capacity=n + 1)
+        st.set_tiling(16, ks)
+        st.set_state(u0, 0)
+        st.synchronize()
+        if captured:
+            g = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(g, stream=st.stream):
+                st.step(n)
+            with torch.cuda.stream(st.stream):
+                g.replay()
+        else:
+            st.step(n)
+        st.synchronize()
+        res.append((st.get_state(), st.waveform(0, n + 1)))
+        st.close()
+    assert np.array_equal(res[0][0], res[1][0]) and np.array_equal(res[0][1], res[1][1])

@@ -53,4 +53,13 @@ __device__ __forceinline__ void src_da(const T *f, const T *df, T sg, T dsg, T g
 // order (teuk_adjoint.cu).
 cudaError_t launch_part_reduce(const double *part, int nblk, double *acc, cudaStream_t st);
 
+// Shared memory of a kernel that solves one row (physical_row, k_seed).
+template <typename T>
+static inline size_t sample_smem_bytes(int Nth)
+{
+    const size_t row = (size_t)((Nth + 1) & ~1);
+    return 2 * row * sizeof(typename V2<T>::t) + ((size_t)NSF + (size_t)NTF * Nth) * sizeof(T) +
+           pair_th_bytes(Nth, (int)sizeof(T));
+}
+
 }  // namespace teuk

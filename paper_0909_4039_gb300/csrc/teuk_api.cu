@@ -20,6 +20,7 @@ using namespace teuk;
 namespace {
 
 constexpr int kGraphChunk = 64;          // steps per captured graph (even)
+constexpr int kOwnSteps = 4;             // calls of so few steps sample in the tile (own_samples)
 constexpr size_t kStagingElems = 1u << 20;  // complex doubles in the staging area
 
 thread_local char g_init_err[512] = "";
@@ -59,6 +60,7 @@ struct teuk_ctx {
     size_t one_smem;
     int persist, nc, grid;
     int pipe;                // the pipelined two-step kernel (grid persistent CTAs)
+    int own;                 // tiles sample their own steps (a call of a few steps)
     size_t persist_smem;
     int ks;                  // time steps per launch of the tiled kernel (1, 2 or 3)
     int wait0;               // teuk_set_wait_limit (< 0: default bound)
@@ -506,6 +508,7 @@ StepParams<T> make_params(const teuk_ctx *c, int in_level)
     p.thtab = (const T *)(c->coef + c->L.thT);
     p.patch = (const c2 *)(c->coef + c->L.patch);
     p.nfix = -1;
+    p.own = c->own;
     p.h_out = nullptr;
     p.tape = nullptr;
     p.patchu = (const c2 *)(c->coef + c->L.patchu);
@@ -949,6 +952,8 @@ int teuk_step(teuk_ctx *c, int64_t nsteps, void *stream)
     cudaStream_t st = (cudaStream_t)stream;
     int64_t left = nsteps;
     int pending = 0;   // steps whose extraction rows wait for a sampling launch
+    const bool split = c->d.scheme == TEUK_SCHEME_SPLIT;
+    c->own = nsteps <= kOwnSteps && own_samples(c->d.precision == TEUK_FP32 ? 4 : 8, implicit_seg((int)c->d.Ntheta));
     if (left > 0 && c->d.scheme == TEUK_SCHEME_SPLIT && !c->shifted) {
         // first step from a physical state: s_{n+1} = LW C_{dt/2} u_n
         CK(launch_one(c, c->cur, st), "first step launch");
@@ -957,11 +962,10 @@ int teuk_step(teuk_ctx *c, int64_t nsteps, void *stream)
         left -= 1;
         pending = 1;
     }
-    const bool split = c->d.scheme == TEUK_SCHEME_SPLIT;
     // the pipelined and persistent kernels sample their own steps: what is left
     // from before them comes first
     auto flush = [&]() -> cudaError_t {
-        if (!split || pending == 0) return cudaSuccess;
+        if (!split || c->own || pending == 0) return cudaSuccess;
         const int n = pending;
         pending = 0;
         return sample_steps(c, n, st);
@@ -1717,10 +1721,7 @@ int batch_rpp(int N) { return 256 / implicit_group(N); }
 size_t batch_tile_smem(int prec, int tr, int N, int ks)
 {
     if (ks == 2) {
-        // (own samples: the copy of the extraction row)
-        if (prec == TEUK_FP32)
-            return split2_smem_bytes<float>(tr, N) + (own_samples(4, implicit_seg(N)) ? 2 * (size_t)N * sizeof(float2) : 0);
-        return split2_smem_bytes<double>(tr, N);
+        return prec == TEUK_FP32 ? split2_smem_bytes<float>(tr, N) : split2_smem_bytes<double>(tr, N);
     }
     return prec == TEUK_FP32 ? split_smem_bytes<float>(tr, N) : split_smem_bytes<double>(tr, N);
 }

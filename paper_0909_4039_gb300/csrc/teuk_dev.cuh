@@ -607,7 +607,7 @@ template <typename T>
 __device__ __forceinline__ T imp_sg(const ImpRow<T> &r, T s2) { return rcp_fast(fma(-r.AD, s2, r.R2)); }
 // The coefficients of one element from sg = 1/Sigma^2, cos theta, the
 // angular row (am, a0, ap) and the pivot e.  The materialised planes of the
-// FP64 path (k_mat_coef) are made by this same function.
+// FP64 path (k_step_planes) are made by this same function.
 template <typename T>
 __device__ __forceinline__ void imp_elem(const ImpConst<T> &K, const ImpRow<T> &r, T sg, T cc, T am, T a0, T ap,
                                          typename V2<T>::t e, typename V2<T>::t &ct, typename V2<T>::t &dg, T &qam,
@@ -1228,7 +1228,7 @@ static_assert(RF_R < 12 && RF_R2 < 12 && RF_AD < 12 && RF_CTR < 12 && RF_CTI < 1
 // cost about 8 % of a step when taken in every tile.
 // beta = c_p b and kap = c_p K of the Lax-Wendroff stages at the position
 // of step-table entry f and theta (sin^2 = S2, cos = C).  The materialised
-// planes of the FP64 path (k_mat_coef) are made by this same function.
+// planes of the FP64 path (k_step_planes) are made by this same function.
 template <typename T>
 __device__ __forceinline__ void lw_coef(const T *f, T S2, T C, T &beta, typename V2<T>::t &kap, T *sg_out = nullptr)
 {
@@ -1636,9 +1636,11 @@ __device__ void extract_warp(const StepParams<T> &p, const typename V2<T>::t *ro
 
 // Programmatic dependent launches (launch_dep): a kernel waits for all that the
 // stream holds before it, then lets the next launch's CTAs take the SMs its own
-// CTAs leave.  Nothing is read or written before the wait, so the order of
-// memory on the stream is that of plain launches; what it spares is the gap
-// between two launches, in which the next one's CTAs are set up.
+// CTAs leave.  Nothing that a kernel writes is read, and nothing written, before
+// the wait, so the order of memory on the stream is that of plain launches; what
+// it spares is the gap between two launches, in which the next one's CTAs are
+// set up.  (Batches read their tile list and parameters before it: those come by
+// copies, which a later launch on the stream never overtakes.)
 __device__ __forceinline__ void launch_turn()
 {
     asm volatile("griddepcontrol.wait;" ::: "memory");

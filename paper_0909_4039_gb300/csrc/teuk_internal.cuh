@@ -170,6 +170,7 @@ template <typename T> struct StepParams {
     int Nr, Nth;
     int tile_rows;           // output rows per CTA (split kernel)
     int ntiles;              // batches: tiles of the instance
+    int own;                 // the tiles sample their own steps (own_samples)
     int pitch;               // shared-memory row pitch in complex elements
     int group;               // threads per theta row in the implicit phase
     int first;               // 1: implicit step dt/2 (input is a physical state)
@@ -224,18 +225,26 @@ constexpr double kPi = 3.14159265358979323846264338327950;
 
 // Lane segments of the implicit row solves.
 constexpr int kSegNarrow = 4;           // theta elements per thread (Ntheta <= 128)
-// Whether a batch's tiles sample their own steps: FP32 rows of up to 128 theta
-// points (seg: the segment).  Two CTAs share an SM there and hundreds of tiles
-// are left to run while one warp solves a row; leaving the rows to a sampling
-// launch took 1.6 % longer (16 uneven instances, 130 steps: 15.64 against
-// 15.39 ms).  A lone state's launch, of few tiles, ends with that warp.
-constexpr bool own_samples(size_t real_bytes, int seg) { return real_bytes == 4 && seg == kSegNarrow; }
 // A batch's tile list: entry (instance | height << kTileShift, first row).
 constexpr int kTileShift = 23;
 constexpr int kSeg = 8;                 // theta elements per thread (Ntheta <= 256)
 constexpr int kSegWide = 32;            // theta elements per thread (Ntheta <= 1024)
 // theta elements per thread of the implicit row solves
 __host__ __device__ inline int implicit_seg(int Nth) { return Nth <= 128 ? kSegNarrow : (Nth <= 256 ? kSeg : kSegWide); }
+// Whether the split kernels' tiles can sample their own steps: FP32 rows of up
+// to 128 theta points (seg: the segment).  A batch's tiles do: two CTAs share an
+// SM there, and the others run while one warp solves the extraction row; leaving
+// the rows to a sampling launch took 1.6 % longer for 16 uneven instances (130
+// steps: 15.64 against 15.39 ms).  A lone state's do in calls of a few steps, to
+// which a sampling launch adds 5 us (16384 x 128, three steps a call, L2 flushed:
+// 71.3 against 75.9 Gpts/s); in long calls the launch is the faster way (200
+// steps: 4.99 against 5.23 ms; 1024 x 32, 100 steps: 0.44 against 0.76 in the tile).
+constexpr bool own_samples(size_t real_bytes, int seg) { return real_bytes == 4 && seg == kSegNarrow; }
+// shared memory of the extraction row's copy in a launch of two or three steps
+inline size_t own_copy_bytes(int Nth, size_t real_bytes)
+{
+    return own_samples(real_bytes, implicit_seg(Nth)) ? 4 * (size_t)Nth * real_bytes : 0;
+}
 // threads per theta row (a power of two, at most a warp)
 __host__ __device__ inline int implicit_group(int Nth)
 {

@@ -463,9 +463,9 @@ template <int KS>
 __global__ void __launch_bounds__(256, 1) k_pair_batch(const StepParams<float> *params, const int2 *tiles)
 {
     __shared__ __align__(16) StepParams<float> sp;
-    launch_turn();
     const int2 e = tiles[blockIdx.x];
     batch_params(sp, params, e);
+    launch_turn();
     pair_tile<KS>(sp, e.y, sp.ntiles);
 }
 

@@ -13,9 +13,9 @@
 //      S = T - (M - D) d_{r*} u, one thread per theta column marching down
 //      the tile with a register window (this part has no theta coupling)
 //   D. implicit half step on the TR output rows
-//   E. store; the CTA holding the extraction node writes h_{n+1} (FP64 sum)
-//      and the raw row into the ring buffer; the last CTA advances the
-//      device step counter.
+//   E. store; the CTA holding the extraction node leaves that row for the
+//      sampling launch (or samples it itself, see own_samples); the last CTA
+//      to read the device step counter advances it.
 // The halo rows are recomputed by both neighbouring CTAs (B is row-local),
 // so one step reads and writes the state exactly once.
 //
@@ -31,28 +31,28 @@
 namespace teuk {
 namespace {
 
-template <typename T, int S>
+template <typename T, int S, bool OWN = false>
 __global__ void __launch_bounds__(256, (sizeof(T) == 4 && S <= 4) ? 2 : 1) k_split_step(const StepParams<T> p)
 {
     launch_turn();
-    split_tile<T, S, 1>(p, (int)blockIdx.x * p.tile_rows, (int)gridDim.x);
+    split_tile<T, S, 1, OWN>(p, (int)blockIdx.x * p.tile_rows, (int)gridDim.x);
 }
 
 // Two time steps per launch (temporal blocking): see split_tile.
-template <typename T, int S>
+template <typename T, int S, bool OWN = false>
 __global__ void __launch_bounds__(256, (sizeof(T) == 4 && S <= 4) ? 2 : 1) k_split_step2(const StepParams<T> p)
 {
     launch_turn();
-    split_tile<T, S, 2>(p, (int)blockIdx.x * p.tile_rows, (int)gridDim.x);
+    split_tile<T, S, 2, OWN>(p, (int)blockIdx.x * p.tile_rows, (int)gridDim.x);
 }
 
 // Three time steps per launch: the tile carries three halo rows on either
 // side, and the state moves once per three steps.
-template <typename T, int S>
+template <typename T, int S, bool OWN = false>
 __global__ void __launch_bounds__(256, (sizeof(T) == 4 && S <= 4) ? 2 : 1) k_split_step3(const StepParams<T> p)
 {
     launch_turn();
-    split_tile<T, S, 3>(p, (int)blockIdx.x * p.tile_rows, (int)gridDim.x);
+    split_tile<T, S, 3, OWN>(p, (int)blockIdx.x * p.tile_rows, (int)gridDim.x);
 }
 
 // Batched split step: every CTA takes entry blockIdx.x of the tile list,
@@ -66,9 +66,9 @@ __global__ void __launch_bounds__(256, (sizeof(T) == 4 && S <= 4) ? 2 : 1)
     k_split_batch(const StepParams<T> *params, const int2 *tiles)
 {
     __shared__ __align__(16) StepParams<T> sp;
-    launch_turn();
     const int2 e = tiles[blockIdx.x];
     batch_params(sp, params, e);
+    launch_turn();
     split_tile<T, S, KS, own_samples(sizeof(T), S)>(sp, e.y, sp.ntiles);
 }
 
@@ -559,7 +559,8 @@ size_t split_smem_bytes(int tile_rows, int Nth)
     return sm;
 }
 
-// Two steps per launch: R = TR + 4 rows.
+// Two steps per launch: R = TR + 4 rows (and a copy of the extraction row, for
+// tiles that sample their own steps).
 template <typename T>
 size_t split2_smem_bytes(int tile_rows, int Nth)
 {
@@ -568,7 +569,7 @@ size_t split2_smem_bytes(int tile_rows, int Nth)
         const size_t pm = pair_smem_bytes(tile_rows, Nth, 2), sm = split_smem_bytes<T>(tile_rows, Nth);
         return pm > sm ? pm : sm;
     }
-    return split_smem_plan(tile_rows + 4, Nth, (int)sizeof(T)).total;
+    return split_smem_plan(tile_rows + 4, Nth, (int)sizeof(T)).total + own_copy_bytes(Nth, sizeof(T));
 }
 
 template <typename T>
@@ -600,6 +601,8 @@ cudaError_t launch_split_step(const StepParams<T> &p, int threads, size_t smem, 
     const int seg = implicit_seg(p.Nth);
     const int v = seg == kSegNarrow ? 0 : (seg == kSeg ? 1 : 2);
     auto fn = v == 0 ? k_split_step<T, kSegNarrow> : (v == 1 ? k_split_step<T, kSeg> : k_split_step<T, kSegWide>);
+    if constexpr (own_samples(sizeof(T), kSegNarrow))
+        if (p.own && !p.imp_only && p.nfix < 0) fn = k_split_step<T, kSegNarrow, true>;
     cudaError_t e = smem_limit_max((const void *)fn);
     if (e != cudaSuccess) return e;
     int grid = (p.Nr + p.tile_rows - 1) / p.tile_rows;
@@ -696,6 +699,8 @@ cudaError_t launch_split_step2(const StepParams<T> &p, int threads, size_t smem,
     if constexpr (sizeof(T) == 4)
         if (pair_eligible(p.Nth)) return launch_pair_step(p, 2, st);
     auto fn = split2_fn<T>(p.Nth);
+    if constexpr (own_samples(sizeof(T), kSegNarrow))
+        if (p.own) fn = k_split_step2<T, kSegNarrow, true>;
     cudaError_t e = smem_limit_max((const void *)fn);
     if (e != cudaSuccess) return e;
     int grid = (p.Nr + p.tile_rows - 1) / p.tile_rows;
@@ -718,7 +723,7 @@ size_t split3_smem_bytes(int tile_rows, int Nth)
         const size_t pm = pair_smem_bytes(tile_rows, Nth, 3), sm = split_smem_bytes<T>(tile_rows, Nth);
         return pm > sm ? pm : sm;
     }
-    return split_smem_plan(tile_rows + 6, Nth, (int)sizeof(T)).total;
+    return split_smem_plan(tile_rows + 6, Nth, (int)sizeof(T)).total + own_copy_bytes(Nth, sizeof(T));
 }
 
 template <typename T>
@@ -746,6 +751,8 @@ cudaError_t launch_split_step3(const StepParams<T> &p, int threads, size_t smem,
     if constexpr (sizeof(T) == 4)
         if (pair_eligible(p.Nth)) return launch_pair_step(p, 3, st);
     auto fn = split3_fn<T>(p.Nth);
+    if constexpr (own_samples(sizeof(T), kSegNarrow))
+        if (p.own) fn = k_split_step3<T, kSegNarrow, true>;
     cudaError_t e = smem_limit_max((const void *)fn);
     if (e != cudaSuccess) return e;
     int grid = (p.Nr + p.tile_rows - 1) / p.tile_rows;

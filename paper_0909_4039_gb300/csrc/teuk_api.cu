@@ -1684,6 +1684,12 @@ struct teuk_batch {
     char err[512];
 };
 
+size_t teuk::batch_tile_bytes(int precision, int tile_rows, int Nth, int ks, bool paired)
+{
+    if (!paired) return split_tile_bytes(tile_rows, Nth, ks, precision == TEUK_FP32 ? 4 : 8);
+    return std::max(pair_smem_bytes(tile_rows, Nth, ks), split_tile_bytes(tile_rows, Nth, 1, 4));
+}
+
 namespace {
 
 __attribute__((format(printf, 3, 4))) int bset_err(teuk_batch *b, int code, const char *fmt, ...)
@@ -1722,20 +1728,11 @@ size_t batch_ws_bytes(teuk_ctx *const *ctxs, int count, size_t *par_bytes, size_
 // Rows of one implicit pass for Ntheta (256 threads / G).
 int batch_rpp(int N) { return 256 / implicit_group(N); }
 
-// Shared memory of a batch tile of height tr with ks steps per launch.
-size_t batch_tile_smem(int prec, int tr, int N, int ks)
-{
-    if (ks == 2) {
-        return prec == TEUK_FP32 ? split2_smem_bytes<float>(tr, N) : split2_smem_bytes<double>(tr, N);
-    }
-    return prec == TEUK_FP32 ? split_smem_bytes<float>(tr, N) : split_smem_bytes<double>(tr, N);
-}
-
 // Default tile height: the largest whole number of implicit passes (tile
 // rows plus halos) whose tile leaves room for as many CTAs per SM as the
 // kernel's registers allow: two for FP32 rows of up to 128 theta points,
 // one otherwise (wider segments and FP64 take over 128 registers a thread).
-int batch_default_tr(const teuk_ctx *c, int ks)
+int batch_default_tr(const teuk_ctx *c, int ks, bool paired)
 {
     const int N = (int)c->d.Ntheta, rpp = batch_rpp(N);
     const size_t budget =
@@ -1744,7 +1741,7 @@ int batch_default_tr(const teuk_ctx *c, int ks)
     for (int R = rpp; R - 2 * ks <= 254; R += rpp) {
         const int tr = R - 2 * ks;
         if (tr < 1) continue;
-        if (batch_tile_smem(c->d.precision, tr, N, ks) > budget && best > 1) break;
+        if (batch_tile_bytes(c->d.precision, tr, N, ks, paired) > budget && best > 1) break;
         best = tr;
         if (tr >= c->d.Nr) break;
     }
@@ -1765,7 +1762,7 @@ int batch_layout(teuk_batch *b)
         const teuk_ctx *c = b->c[i];
         whole += (c->d.Nr + b->tr[i] - 1) / b->tr[i];
         const int N = (int)c->d.Ntheta;
-        size_t sm = batch_tile_smem(b->prec, b->tr[i], N, b->ks);
+        size_t sm = batch_tile_bytes(b->prec, b->tr[i], N, b->ks, b->paired);
         smem = sm > smem ? sm : smem;
     }
     if (smem > 227 * 1024) return bset_err(b, TEUK_E_INVAL, "a tile of the batch does not fit in shared memory");
@@ -1995,7 +1992,7 @@ int teuk_batch_create(teuk_ctx *const *ctxs, int count, void *d_ws, size_t ws_by
     for (int k = 0; k < 3; ++k) b->off_par[k] = (size_t)k * b->par_bytes;
     b->ks = split_batch_available(seg, 2) ? 2 : 1;
     b->tr.resize(count);
-    for (int i = 0; i < count; ++i) b->tr[i] = batch_default_tr(ctxs[i], b->ks);
+    for (int i = 0; i < count; ++i) b->tr[i] = batch_default_tr(ctxs[i], b->ks, b->paired);
     r = batch_layout(b);
     if (r != TEUK_OK) {
         memcpy(g_init_err, b->err, sizeof(g_init_err));
@@ -2098,7 +2095,7 @@ int teuk_batch_autotune(teuk_batch *b, int trial_steps, void *stream)
     for (int ks = 1; ks <= 2 && rc == TEUK_OK; ++ks) {
         if (!split_batch_available(b->seg, ks)) continue;
         b->ks = ks;
-        for (size_t i = 0; i < b->c.size(); ++i) b->tr[i] = batch_default_tr(b->c[i], ks);
+        for (size_t i = 0; i < b->c.size(); ++i) b->tr[i] = batch_default_tr(b->c[i], ks, b->paired);
         for (int N : classes) {
             const int rpp = batch_rpp(N);
             std::vector<int> keep = b->tr;

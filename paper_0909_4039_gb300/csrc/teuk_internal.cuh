@@ -284,6 +284,13 @@ __host__ __device__ inline SplitSmem split_smem_plan(int R, int N, int tsize)
     return s;
 }
 
+// Dynamic shared memory of split_tile (k_split_step, 2, 3 and k_split_batch) for
+// a tile of tile_rows output rows and ks steps per launch.
+inline size_t split_tile_bytes(int tile_rows, int Nth, int ks, size_t real_bytes)
+{
+    return split_smem_plan(tile_rows + 2 * ks, Nth, (int)real_bytes).total + (ks > 1 ? own_copy_bytes(Nth, real_bytes) : 0);
+}
+
 // Shared-memory carve-up of the persistent split kernel: theta tables, a
 // copy of the extraction row (state and step-table entry) and two tile
 // buffers, each with the two state planes [R][N], the pivots [R][N] and the
@@ -495,6 +502,12 @@ int split_batch_blocks_per_sm(int seg, size_t smem, int ks);
 template <typename T>
 cudaError_t launch_split_batch(const StepParams<T> *d_params, const int2 *d_tiles, int ntiles, int seg, size_t smem,
                                int ks, cudaStream_t st);
+// Dynamic shared memory of a batch tile with ks steps per launch, by the kernels
+// that run it: k_pair_batch for the full steps of a batch whose every instance
+// is eligible (paired; k_split_batch with one step then takes first steps at the
+// same height), k_split_batch for every other batch, whatever its instances
+// would run alone.
+size_t batch_tile_bytes(int precision, int tile_rows, int Nth, int ks, bool paired);
 inline bool split_batch_available(int seg, int ks) { return ks == 1 || (ks == 2 && seg != kSegWide); }
 
 cudaError_t launch_convert_to(int prec, const double2 *src, void *dst, size_t n, cudaStream_t st);

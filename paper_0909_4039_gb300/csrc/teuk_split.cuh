@@ -551,7 +551,7 @@ cudaError_t launch_step_planes(const StepParams<T> &p, cudaStream_t st)
 template <typename T>
 size_t split_smem_bytes(int tile_rows, int Nth)
 {
-    size_t sm = split_smem_plan(tile_rows + 2, Nth, (int)sizeof(T)).total;
+    size_t sm = split_tile_bytes(tile_rows, Nth, 1, sizeof(T));
     if (sizeof(T) == 4 && pair_eligible(Nth)) {
         const size_t pm = pair_smem_bytes(tile_rows, Nth, 1);
         sm = pm > sm ? pm : sm;
@@ -569,7 +569,7 @@ size_t split2_smem_bytes(int tile_rows, int Nth)
         const size_t pm = pair_smem_bytes(tile_rows, Nth, 2), sm = split_smem_bytes<T>(tile_rows, Nth);
         return pm > sm ? pm : sm;
     }
-    return split_smem_plan(tile_rows + 4, Nth, (int)sizeof(T)).total + own_copy_bytes(Nth, sizeof(T));
+    return split_tile_bytes(tile_rows, Nth, 2, sizeof(T));
 }
 
 template <typename T>
@@ -598,6 +598,7 @@ cudaError_t launch_split_step(const StepParams<T> &p, int threads, size_t smem, 
 {
     if constexpr (sizeof(T) == 4)
         if (!p.first && !p.imp_only && p.nfix < 0 && pair_eligible(p.Nth)) return launch_pair_step(p, 1, st);
+    if (smem < split_tile_bytes(p.tile_rows, p.Nth, 1, sizeof(T))) return cudaErrorInvalidValue;
     const int seg = implicit_seg(p.Nth);
     const int v = seg == kSegNarrow ? 0 : (seg == kSeg ? 1 : 2);
     auto fn = v == 0 ? k_split_step<T, kSegNarrow> : (v == 1 ? k_split_step<T, kSeg> : k_split_step<T, kSegWide>);
@@ -698,6 +699,7 @@ cudaError_t launch_split_step2(const StepParams<T> &p, int threads, size_t smem,
     if (p.first || p.imp_only) return cudaErrorInvalidValue;   // two full steps only
     if constexpr (sizeof(T) == 4)
         if (pair_eligible(p.Nth)) return launch_pair_step(p, 2, st);
+    if (smem < split_tile_bytes(p.tile_rows, p.Nth, 2, sizeof(T))) return cudaErrorInvalidValue;
     auto fn = split2_fn<T>(p.Nth);
     if constexpr (own_samples(sizeof(T), kSegNarrow))
         if (p.own) fn = k_split_step2<T, kSegNarrow, true>;
@@ -723,7 +725,7 @@ size_t split3_smem_bytes(int tile_rows, int Nth)
         const size_t pm = pair_smem_bytes(tile_rows, Nth, 3), sm = split_smem_bytes<T>(tile_rows, Nth);
         return pm > sm ? pm : sm;
     }
-    return split_smem_plan(tile_rows + 6, Nth, (int)sizeof(T)).total + own_copy_bytes(Nth, sizeof(T));
+    return split_tile_bytes(tile_rows, Nth, 3, sizeof(T));
 }
 
 template <typename T>
@@ -750,6 +752,7 @@ cudaError_t launch_split_step3(const StepParams<T> &p, int threads, size_t smem,
     if (p.first || p.imp_only) return cudaErrorInvalidValue;   // three full steps only
     if constexpr (sizeof(T) == 4)
         if (pair_eligible(p.Nth)) return launch_pair_step(p, 3, st);
+    if (smem < split_tile_bytes(p.tile_rows, p.Nth, 3, sizeof(T))) return cudaErrorInvalidValue;
     auto fn = split3_fn<T>(p.Nth);
     if constexpr (own_samples(sizeof(T), kSegNarrow))
         if (p.own) fn = k_split_step3<T, kSegNarrow, true>;

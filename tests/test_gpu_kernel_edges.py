@@ -135,3 +135,37 @@ def test_steps_under_stream_capture(precision, ks):
         res.append((st.get_state(), st.waveform(0, n + 1)))
         st.close()
     assert np.array_equal(res[0][0], res[1][0]) and np.array_equal(res[0][1], res[1][1])
+
+
+@pytest.mark.parametrize("widths", [(256, 250), (255, 252), (256, 129)])
+def test_fp32_batch_of_packed_and_scalar_widths(widths):
+    """FP32 rows of 129 to 256 points run on packed pairs alone where Ntheta is
+    a multiple of 4 and in the scalar kernel otherwise; a batch that mixes the
+    two runs the scalar kernel for all of them.  At the default heights, at low
+    ones and with one step a launch, each instance gets its solo run's bits."""
+    from oracle import oracle as O
+    from paper_0909_4039_gb300 import teuk
+    ws = [_w(310 + 7 * k, Nth, 2 - k, 8.0 + k) for k, Nth in enumerate(widths)]
+    u0, n, alone = [inputs.random_state(w.Nr, w.Ntheta, seed=40 + k) for k, w in enumerate(ws)], 6, []
+    for w, u in zip(ws, u0):
+        st = gpu_stepper(w, "fp32", wave_capacity=n + 1)
+        st.set_state(u, 0)
+        st.step(n)
+        alone.append((st.get_state(), st.waveform(0, n + 1)))
+        st.close()
+        uo, ho = O.run(oracle_problem(w), u, n)
+        assert rel_l2(alone[-1][0], uo) <= FP32_TOL and rel_l2(alone[-1][1], ho) <= FP32_TOL
+    sts = [gpu_stepper(w, "fp32", wave_capacity=n + 1) for w in ws]
+    b = teuk.Batch(sts)
+    for heights, ks in ((None, None), ([4, 4], 2), ([1, 12], 2), ([6, 3], 1)):
+        if heights:
+            b.set_tiling(heights, ks)
+        for st, u in zip(sts, u0):
+            st.set_state(u, 0)
+        b.step(n)
+        b.synchronize()
+        for st, (u, h) in zip(sts, alone):
+            assert np.array_equal(st.get_state(), u) and np.array_equal(st.waveform(0, n + 1), h)
+    b.close()
+    for st in sts:
+        st.close()

@@ -60,6 +60,10 @@ __global__ void __launch_bounds__(32) k_sample(const StepParams<T> p, const type
 // Threads of a sampling CTA: one warp has the row to solve, and four load its
 // tables (7 Ntheta entries one after the other held a lone warp for 10 of the
 // 22 us that a launch of 64 x 16 rows of 128 took).
+// (One CTA per SM is asked for: without that, the compiler gave the kernels of 32
+// elements a lane 32 registers and spilled the row; 1500 x 300 in calls of one
+// step, us per call with and without: FP64 410 and 540, four FP32 instances 237
+// and 287.)
 constexpr int kSampleThreads = 128;
 
 // CTA (b, instance): the b-th step after ctl->sampled, if it has been taken.
@@ -86,14 +90,14 @@ __device__ __forceinline__ void sample_step(const StepParams<T> &p)
 }
 
 template <typename T, int S>
-__global__ void __launch_bounds__(kSampleThreads) k_sample_steps(const StepParams<T> p)
+__global__ void __launch_bounds__(kSampleThreads, 1) k_sample_steps(const StepParams<T> p)
 {
     launch_turn();
     sample_step<T, S>(p);
 }
 
 template <typename T, int S>
-__global__ void __launch_bounds__(kSampleThreads) k_sample_steps_batch(const StepParams<T> *params)
+__global__ void __launch_bounds__(kSampleThreads, 1) k_sample_steps_batch(const StepParams<T> *params)
 {
     launch_turn();
     __shared__ __align__(16) StepParams<T> sp;

@@ -473,7 +473,9 @@ __device__ __forceinline__ void row_store(typename V2<T>::t *phi, typename V2<T>
                                           int lenw, bool vec)
 {
     if (lenw <= 0) return;
-    if (vec && lenw == S) {
+    // (whole segments, but for FP32 rows of 128 < Ntheta <= 256, where vec asks for
+    // multiples of 4 only; the test of it took 0.3 % of a batch of narrow rows)
+    if (vec && (sizeof(T) == 8 || S != kSeg || lenw == S)) {
         vstore<S>(phi + j0, w);
         vstore<S>(pi + j0, y);
     } else {
@@ -1634,6 +1636,16 @@ __device__ void extract_warp(const StepParams<T> &p, const typename V2<T>::t *ro
     for (int j = lane; j < N; j += 32) dst[1 + j] = make_double2((double)row[j].x, (double)row[j].y);
 }
 
+// Source phase q of a launch from step n: of Eq. 13 (even q) or 14 (odd) of its
+// step q / 2, times the stage's length dt/2 or dt.  An FP64 sincos takes about
+// 3 us of one warp.
+__device__ __noinline__ void tile_phase(double2 *sph, long long n, double dt, double mOmega, int q)
+{
+    const double t = (double)(n + (q >> 1)) * dt, len = (q & 1) ? dt : 0.5 * dt;
+    const double2 e = phase_at(mOmega, (q & 1) ? t + 0.5 * dt : t);
+    sph[q] = make_double2(len * e.x, len * e.y);
+}
+
 // Programmatic dependent launches (launch_dep): a kernel waits for all that the
 // stream holds before it, then lets the next launch's CTAs take the SMs its own
 // CTAs leave.  Nothing that a kernel writes is read, and nothing written, before
@@ -1673,7 +1685,8 @@ __device__ __forceinline__ void batch_params(StepParams<T> &sp, const StepParams
 // k + 1 .. R - 2 - k, so the last one updates the TR output rows; the state
 // read and written per step falls to 1/KS at the cost of recomputing the
 // extra halo rows.  The result is bitwise that of KS single steps.
-template <typename T, int S, int KS, bool OWN = false>
+// BATCH: a tile of a batch (k_split_batch).
+template <typename T, int S, int KS, bool OWN = false, bool BATCH = false>
 __device__ __forceinline__ void split_tile(const StepParams<T> &p, int i0, int ntiles)
 {
     typedef typename V2<T>::t c2;
@@ -1713,35 +1726,23 @@ __device__ __forceinline__ void split_tile(const StepParams<T> &p, int i0, int n
             }
         }
     }
-    // The last warp reads the step index while thread 0 starts the copies.
-    if (tid >= NT - 32) {
-        const int q = tid - (NT - 32);
+    // One thread reads the step index and counts the tile in: of the last warp,
+    // while thread 0 starts the copies, or in a batch of narrow FP32 rows thread 0
+    // before them (64 uneven instances, 64 steps: 31.14 against 31.37 ms; lone
+    // 1024 x 32 FP32 with thread 0 4.0 us a step against 3.8, 3001 x 90 8.2 against 8.0).
+    if (tid == (BATCH && own_samples(sizeof(T), S) ? 0 : NT - 32)) {
         const long long n = p.nfix >= 0 ? p.nfix : *((volatile long long *)&p.ctl->step);
-        __syncwarp();
-        if (q == 0) {
-            s_n = n;
-            if (!p.imp_only && p.nfix < 0) {
-                // The last CTA to read the step index advances it.  Later kernels
-                // on the stream see the new value; no CTA of this launch reads it
-                // again, so no CTA has to wait for its own stores first.
-                __threadfence();
-                unsigned t = atomicAdd(&p.ctl->ticket, 1u);
-                if (t == (unsigned)ntiles - 1u) {
-                    p.ctl->ticket = 0u;
-                    p.ctl->step = n + KS;
-                }
+        s_n = n;
+        if (!p.imp_only && p.nfix < 0) {
+            // The last CTA to read the step index advances it.  Later kernels
+            // on the stream see the new value; no CTA of this launch reads it
+            // again, so no CTA has to wait for its own stores first.
+            __threadfence();
+            unsigned t = atomicAdd(&p.ctl->ticket, 1u);
+            if (t == (unsigned)ntiles - 1u) {
+                p.ctl->ticket = 0u;
+                p.ctl->step = n + KS;
             }
-        }
-        // Source phases of Eqs. 13 and 14 times their stage lengths dt/2 and dt,
-        // one lane each.  An FP64 sincos takes about 3 us of one warp; taken one
-        // after the other by the thread that starts the tile's copies, the 2 KS
-        // of them held a source tile, and with it the launch, for 6 us a step.
-        // (Done here and not after the tables' barrier: with the row solve's
-        // registers live there, the batch's tiles took 1 % longer.)
-        if (src && q < 2 * KS) {
-            const double t = (double)(n + (q >> 1)) * p.dt64, len = (q & 1) ? p.dt64 : 0.5 * p.dt64;
-            const double2 e = phase_at(p.mOmega, (q & 1) ? t + 0.5 * p.dt64 : t);
-            sph[q] = make_double2(len * e.x, len * e.y);
         }
     }
     // ---- A: tile rows g0 .. g0+R-1 (state), r and theta tables; the row
@@ -1825,6 +1826,14 @@ __device__ __forceinline__ void split_tile(const StepParams<T> &p, int i0, int n
         s_plan[lr] = (gi >= 0 && gi < Nr) ? K.plan[gi] : 0;
     }
     __syncthreads();
+    // Source phases, one lane of the last warp each, while the other warps start on
+    // the row solves (a barrier ends those): one after the other by the thread that
+    // starts the copies, the 2 KS of them held a source tile, and with it the
+    // launch, for 6 us a step.  Inlined, or taken before the tables' barrier with
+    // the step index in every lane, they cost the whole kernel registers: 64 uneven
+    // FP32 instances 31.67 against 31.14 ms (64 steps), 16384 x 300 FP32 338 against
+    // 334 us a step, 1024 x 32 FP64 17.7 against 17.4.
+    if (src && tid >= NT - 32 && tid - (NT - 32) < 2 * KS) tile_phase(sph, s_n, p.dt64, p.mOmega, tid - (NT - 32));
     const int g = tid & (G - 1), tq = tid >> lgG;   // lane in the row group, row of the pass
     const int wq = (tid & ~31) >> lgG;              // first row of the warp's in the pass
     const bool vec = p.vec != 0;
@@ -1845,8 +1854,10 @@ __device__ __forceinline__ void split_tile(const StepParams<T> &p, int i0, int n
             // FP64 a warp occupies its scheduler's FP64 pipe for 64 cycles per
             // instruction whatever its lanes hold, so the empty rows of a
             // short tile's pass cost as much as its real ones: 1024 x 32 FP64
-            // 60 -> 35 us per step, 96 x 16 64 -> 39.
-            if (base + wq >= hi) continue;
+            // 60 -> 35 us per step, 96 x 16 64 -> 39.  (FP32 rows of more than 256
+            // points spill: 1500 x 300 52 -> 42.  Narrower FP32 rows lost 0.4 % of a
+            // batch's time to the branch.)
+            if ((sizeof(T) == 8 || S == kSegWide) && base + wq >= hi) continue;
             int lr = base + tq;
             bool in_tile = lr < hi;
             int gi = g0 + lr;

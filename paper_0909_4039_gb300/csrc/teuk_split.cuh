@@ -69,7 +69,7 @@ __global__ void __launch_bounds__(256, (sizeof(T) == 4 && S <= 4) ? 2 : 1)
     const int2 e = tiles[blockIdx.x];
     batch_params(sp, params, e);
     launch_turn();
-    split_tile<T, S, KS, own_samples(sizeof(T), S)>(sp, e.y, sp.ntiles);
+    split_tile<T, S, KS, own_samples(sizeof(T), S), true>(sp, e.y, sp.ntiles);
 }
 
 // Stored scan plans: the levels scan_plan chooses for every row of the

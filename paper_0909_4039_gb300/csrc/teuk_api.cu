@@ -241,7 +241,10 @@ double host_atheta_bound(const teuk_grid_desc &d)
 //   share its pipes, so their counts add up.  (Model against measurement:
 //   16384 x 128, 36 rows, two steps 349 / 365 us; 1024 x 32, 7 rows, three
 //   steps 14 / 17.)
-//   FP32: 0.6 Rpad + 0.4 R row-times a step (Rpad: whole warps of rows), one
+//   FP32: 0.6 Rpad + 0.4 R row-times a step (Rpad: whole warps of rows; whole
+//   passes of the eight warps for Ntheta > 256, whose spilled rows leave an SM's
+//   warps nothing to gain from fewer of them: 16384 x 300, two steps, 27 rows
+//   325 us a step, 36 rows 335, which whole warps rank the other way), one
 //   row-time 0.188 us for 128 theta points, shared by the k CTAs of an SM,
 //   20 % more for k = 1 (no second CTA to overlap latency with), and 5 us a
 //   launch.  (16384 x 128, 28 rows, two steps 26 / 25 us; 65536 x 256, 36
@@ -297,10 +300,11 @@ static bool tiled_cand(const teuk_ctx *c, int TR, int ks, int nsm, TileCand *out
     auto up = [](int a, int b) { return (a + b - 1) / b; };
     double cost = 0.0;   // us per launch
     if (f32) {
+        const int rpad = S == kSegWide ? threads / implicit_group(N) : rpw;
         double rows = 0.0;
         for (int q = 0; q < ks; ++q) {
             const int ri = TR + 2 * (ks - q);
-            rows += 0.6 * up(ri, rpw) * rpw + 0.4 * (ri - 2);
+            rows += 0.6 * up(ri, rpad) * rpad + 0.4 * (ri - 2);
         }
         const long long co = per < k ? per : k;   // CTAs that share an SM
         cost = 5.0 + waves * co * rows * row_time(N) * (co == 1 ? 1.2 : 1.0);

@@ -584,6 +584,16 @@ cudaError_t launch_one(teuk_ctx *c, int in_level, cudaStream_t st)
     return c->d.scheme == TEUK_SCHEME_SPLIT ? launch_split<double>(c, p, st) : launch_literal_step<double>(p, st);
 }
 
+// The last two steps of a call with three steps per launch, in one launch at the
+// same tile height (16384 x 128 FP32, two steps a call: 53 us against 64 in two
+// launches).
+cudaError_t launch_two(teuk_ctx *c, int in_level, cudaStream_t st)
+{
+    if (c->d.precision == TEUK_FP32)
+        return launch_split_step2<float>(make_params<float>(c, in_level), c->threads, c->smem2, st);
+    return launch_split_step2<double>(make_params<double>(c, in_level), c->threads, c->smem2, st);
+}
+
 // One launch of the configured kernel from level in_level: two or three
 // steps when the tiled kernel takes that many per launch and the state is
 // shifted (full steps follow), else one; *steps receives the count.
@@ -1025,6 +1035,9 @@ int teuk_step(teuk_ctx *c, int64_t nsteps, void *stream)
         if (pending + ks > kRawSlots) CK(flush(), "samples");
         if (left >= ks) {
             CK(launch_unit(c, c->cur, st, &k), "step launch");
+        } else if (ks == 3 && left == 2) {
+            k = 2;
+            CK(launch_two(c, c->cur, st), "step launch");
         } else {
             CK(launch_one(c, c->cur, st), "step launch");
         }

@@ -107,6 +107,8 @@ Layout make_layout(const teuk_grid_desc &d)
     if (!f32 && d.scheme == TEUK_SCHEME_SPLIT) off = align256(off + c2 * 2 * N * patch_rows);
     L.w = off; off = align256(off + sizeof(double) * N);
     L.seed = off; off = align256(off + 2 * sizeof(double2) * N);
+    L.th2 = off;
+    if (f32 && implicit_seg((int)N) == kSeg) off = align256(off + sizeof(unsigned long long) * kPairTh * 128);
     L.ctl = off; off = align256(off + sizeof(Ctl));
     L.raw = off; off = align256(off + c2 * 2 * N * (size_t)kRawSlots);
     L.staging_elems = 0;
@@ -290,9 +292,9 @@ static bool tiled_cand(const teuk_ctx *c, int TR, int ks, int nsm, TileCand *out
     else sm = f32 ? split3_smem_bytes<float>(TR, N) : split3_smem_bytes<double>(TR, N);
     if (sm > 227 * 1024) return false;
     int k;
-    if (ks == 1) k = f32 ? split_blocks_per_sm<float>(N, threads, sm) : split_blocks_per_sm<double>(N, threads, sm);
-    else if (ks == 2) k = f32 ? split2_blocks_per_sm<float>(N, threads, sm) : split2_blocks_per_sm<double>(N, threads, sm);
-    else k = f32 ? split3_blocks_per_sm<float>(N, threads, sm) : split3_blocks_per_sm<double>(N, threads, sm);
+    if (ks == 1) k = f32 ? split_blocks_per_sm<float>(TR, N, threads, sm) : split_blocks_per_sm<double>(TR, N, threads, sm);
+    else if (ks == 2) k = f32 ? split2_blocks_per_sm<float>(TR, N, threads, sm) : split2_blocks_per_sm<double>(TR, N, threads, sm);
+    else k = f32 ? split3_blocks_per_sm<float>(TR, N, threads, sm) : split3_blocks_per_sm<double>(TR, N, threads, sm);
     if (k < 1) return false;
     const long long Nr = c->d.Nr;
     const long long tiles = (Nr + TR - 1) / TR, per = (tiles + nsm - 1) / nsm, waves = (per + k - 1) / k;
@@ -515,6 +517,7 @@ StepParams<T> make_params(const teuk_ctx *c, int in_level)
         p.mat.lw = (const c2 *)(m + ((kStepPlaneReals * t + 255) & ~(size_t)255));
     }
     p.thtab = (const T *)(c->coef + c->L.thT);
+    p.th2 = (const unsigned long long *)(c->coef + c->L.th2);
     p.patch = (const c2 *)(c->coef + c->L.patch);
     p.nfix = -1;
     p.own = c->own;
@@ -1687,7 +1690,7 @@ struct teuk_batch {
     std::vector<int> tr;             // tile height per instance
     std::vector<int> nt;             // tiles per instance
     int prec, seg;
-    bool paired;                     // every instance takes the FP32 kernels on packed pairs
+    bool paired;                     // the FP32 kernels on packed pairs take the full steps of every instance
     char *ws;                        // caller-owned device workspace
     size_t ws_bytes, par_bytes;      // par_bytes: one parameter table
     size_t off_par[3], off_tiles;    // tables: in = cur, in = cur ^ 1, first step; tile list
@@ -1745,6 +1748,14 @@ size_t batch_ws_bytes(teuk_ctx *const *ctxs, int count, size_t *par_bytes, size_
 // Rows of one implicit pass for Ntheta (256 threads / G).
 int batch_rpp(int N) { return 256 / implicit_group(N); }
 
+// Whether every instance's width has a pair kernel.
+bool batch_pairs(const teuk_batch *b)
+{
+    bool all = b->prec == TEUK_FP32;
+    for (const teuk_ctx *c : b->c) all = all && pair_eligible((int)c->d.Ntheta);
+    return all;
+}
+
 // Default tile height: the largest whole number of implicit passes (tile
 // rows plus halos) whose tile leaves room for as many CTAs per SM as the
 // kernel's registers allow: two for FP32 rows of up to 128 theta points,
@@ -1765,6 +1776,14 @@ int batch_default_tr(const teuk_ctx *c, int ks, bool paired)
     return best;
 }
 
+// Half of instance i's tile height: half of the tile's row-solve passes, if it has two.
+int batch_half(const teuk_batch *b, int i)
+{
+    const int rpp = batch_rpp((int)b->c[i]->d.Ntheta);
+    const int h = ((b->tr[i] + 2 * b->ks) / 2 + rpp - 1) / rpp * rpp - 2 * b->ks;
+    return h >= 1 && h < b->tr[i] ? h : b->tr[i];
+}
+
 // Tile list (instances interleaved tile by tile) and shared memory for the
 // current tile heights; drops the captured graph.
 int batch_layout(teuk_batch *b)
@@ -1773,14 +1792,15 @@ int batch_layout(teuk_batch *b)
     if (b->graph) cudaGraphExecDestroy(b->graph);
     b->graph = nullptr;
     b->graph_stream = nullptr;
+    b->paired = b->prec == TEUK_FP32;
+    for (int i = 0; i < n; ++i) b->paired = b->paired && pair_runs(b->tr[i], (int)b->c[i]->d.Ntheta, b->ks);
     size_t smem = 0;
     long long whole = 0;   // tiles of full height
     for (int i = 0; i < n; ++i) {
         const teuk_ctx *c = b->c[i];
         whole += (c->d.Nr + b->tr[i] - 1) / b->tr[i];
         const int N = (int)c->d.Ntheta;
-        size_t sm = batch_tile_bytes(b->prec, b->tr[i], N, b->ks, b->paired);
-        smem = sm > smem ? sm : smem;
+        for (int h : {b->tr[i], batch_half(b, i)}) smem = std::max(smem, batch_tile_bytes(b->prec, h, N, b->ks, b->paired));
     }
     if (smem > 227 * 1024) return bset_err(b, TEUK_E_INVAL, "a tile of the batch does not fit in shared memory");
     int k = b->prec == TEUK_FP32 ? split_batch_blocks_per_sm<float>(b->seg, smem, b->ks)
@@ -1805,10 +1825,7 @@ int batch_layout(teuk_batch *b)
         for (bool more = true; more;) {
             more = false;
             for (int i = 0; i < n; ++i) {
-                const int Nr = (int)b->c[i]->d.Nr, rpp = batch_rpp((int)b->c[i]->d.Ntheta);
-                // half of the tile's row-solve passes, if it has two
-                const int hr = ((b->tr[i] + 2 * b->ks) / 2 + rpp - 1) / rpp * rpp - 2 * b->ks;
-                const int h = half && hr >= 1 && hr < b->tr[i] ? hr : b->tr[i];
+                const int Nr = (int)b->c[i]->d.Nr, h = half ? batch_half(b, i) : b->tr[i];
                 if (row[i] >= (half ? Nr : (int)((1.0 - tail) * Nr))) continue;
                 b->htiles.push_back(make_int2(i | h << kTileShift, row[i]));
                 row[i] += h;
@@ -2001,15 +2018,13 @@ int teuk_batch_create(teuk_ctx *const *ctxs, int count, void *d_ws, size_t ws_by
     b->c.assign(ctxs, ctxs + count);
     b->prec = prec;
     b->seg = seg;
-    b->paired = prec == TEUK_FP32;
-    for (int i = 0; i < count; ++i) b->paired = b->paired && pair_eligible((int)ctxs[i]->d.Ntheta);
     b->ws = (char *)d_ws;
     b->ws_bytes = ws_bytes;
     batch_ws_bytes(ctxs, count, &b->par_bytes, &b->off_tiles);
     for (int k = 0; k < 3; ++k) b->off_par[k] = (size_t)k * b->par_bytes;
     b->ks = split_batch_available(seg, 2) ? 2 : 1;
     b->tr.resize(count);
-    for (int i = 0; i < count; ++i) b->tr[i] = batch_default_tr(ctxs[i], b->ks, b->paired);
+    for (int i = 0; i < count; ++i) b->tr[i] = batch_default_tr(ctxs[i], b->ks, batch_pairs(b));
     r = batch_layout(b);
     if (r != TEUK_OK) {
         memcpy(g_init_err, b->err, sizeof(g_init_err));
@@ -2112,7 +2127,7 @@ int teuk_batch_autotune(teuk_batch *b, int trial_steps, void *stream)
     for (int ks = 1; ks <= 2 && rc == TEUK_OK; ++ks) {
         if (!split_batch_available(b->seg, ks)) continue;
         b->ks = ks;
-        for (size_t i = 0; i < b->c.size(); ++i) b->tr[i] = batch_default_tr(b->c[i], ks, b->paired);
+        for (size_t i = 0; i < b->c.size(); ++i) b->tr[i] = batch_default_tr(b->c[i], ks, batch_pairs(b));
         for (int N : classes) {
             const int rpp = batch_rpp(N);
             std::vector<int> keep = b->tr;

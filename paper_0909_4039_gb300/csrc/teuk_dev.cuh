@@ -1037,7 +1037,7 @@ __device__ __forceinline__ int interior_row(int lr, int g0, int Nr)
 }
 
 // One row, by one warp, through the solve its grid's step kernels use
-// (128 < Ntheta <= 256 in FP32: HALVES, needing the paired theta table th2;
+// (kPaired: implicit_pair on the row's halves, with the paired theta table th2,
 // lane g of G = 32); else implicit_row_fwd.
 template <typename T, int S>
 __device__ __forceinline__ void implicit_row_one(const ImpConst<T> &K, typename V2<T>::t *phi, typename V2<T>::t *pi, int gi,
@@ -1818,7 +1818,8 @@ __device__ __forceinline__ void split_tile(const StepParams<T> &p, int i0, int n
         }
     }
     for (int idx = tid; idx < NTF * N; idx += NT) sTh[idx] = p.thtab[idx];
-    if constexpr (kPaired<T, S>) pair_th_fill(sTh2, p.thtab, N, tid, NT);
+    if constexpr (kPaired<T, S>)
+        if (plan.th2) pair_th_fill(sTh2, p.thtab, N, tid, NT);
     // Every implicit step of the launch uses K: with more steps per launch K
     // is the full step (the launcher refuses first steps and state outputs).
     for (int lr = tid; lr < R; lr += NT) {
@@ -1872,9 +1873,14 @@ __device__ __forceinline__ void split_tile(const StepParams<T> &p, int i0, int n
                 }
             }
             if constexpr (kPaired<T, S>) {
-                implicit_row_one<T, S>(Ki, sPhi + lrc * P, sPi + lrc * P, active ? gi : 1,
-                                       sSt + 2 * interior_row(lrc, g0, Nr) * NSF, sTh, sTh2, N, active, in_tile, g, G, vec,
-                                       s_plan[lrc], t1f, t1g);
+                // (two calls, so that the loads of a shared-memory table are known as such)
+                auto row = [&](const unsigned long long *th2) {
+                    implicit_row_one<T, S>(Ki, sPhi + lrc * P, sPi + lrc * P, active ? gi : 1,
+                                           sSt + 2 * interior_row(lrc, g0, Nr) * NSF, sTh, th2, N, active, in_tile, g, G,
+                                           vec, s_plan[lrc], t1f, t1g);
+                };
+                if (plan.th2) row(sTh2);
+                else row(p.th2);
                 continue;
             }
             // FP64 (first steps): the stored segment products spare FP64 arithmetic,
@@ -1910,7 +1916,7 @@ __device__ __forceinline__ void split_tile(const StepParams<T> &p, int i0, int n
     auto own_sample = [&](c2 *rf, c2 *rg, long long n) {
         if (tid < 32) {
             const bool mine = tid < G, active = mine && p.i_ext >= 1 && p.i_ext <= Nr - 2;
-            implicit_row_one<T, S>(p.half, rf, rg, p.i_ext, sSt + 2 * lx * NSF, sTh, sTh2, N, active, mine, tid & (G - 1), G,
+            implicit_row_one<T, S>(p.half, rf, rg, p.i_ext, sSt + 2 * lx * NSF, sTh, p.th2, N, active, mine, tid & (G - 1), G,
                                    vec, p.half.plan[p.i_ext]);
             __syncwarp();
             extract_warp<T>(p, rf, n);
@@ -2053,7 +2059,7 @@ __device__ __forceinline__ void split_tile(const StepParams<T> &p, int i0, int n
                 } else {
                     const bool mine = tid < G, active = mine && p.i_ext >= 1 && p.i_ext <= Nr - 2;
                     c2 *rf = sPhi + lx * P, *rg = sPi + lx * P;
-                    implicit_row_one<T, S>(p.half, rf, rg, p.i_ext, sSt + 2 * lx * NSF, sTh, sTh2, N, active, mine,
+                    implicit_row_one<T, S>(p.half, rf, rg, p.i_ext, sSt + 2 * lx * NSF, sTh, p.th2, N, active, mine,
                                            tid & (G - 1), G, vec, p.half.plan[p.i_ext]);
                     __syncwarp();
                     h = sample_warp<T>(p, rf);

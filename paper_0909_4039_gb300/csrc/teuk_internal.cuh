@@ -191,6 +191,7 @@ template <typename T> struct StepParams {
     StepPlanes<T> mat;       // materialised coefficients (mat_on)
     int mat_on;              // 1: full steps read them (FP64 state)
     const T *thtab;          // [NTF][Nth]
+    const unsigned long long *th2;   // paired theta table of the FP32 row solves (teuk_pair.cuh), [kPairTh][128]
     const c2 *patch;         // [np][2][Nth]
     const double *w;         // [Nth]
     const double2 *seed;     // [2][Nth]: C_{dt/2}^H E^H 1 on the extraction row (FP64 state)
@@ -222,6 +223,9 @@ template <typename T> struct StepParams {
 // SDIRK2 constant gamma = 1 - 1/sqrt(2) (Alexander 1977).
 constexpr double kGamma = 0.29289321881345247559915563789515;
 constexpr double kPi = 3.14159265358979323846264338327950;
+
+// Fields of the paired theta table (sin^2, cos, AM, A0, AP); it exists for FP32 rows of 128 < Ntheta <= 256.
+constexpr int kPairTh = 5;
 
 // Lane segments of the implicit row solves.
 constexpr int kSegNarrow = 4;           // theta elements per thread (Ntheta <= 128)
@@ -260,12 +264,15 @@ __host__ __device__ inline int implicit_group(int Nth)
 // the tile rows' Thomas pivots; rt holds the step-table entries (SField) of
 // the tile's positions, nodes and half nodes interleaved as in the global
 // table.
-// th2: the paired theta table of the FP32 row solves (teuk_pair.cuh): five
-// fields of 128 pairs, for 128 < Ntheta <= 256.
+// th2: a copy of the paired theta table of the FP32 row solves (teuk_pair.cuh),
+// for 128 < Ntheta <= 256; 0 in tiles that it would make too large, whose row
+// solves read the table from global memory (2000 x 250, two steps a launch:
+// 16.1 us a step that way, 15.3 with the copy).
 __host__ __device__ inline unsigned pair_th_bytes(int N, int tsize)
 {
-    return tsize == 4 && implicit_seg(N) == kSeg ? 5u * 128u * 8u : 0u;
+    return tsize == 4 && implicit_seg(N) == kSeg ? (unsigned)kPairTh * 128u * 8u : 0u;
 }
+constexpr unsigned kPairThFits = 224u * 1024u;   // a block's limit less static parts
 struct SplitSmem {
     unsigned phi, pi, piv, rt, th, th2, total;
 };
@@ -279,16 +286,26 @@ __host__ __device__ inline SplitSmem split_smem_plan(int R, int N, int tsize)
     s.piv = smem_align16(s.pi + plane);
     s.rt = s.piv;   // no pivot plane: the row solves read the pivots from global memory (L2)
     s.th = smem_align16(s.rt + (unsigned)(2 * R - 1) * NSF * (unsigned)tsize);
-    s.th2 = smem_align16(s.th + (unsigned)NTF * (unsigned)N * (unsigned)tsize);
-    s.total = smem_align16(s.th2 + pair_th_bytes(N, tsize));
+    s.total = smem_align16(s.th + (unsigned)NTF * (unsigned)N * (unsigned)tsize);
+    s.th2 = 0;
+    if (pair_th_bytes(N, tsize) && s.total + pair_th_bytes(N, tsize) <= kPairThFits) {
+        s.th2 = s.total;
+        s.total += pair_th_bytes(N, tsize);
+    }
     return s;
 }
 
 // Dynamic shared memory of split_tile (k_split_step, 2, 3 and k_split_batch) for
-// a tile of tile_rows output rows and ks steps per launch.
+// a tile of tile_rows output rows and up to ks steps per launch (a smaller tile
+// may take more: it may hold the copy of the theta table).
 inline size_t split_tile_bytes(int tile_rows, int Nth, int ks, size_t real_bytes)
 {
-    return split_smem_plan(tile_rows + 2 * ks, Nth, (int)real_bytes).total + (ks > 1 ? own_copy_bytes(Nth, real_bytes) : 0);
+    size_t most = 0;
+    for (int k = 1; k <= ks; ++k) {
+        const size_t b = split_smem_plan(tile_rows + 2 * k, Nth, (int)real_bytes).total + (k > 1 ? own_copy_bytes(Nth, real_bytes) : 0);
+        most = b > most ? b : most;
+    }
+    return most;
 }
 
 // Shared-memory carve-up of the persistent split kernel: theta tables, a
@@ -322,15 +339,14 @@ __host__ __device__ inline PersistSmem persist_smem_plan(int R, int N, int tsize
 // [2R][NSF] and the scan plans of its rows (R + 8 ints, the copy starts on
 // a 16-byte boundary of the global plan array).
 struct PipeSmem {
-    unsigned th, th2, xphi, xpi, buf, pi, piv, st, plan, bsize, total;
+    unsigned th, xphi, xpi, buf, pi, piv, st, plan, bsize, th2, total;
 };
 __host__ __device__ inline PipeSmem pipe_smem_plan(int R, int N, int tsize)
 {
     PipeSmem s;
     const unsigned c2 = 2u * (unsigned)tsize, plane = (unsigned)R * (unsigned)N * c2;
     s.th = 0;
-    s.th2 = smem_align16((unsigned)NTF * (unsigned)N * (unsigned)tsize);
-    s.xphi = smem_align16(s.th2 + pair_th_bytes(N, tsize));
+    s.xphi = smem_align16((unsigned)NTF * (unsigned)N * (unsigned)tsize);
     s.xpi = smem_align16(s.xphi + (unsigned)N * c2);
     s.buf = smem_align16(s.xpi + (unsigned)N * c2);
     s.pi = smem_align16(plane);
@@ -339,12 +355,17 @@ __host__ __device__ inline PipeSmem pipe_smem_plan(int R, int N, int tsize)
     s.plan = smem_align16(s.st + 2u * (unsigned)R * NSF * (unsigned)tsize);
     s.bsize = smem_align16(s.plan + ((unsigned)R + 8u) * 4u);
     s.total = s.buf + 2u * s.bsize;
+    s.th2 = 0;   // as in SplitSmem
+    if (pair_th_bytes(N, tsize) && s.total + pair_th_bytes(N, tsize) <= kPairThFits) {
+        s.th2 = s.total;
+        s.total += pair_th_bytes(N, tsize);
+    }
     return s;
 }
 
 // ---------------------------------------------------------------- host side
 struct Layout {
-    size_t rtab64, rtabT, stab, dstab, th64, thT, piv, pivh, plan, planh, seg, segh, patch, patchu, patchd, w, seed, ctl, raw, staging,
+    size_t rtab64, rtabT, stab, dstab, th64, thT, piv, pivh, plan, planh, seg, segh, patch, patchu, patchd, w, seed, th2, ctl, raw, staging,
         scratch;
     size_t mat, mat_bytes;   // materialised coefficients (FP64 split scheme; 0 bytes otherwise)
     size_t total;
@@ -443,29 +464,32 @@ void persist_explain(int Nth, int nc, size_t smem, char *buf, size_t len);   // 
 template <typename T>
 cudaError_t launch_split_persist(const StepParams<T> &p, int nc, int grid, size_t smem, cudaStream_t st);
 template <typename T>
-int split_blocks_per_sm(int Nth, int threads, size_t smem);   // 0 if the launch cannot fit
+int split_blocks_per_sm(int tile_rows, int Nth, int threads, size_t smem);   // 0 if the launch cannot fit
 // Two time steps per launch (k_split_step2): tile of tile_rows output rows
 // with two halo rows on either side.  Full steps only (not the first step
 // from a physical state, not the state output).
 template <typename T>
 size_t split2_smem_bytes(int tile_rows, int Nth);
 template <typename T>
-int split2_blocks_per_sm(int Nth, int threads, size_t smem);
+int split2_blocks_per_sm(int tile_rows, int Nth, int threads, size_t smem);
 template <typename T>
 cudaError_t launch_split_step2(const StepParams<T> &p, int threads, size_t smem, cudaStream_t st);
 // The same with three time steps per launch (tiles of tile_rows + 6 rows).
 template <typename T>
 size_t split3_smem_bytes(int tile_rows, int Nth);
 template <typename T>
-int split3_blocks_per_sm(int Nth, int threads, size_t smem);
+int split3_blocks_per_sm(int tile_rows, int Nth, int threads, size_t smem);
 template <typename T>
 cudaError_t launch_split_step3(const StepParams<T> &p, int threads, size_t smem, cudaStream_t st);
 // The FP32 step kernels on packed pairs (teuk_pair_tile.cuh): ks = 1 .. 3 full
 // steps per launch for 128 < Ntheta <= 256, a multiple of 4 (whole lane
 // segments and bulk-copyable rows).  They take the place of k_split_step / 2 /
-// 3 and of the batched kernel there; first steps, state output and steps on
-// caller buffers stay with k_split_step.
+// 3 and of the batched kernel there, at the heights whose tile fits (pair_runs:
+// a pair tile's rows are 256 points long, so that it holds half the rows of
+// 132 points that k_split_step's does; the results are the same bits); first
+// steps, state output and steps on caller buffers stay with k_split_step.
 bool pair_eligible(int Nth);
+bool pair_runs(int tile_rows, int Nth, int ks);
 size_t pair_smem_bytes(int tile_rows, int Nth, int ks);
 int pair_blocks_per_sm(int ks, size_t smem);
 cudaError_t launch_pair_step(const StepParams<float> &p, int ks, cudaStream_t st);

@@ -6,6 +6,12 @@ namespace teuk {
 
 bool pair_eligible(int Nth) { return Nth > 128 && Nth <= 256 && Nth % 4 == 0; }
 
+bool pair_runs(int tile_rows, int Nth, int ks)
+{
+    // the limit of a block, less the batched kernel's static part (1.7 KB)
+    return pair_eligible(Nth) && pair_smem_bytes(tile_rows, Nth, ks) <= 225 * 1024;
+}
+
 size_t pair_smem_bytes(int tile_rows, int Nth, int ks) { return pair_smem_plan(tile_rows + 2 * ks, Nth).total; }
 
 static void (*pair_fn(int ks))(const StepParams<float>)
@@ -32,7 +38,7 @@ int pair_batch_blocks_per_sm(int ks, size_t smem) { return blocks_per_sm((const 
 
 cudaError_t launch_pair_step(const StepParams<float> &p, int ks, cudaStream_t st)
 {
-    if (p.first || p.imp_only || p.nfix >= 0 || !pair_eligible(p.Nth)) return cudaErrorInvalidValue;
+    if (p.first || p.imp_only || p.nfix >= 0 || !pair_runs(p.tile_rows, p.Nth, ks)) return cudaErrorInvalidValue;
     auto fn = pair_fn(ks);
     cudaError_t e = smem_limit_max((const void *)fn);
     if (e != cudaSuccess) return e;

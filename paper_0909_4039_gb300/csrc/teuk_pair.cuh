@@ -256,9 +256,7 @@ struct PairRow {
     bool active, in_tile;
 };
 
-constexpr int kPairTh = 5;   // fields of the paired theta table: sin^2, cos, AM, A0, AP
-
-// Fills the paired theta table: entry j holds the values at theta j and
+// Fills the paired theta table (StepParams::th2, and the tiles' copies): entry j holds the values at theta j and
 // 128 + j; zero past the row's end, so that padding elements have no coupling.
 __device__ __forceinline__ void pair_th_fill(f2x *th2, const float *thtab, int N, int tid, int NT)
 {

@@ -93,6 +93,7 @@ __global__ void __launch_bounds__(256) k_scan_plans(const StepParams<T> p, int *
     len = len < 0 ? 0 : (len > S ? S : len);
     if (!active) len = 0;
     if constexpr (kPaired<T, S>) {
+        if (blockIdx.x == 0) pair_th_fill((f2x *)p.th2, p.thtab, N, tid, (int)blockDim.x);
         // one warp per row; segments of four elements, lane g's at 4 g and at 128 + 4 g
         for (int h = 0; h < 2; ++h) {
             const ImpConst<T> &K = h ? p.half : p.full;
@@ -273,7 +274,8 @@ __global__ void __launch_bounds__(NTH, (NTH == 256 && sizeof(T) == 4 && S <= 4) 
         if ((int)blockIdx.x < ntiles) issue((int)blockIdx.x, 0);
     }
     for (int idx = tid; idx < NTF * N; idx += NT) sTh[idx] = p.thtab[idx];
-    if constexpr (kPaired<T, S>) pair_th_fill(sTh2, p.thtab, N, tid, NT);
+    if constexpr (kPaired<T, S>)
+        if (L.th2) pair_th_fill(sTh2, p.thtab, N, tid, NT);
     __syncthreads();
 
     const int g = tid % G;
@@ -325,10 +327,15 @@ __global__ void __launch_bounds__(NTH, (NTH == 256 && sizeof(T) == 4 && S <= 4) 
                         continue;
                     }
                 }
-                if constexpr (kPaired<T, S>)
-                    implicit_row_one<T, S>(K, sPhi + lrc * P, sPi + lrc * P, active ? gi : 1,
-                                           sSt + 2 * interior_row(lrc, g0, Nr) * NSF, sTh, sTh2, N, active, in_tile, g, G, vec, plan);
-                else
+                if constexpr (kPaired<T, S>) {
+                    auto row = [&](const unsigned long long *th2) {
+                        implicit_row_one<T, S>(K, sPhi + lrc * P, sPi + lrc * P, active ? gi : 1,
+                                               sSt + 2 * interior_row(lrc, g0, Nr) * NSF, sTh, th2, N, active, in_tile, g, G,
+                                               vec, plan);
+                    };
+                    if (L.th2) row(sTh2);
+                    else row(p.th2);
+                } else
                     implicit_row_fwd<T, S>(K, sPhi + lrc * P, sPi + lrc * P, K.piv + (size_t)(active ? gi : 1) * N, sSt + 2 * lrc * NSF, sTh, N,
                                            active, in_tile, g, G, vec, plan);
             }
@@ -370,7 +377,7 @@ __global__ void __launch_bounds__(NTH, (NTH == 256 && sizeof(T) == 4 && S <= 4) 
                 __syncwarp();
                 const bool mine = tid < G;
                 const bool active = mine && p.i_ext >= 1 && p.i_ext <= Nr - 2;
-                implicit_row_one<T, S>(p.half, xPhi, xPi, p.i_ext, sSt + 2 * lx * NSF, sTh, sTh2, N, active, mine, tid % G, G,
+                implicit_row_one<T, S>(p.half, xPhi, xPi, p.i_ext, sSt + 2 * lx * NSF, sTh, p.th2, N, active, mine, tid % G, G,
                                        vec, p.half.plan[p.i_ext]);
                 __syncwarp();
                 extract_warp<T>(p, xPhi, slot);
@@ -552,7 +559,7 @@ template <typename T>
 size_t split_smem_bytes(int tile_rows, int Nth)
 {
     size_t sm = split_tile_bytes(tile_rows, Nth, 1, sizeof(T));
-    if (sizeof(T) == 4 && pair_eligible(Nth)) {
+    if (sizeof(T) == 4 && pair_runs(tile_rows, Nth, 1)) {
         const size_t pm = pair_smem_bytes(tile_rows, Nth, 1);
         sm = pm > sm ? pm : sm;
     }
@@ -564,7 +571,7 @@ size_t split_smem_bytes(int tile_rows, int Nth)
 template <typename T>
 size_t split2_smem_bytes(int tile_rows, int Nth)
 {
-    if (sizeof(T) == 4 && pair_eligible(Nth)) {
+    if (sizeof(T) == 4 && pair_runs(tile_rows, Nth, 2)) {
         // (a first step runs the one-step kernel at the same height)
         const size_t pm = pair_smem_bytes(tile_rows, Nth, 2), sm = split_smem_bytes<T>(tile_rows, Nth);
         return pm > sm ? pm : sm;
@@ -573,14 +580,14 @@ size_t split2_smem_bytes(int tile_rows, int Nth)
 }
 
 template <typename T>
-int split_blocks_per_sm(int Nth, int threads, size_t smem)
+int split_blocks_per_sm(int tile_rows, int Nth, int threads, size_t smem)
 {
     const int seg = implicit_seg(Nth);
     auto fn = seg == kSegNarrow ? k_split_step<T, kSegNarrow> : (seg == kSeg ? k_split_step<T, kSeg> : k_split_step<T, kSegWide>);
     // both kernels run at one height: full steps on pairs, first steps here
     int cap = 1 << 20;
     if constexpr (sizeof(T) == 4)
-        if (pair_eligible(Nth)) cap = pair_blocks_per_sm(1, smem);
+        if (pair_runs(tile_rows, Nth, 1)) cap = pair_blocks_per_sm(1, smem);
     if (smem_limit_max((const void *)fn) != cudaSuccess) {
         cudaGetLastError();
         return 0;
@@ -597,7 +604,7 @@ template <typename T>
 cudaError_t launch_split_step(const StepParams<T> &p, int threads, size_t smem, cudaStream_t st)
 {
     if constexpr (sizeof(T) == 4)
-        if (!p.first && !p.imp_only && p.nfix < 0 && pair_eligible(p.Nth)) return launch_pair_step(p, 1, st);
+        if (!p.first && !p.imp_only && p.nfix < 0 && pair_runs(p.tile_rows, p.Nth, 1)) return launch_pair_step(p, 1, st);
     if (smem < split_tile_bytes(p.tile_rows, p.Nth, 1, sizeof(T))) return cudaErrorInvalidValue;
     const int seg = implicit_seg(p.Nth);
     const int v = seg == kSegNarrow ? 0 : (seg == kSeg ? 1 : 2);
@@ -676,10 +683,10 @@ static void (*split2_fn(int Nth))(const StepParams<T>)
 }
 
 template <typename T>
-int split2_blocks_per_sm(int Nth, int threads, size_t smem)
+int split2_blocks_per_sm(int tile_rows, int Nth, int threads, size_t smem)
 {
     if constexpr (sizeof(T) == 4)
-        if (pair_eligible(Nth)) return pair_blocks_per_sm(2, smem);
+        if (pair_runs(tile_rows, Nth, 2)) return pair_blocks_per_sm(2, smem);
     auto fn = split2_fn<T>(Nth);
     if (smem_limit_max((const void *)fn) != cudaSuccess) {
         cudaGetLastError();
@@ -698,7 +705,7 @@ cudaError_t launch_split_step2(const StepParams<T> &p, int threads, size_t smem,
 {
     if (p.first || p.imp_only) return cudaErrorInvalidValue;   // two full steps only
     if constexpr (sizeof(T) == 4)
-        if (pair_eligible(p.Nth)) return launch_pair_step(p, 2, st);
+        if (pair_runs(p.tile_rows, p.Nth, 2)) return launch_pair_step(p, 2, st);
     if (smem < split_tile_bytes(p.tile_rows, p.Nth, 2, sizeof(T))) return cudaErrorInvalidValue;
     auto fn = split2_fn<T>(p.Nth);
     if constexpr (own_samples(sizeof(T), kSegNarrow))
@@ -720,7 +727,7 @@ static void (*split3_fn(int Nth))(const StepParams<T>)
 template <typename T>
 size_t split3_smem_bytes(int tile_rows, int Nth)
 {
-    if (sizeof(T) == 4 && pair_eligible(Nth)) {
+    if (sizeof(T) == 4 && pair_runs(tile_rows, Nth, 3)) {
         // (a first step runs the one-step kernel at the same height)
         const size_t pm = pair_smem_bytes(tile_rows, Nth, 3), sm = split_smem_bytes<T>(tile_rows, Nth);
         return pm > sm ? pm : sm;
@@ -729,10 +736,10 @@ size_t split3_smem_bytes(int tile_rows, int Nth)
 }
 
 template <typename T>
-int split3_blocks_per_sm(int Nth, int threads, size_t smem)
+int split3_blocks_per_sm(int tile_rows, int Nth, int threads, size_t smem)
 {
     if constexpr (sizeof(T) == 4)
-        if (pair_eligible(Nth)) return pair_blocks_per_sm(3, smem);
+        if (pair_runs(tile_rows, Nth, 3)) return pair_blocks_per_sm(3, smem);
     auto fn = split3_fn<T>(Nth);
     if (smem_limit_max((const void *)fn) != cudaSuccess) {
         cudaGetLastError();
@@ -751,7 +758,7 @@ cudaError_t launch_split_step3(const StepParams<T> &p, int threads, size_t smem,
 {
     if (p.first || p.imp_only) return cudaErrorInvalidValue;   // three full steps only
     if constexpr (sizeof(T) == 4)
-        if (pair_eligible(p.Nth)) return launch_pair_step(p, 3, st);
+        if (pair_runs(p.tile_rows, p.Nth, 3)) return launch_pair_step(p, 3, st);
     if (smem < split_tile_bytes(p.tile_rows, p.Nth, 3, sizeof(T))) return cudaErrorInvalidValue;
     auto fn = split3_fn<T>(p.Nth);
     if constexpr (own_samples(sizeof(T), kSegNarrow))

@@ -169,3 +169,35 @@ def test_fp32_batch_of_packed_and_scalar_widths(widths):
     b.close()
     for st in sts:
         st.close()
+
+
+@pytest.mark.parametrize("Nth,tall", [(132, (97, 94, 92)), (200, (64, 61, 59)), (250, (51, 48, 46))])
+def test_fp32_tall_tiles_of_paired_widths(Nth, tall):
+    """Heights beyond a pair tile's (and, at 250 points, the tallest plain tiles):
+    accepted for a lone state with one, two and three steps a launch and in a
+    batch, with the bits of the default tiles."""
+    from paper_0909_4039_gb300 import teuk
+    w, n, got = _w(330, Nth), 7, []
+    u0 = inputs.random_state(w.Nr, Nth, seed=50)
+    for ks, tr in [(None, None), *enumerate(tall, 1)]:
+        st = gpu_stepper(w, "fp32", wave_capacity=n + 1)
+        if tr:
+            st.set_tiling(tr, ks)
+            assert st.tiling()["tile_rows"] == tr
+        st.set_state(u0, 0)
+        st.step(n)
+        got.append((st.get_state(), st.waveform(0, n + 1)))
+        st.close()
+    st = gpu_stepper(w, "fp32", wave_capacity=n + 1)
+    b = teuk.Batch([st])
+    for ks in (2, 1):
+        # (the batched kernel's parameters take a kilobyte of their own)
+        b.set_tiling([tall[ks - 1] - 1], ks)
+        st.set_state(u0, 0)
+        b.step(n)
+        b.synchronize()
+        got.append((st.get_state(), st.waveform(0, n + 1)))
+    b.close()
+    st.close()
+    for u, h in got[1:]:
+        assert np.array_equal(u, got[0][0]) and np.array_equal(h, got[0][1])

@@ -60,7 +60,6 @@ struct teuk_ctx {
     size_t one_smem;
     int persist, nc, grid;
     int pipe;                // the pipelined two-step kernel (grid persistent CTAs)
-    int own;                 // tiles sample their own steps (a call of a few steps)
     size_t persist_smem;
     int ks;                  // time steps per launch of the tiled kernel (1, 2 or 3)
     int wait0;               // teuk_set_wait_limit (< 0: default bound)
@@ -520,7 +519,7 @@ StepParams<T> make_params(const teuk_ctx *c, int in_level)
     p.th2 = (const unsigned long long *)(c->coef + c->L.th2);
     p.patch = (const c2 *)(c->coef + c->L.patch);
     p.nfix = -1;
-    p.own = c->own;
+    p.own = 0;
     p.h_out = nullptr;
     p.tape = nullptr;
     p.patchu = (const c2 *)(c->coef + c->L.patchu);
@@ -577,50 +576,33 @@ cudaError_t compute_seed(teuk_ctx *c, cudaStream_t st)
     return launch_seed(make_params<double>(c, 0), (double2 *)(c->coef + c->L.seed), st);
 }
 
-cudaError_t launch_one(teuk_ctx *c, int in_level, cudaStream_t st)
+// Time steps of a launch of the configured kernel: two or three when it takes
+// that many and the state is shifted (full steps follow), else one.
+int unit_steps(const teuk_ctx *c) { return c->d.scheme == TEUK_SCHEME_SPLIT && c->ks >= 2 && c->shifted ? c->ks : 1; }
+
+// Whether the tiles of a call of nsteps steps sample their own steps (own_samples).
+bool own_call(const teuk_ctx *c, int64_t nsteps)
 {
-    if (c->d.precision == TEUK_FP32) {
-        StepParams<float> p = make_params<float>(c, in_level);
-        return c->d.scheme == TEUK_SCHEME_SPLIT ? launch_split<float>(c, p, st) : launch_literal_step<float>(p, st);
-    }
-    StepParams<double> p = make_params<double>(c, in_level);
-    return c->d.scheme == TEUK_SCHEME_SPLIT ? launch_split<double>(c, p, st) : launch_literal_step<double>(p, st);
+    return nsteps <= kOwnSteps && own_samples(c->d.precision == TEUK_FP32 ? 4 : 8, implicit_seg((int)c->d.Ntheta));
 }
 
-// The last two steps of a call with three steps per launch, in one launch at the
-// same tile height (16384 x 128 FP32, two steps a call: 53 us against 64 in two
-// launches).
-cudaError_t launch_two(teuk_ctx *c, int in_level, cudaStream_t st)
+// One launch of ks steps (1, or 2 and 3 of a shifted state) from level in_level;
+// own: its tiles sample them.
+template <typename T>
+cudaError_t launch_steps_of(teuk_ctx *c, int in_level, int ks, bool own, cudaStream_t st)
 {
-    if (c->d.precision == TEUK_FP32)
-        return launch_split_step2<float>(make_params<float>(c, in_level), c->threads, c->smem2, st);
-    return launch_split_step2<double>(make_params<double>(c, in_level), c->threads, c->smem2, st);
+    StepParams<T> p = make_params<T>(c, in_level);
+    p.own = own;
+    if (ks == 3) return launch_split_step3<T>(p, c->threads, c->smem2, st);
+    if (ks == 2)
+        return c->pipe ? launch_split_pipe<T>(p, c->nc, c->grid, c->smem2, st)
+                       : launch_split_step2<T>(p, c->threads, c->smem2, st);
+    return c->d.scheme == TEUK_SCHEME_SPLIT ? launch_split<T>(c, p, st) : launch_literal_step<T>(p, st);
 }
-
-// One launch of the configured kernel from level in_level: two or three
-// steps when the tiled kernel takes that many per launch and the state is
-// shifted (full steps follow), else one; *steps receives the count.
-cudaError_t launch_unit(teuk_ctx *c, int in_level, cudaStream_t st, int *steps)
+cudaError_t launch_steps(teuk_ctx *c, int in_level, int ks, bool own, cudaStream_t st)
 {
-    if (c->d.scheme == TEUK_SCHEME_SPLIT && c->ks == 3 && c->shifted) {
-        *steps = 3;
-        if (c->d.precision == TEUK_FP32)
-            return launch_split_step3<float>(make_params<float>(c, in_level), c->threads, c->smem2, st);
-        return launch_split_step3<double>(make_params<double>(c, in_level), c->threads, c->smem2, st);
-    }
-    if (c->d.scheme == TEUK_SCHEME_SPLIT && c->ks == 2 && c->shifted) {
-        *steps = 2;
-        if (c->d.precision == TEUK_FP32) {
-            StepParams<float> p = make_params<float>(c, in_level);
-            return c->pipe ? launch_split_pipe<float>(p, c->nc, c->grid, c->smem2, st)
-                           : launch_split_step2<float>(p, c->threads, c->smem2, st);
-        }
-        StepParams<double> p = make_params<double>(c, in_level);
-        return c->pipe ? launch_split_pipe<double>(p, c->nc, c->grid, c->smem2, st)
-                       : launch_split_step2<double>(p, c->threads, c->smem2, st);
-    }
-    *steps = 1;
-    return launch_one(c, in_level, st);
+    return c->d.precision == TEUK_FP32 ? launch_steps_of<float>(c, in_level, ks, own, st)
+                                       : launch_steps_of<double>(c, in_level, ks, own, st);
 }
 
 // Physical state u_n = C_{dt/2} s_n of a shifted split-scheme state, written
@@ -975,10 +957,10 @@ int teuk_step(teuk_ctx *c, int64_t nsteps, void *stream)
     int64_t left = nsteps;
     int pending = 0;   // steps whose extraction rows wait for a sampling launch
     const bool split = c->d.scheme == TEUK_SCHEME_SPLIT;
-    c->own = nsteps <= kOwnSteps && own_samples(c->d.precision == TEUK_FP32 ? 4 : 8, implicit_seg((int)c->d.Ntheta));
+    const bool own = own_call(c, nsteps);
     if (left > 0 && c->d.scheme == TEUK_SCHEME_SPLIT && !c->shifted) {
         // first step from a physical state: s_{n+1} = LW C_{dt/2} u_n
-        CK(launch_one(c, c->cur, st), "first step launch");
+        CK(launch_steps(c, c->cur, 1, own, st), "first step launch");
         c->cur ^= 1;
         c->shifted = 1;
         left -= 1;
@@ -987,13 +969,13 @@ int teuk_step(teuk_ctx *c, int64_t nsteps, void *stream)
     // the pipelined and persistent kernels sample their own steps: what is left
     // from before them comes first
     auto flush = [&]() -> cudaError_t {
-        if (!split || c->own || pending == 0) return cudaSuccess;
+        if (!split || own || pending == 0) return cudaSuccess;
         const int n = pending;
         pending = 0;
         return sample_steps(c, n, st);
     };
     // steps per launch from here on (the state is shifted)
-    const int ks = (c->d.scheme == TEUK_SCHEME_SPLIT && c->ks >= 2) ? c->ks : 1;
+    const int ks = unit_steps(c);
     // steps per captured graph: a multiple of ks over an even number of launches
     const int chunk = ks == 3 ? 3 * kGraphChunk / 2 : kGraphChunk;
     bool use_graph = st != nullptr && c->d.scheme == TEUK_SCHEME_SPLIT && left >= 2 * chunk;
@@ -1010,9 +992,8 @@ int teuk_step(teuk_ctx *c, int64_t nsteps, void *stream)
             int lev = g, done = 0;
             cudaError_t le = cudaSuccess;
             while (done < chunk && le == cudaSuccess) {
-                int k = 0;
-                le = launch_unit(c, lev, st, &k);
-                done += k;
+                le = launch_steps(c, lev, ks, own, st);
+                done += ks;
                 lev ^= 1;
             }
             cudaError_t ee = cudaStreamEndCapture(st, &graph);
@@ -1034,16 +1015,12 @@ int teuk_step(teuk_ctx *c, int64_t nsteps, void *stream)
         }
     }
     while (left > 0) {
-        int k = 1;
-        if (pending + ks > kRawSlots) CK(flush(), "samples");
-        if (left >= ks) {
-            CK(launch_unit(c, c->cur, st, &k), "step launch");
-        } else if (ks == 3 && left == 2) {
-            k = 2;
-            CK(launch_two(c, c->cur, st), "step launch");
-        } else {
-            CK(launch_one(c, c->cur, st), "step launch");
-        }
+        // (with three steps a launch the last two steps of a call go in one launch of
+        // two at the same tile height: 16384 x 128 FP32, two steps a call, 53 us
+        // against 64 in two launches)
+        const int k = left >= ks ? ks : (int)left;
+        if (pending + k > kRawSlots) CK(flush(), "samples");
+        CK(launch_steps(c, c->cur, k, own, st), "step launch");
         c->cur ^= 1;
         left -= k;
         pending += k;
@@ -1153,35 +1130,51 @@ static int autotune_impl(teuk_ctx *c, int trial_steps, void *flush, size_t flush
         for (size_t k = 0; k < cand.size() && e == cudaSuccess; ++k) {
             if (!apply_cand(c, cand[k])) continue;
             c->shifted = 1;
-            int lev = c->cur, ku = 0, steps = 0;
-            for (int w = 0; w < 3 && e == cudaSuccess; ++w, lev ^= 1) e = launch_unit(c, lev, st, &ku);
+            const int ku = unit_steps(c);
+            int lev = c->cur, pending = 0;
+            // A timed launch is a call of ku steps (cold) or part of a long one (warm);
+            // its steps' samples are timed with it.
+            const bool own = flush && own_call(c, ku), tiled = !c->pipe && !c->persist;
+            auto samples = [&](bool now) {
+                if (own || !tiled || pending == 0 || (!now && pending + ku <= kRawSlots)) return cudaSuccess;
+                const int np = pending;
+                pending = 0;
+                return sample_steps(c, np, st);
+            };
+            auto unit = [&] {
+                cudaError_t le = samples(false);
+                if (le == cudaSuccess) le = launch_steps(c, lev, ku, own, st);
+                lev ^= 1;
+                pending += ku;
+                return le;
+            };
+            for (int w = 0; w < 3 && e == cudaSuccess; ++w) e = unit();
+            if (e == cudaSuccess) e = samples(true);
             float t = 0.0f;
             if (flush) {
                 per.clear();
-                for (int w = 0; w < trial_steps && e == cudaSuccess; ++w, lev ^= 1) {
+                for (int w = 0; w < trial_steps && e == cudaSuccess; ++w) {
                     float ms = 0.0f;
                     e = cudaMemsetAsync(flush, w & 0xff, flush_bytes, st);
                     if (e == cudaSuccess) e = cudaEventRecord(e0, st);
-                    if (e == cudaSuccess) e = launch_unit(c, lev, st, &ku);
+                    if (e == cudaSuccess) e = unit();
+                    if (e == cudaSuccess) e = samples(true);
                     if (e == cudaSuccess) e = cudaEventRecord(e1, st);
                     if (e == cudaSuccess) e = cudaEventSynchronize(e1);
                     if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, e0, e1);
-                    if (e == cudaSuccess && ku > 0) per.push_back(ms / (float)ku);
+                    if (e == cudaSuccess) per.push_back(ms / (float)ku);
                 }
                 if (per.empty()) continue;
                 std::nth_element(per.begin(), per.begin() + per.size() / 2, per.end());
                 t = per[per.size() / 2];
             } else {
                 if (e == cudaSuccess) e = cudaEventRecord(e0, st);
-                for (int w = 0; w < trial_steps && e == cudaSuccess; ++w, lev ^= 1) {
-                    e = launch_unit(c, lev, st, &ku);
-                    steps += ku;
-                }
+                for (int w = 0; w < trial_steps && e == cudaSuccess; ++w) e = unit();
+                if (e == cudaSuccess) e = samples(true);
                 if (e == cudaSuccess) e = cudaEventRecord(e1, st);
                 if (e == cudaSuccess) e = cudaEventSynchronize(e1);
                 if (e == cudaSuccess) e = cudaEventElapsedTime(&t, e0, e1);
-                if (steps < 1) continue;
-                t /= (float)steps;   // time per step
+                t /= (float)trial_steps * (float)ku;   // time per step
             }
             if (e == cudaSuccess && t < score[k]) score[k] = t;
         }

@@ -65,7 +65,6 @@ struct teuk_ctx {
     int wait0;               // teuk_set_wait_limit (< 0: default bound)
     size_t smem2;            // shared memory of the two- or three-step kernel
     const void *adj_ws;      // adjoint workspace whose coefficient planes teuk_adjoint_prepare filled
-    int delta_ok;            // its delta vector is for the present weights
     // graphs, one per starting level
     cudaGraphExec_t graph[2];
     cudaStream_t graph_stream[2];
@@ -106,6 +105,8 @@ Layout make_layout(const teuk_grid_desc &d)
     if (!f32 && d.scheme == TEUK_SCHEME_SPLIT) off = align256(off + c2 * 2 * N * patch_rows);
     L.w = off; off = align256(off + sizeof(double) * N);
     L.seed = off; off = align256(off + 2 * sizeof(double2) * N);
+    L.delta = off;
+    if (!f32 && d.scheme == TEUK_SCHEME_SPLIT) off = align256(off + 2 * sizeof(double2) * N);
     L.th2 = off;
     if (f32 && implicit_seg((int)N) == kSeg) off = align256(off + sizeof(unsigned long long) * kPairTh * 128);
     L.ctl = off; off = align256(off + sizeof(Ctl));
@@ -576,6 +577,13 @@ cudaError_t compute_seed(teuk_ctx *c, cudaStream_t st)
     return launch_seed(make_params<double>(c, 0), (double2 *)(c->coef + c->L.seed), st);
 }
 
+// The sample's spin derivative for the weights as they are (FP64 split scheme).
+cudaError_t compute_delta(teuk_ctx *c, cudaStream_t st)
+{
+    if (c->d.scheme != TEUK_SCHEME_SPLIT || c->d.precision == TEUK_FP32) return cudaSuccess;
+    return launch_delta(make_params<double>(c, 0), (double2 *)(c->coef + c->L.delta), st);
+}
+
 // Time steps of a launch of the configured kernel: two or three when it takes
 // that many and the state is shifted (full steps follow), else one.
 int unit_steps(const teuk_ctx *c) { return c->d.scheme == TEUK_SCHEME_SPLIT && c->ks >= 2 && c->shifted ? c->ks : 1; }
@@ -871,7 +879,9 @@ int teuk_set_weights(teuk_ctx *c, const double *w)
         CK(compute_plans(c, 0), "scan plans");
     }
     CK(compute_seed(c, 0), "sample adjoint");
-    c->delta_ok = 0;
+    // (of a context whose adjoint is prepared: its later steps, and graphs that
+    // hold earlier ones, read the vector where it stands)
+    if (c->adj_ws) CK(compute_delta(c, 0), "sample spin derivative");
     CK(cudaDeviceSynchronize(), "weights sync");
     return TEUK_OK;
 }
@@ -1422,8 +1432,8 @@ AdjPlanes adjoint_planes(const teuk_ctx *c, const void *ws)
     A.af = (const double2 *)(b + L.off[1]);
     A.dlw = (const double2 *)(b + L.off[2]);
     A.dimp = (const double2 *)(b + L.off[3]);
-    A.delta = (const double2 *)(b + L.off[4]);
-    A.plan = (const int *)(b + L.off[5]);
+    A.plan = (const int *)(b + L.off[4]);
+    A.delta = (const double2 *)(c->coef + c->L.delta);
     return A;
 }
 
@@ -1507,9 +1517,8 @@ int teuk_adjoint_prepare(teuk_ctx *c, void *d_ws, void *stream)
         const StepParams<double> p = make_params<double>(c, 0);
         const AdjPlanes A = adjoint_planes(c, d_ws);
         cudaError_t e = launch_adjoint_f64_planes(p, A, st);
-        if (e == cudaSuccess) e = launch_delta(p, (double2 *)A.delta, st);
+        if (e == cudaSuccess) e = compute_delta(c, st);
         if (e != cudaSuccess) return cuda_err(c, e, "adjoint planes");
-        c->delta_ok = 1;
     }
     c->adj_ws = d_ws;
     return TEUK_OK;
@@ -1578,15 +1587,8 @@ static int adjoint_spin(teuk_ctx *c, const void *d_lam_in, void *d_lam_out, cons
             e = launch_adjoint_spin<double>(p, tr, (const double2 *)d_s, (const double2 *)d_tape, (const double2 *)d_gseed,
                                             part, acc, st);
         } else {
-            const AdjPlanes A = adjoint_planes(c, d_ws);
-            e = cudaSuccess;
-            if (!c->delta_ok) {   // the weights have changed since teuk_adjoint_prepare
-                e = launch_delta(p, (double2 *)A.delta, st);
-                if (e == cudaSuccess) c->delta_ok = 1;
-            }
-            if (e == cudaSuccess)
-                e = launch_adjoint_f64(p, adjoint_f64_tile_rows(c, true), true, (const double2 *)d_s, (const double2 *)d_tape,
-                                       (const double2 *)d_gseed, A, part, acc, st);
+            e = launch_adjoint_f64(p, adjoint_f64_tile_rows(c, true), true, (const double2 *)d_s, (const double2 *)d_tape,
+                                   (const double2 *)d_gseed, adjoint_planes(c, d_ws), part, acc, st);
         }
     }
     if (e != cudaSuccess) return cuda_err(c, e, "adjoint step (spin)");

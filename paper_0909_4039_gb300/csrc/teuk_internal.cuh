@@ -130,26 +130,27 @@ constexpr int kLwStencil = 4;           // pairs per element of the stencil plan
 // element to the end of its lane segment, [Nr][Nth]; af, the segments'
 // products of the transposed forward multipliers, [Nr][G]; plan, the scan
 // levels of the transposed solves, [Nr]; the spin derivatives of the stencil
-// (dlw, as StepPlanes::lw) and of the implicit operator (dimp, [Nr][3][Nth] pairs: dW's diagonal, dc_t, dW's off-diagonals);
-// delta, the sample's spin derivative on the extraction row, [2][Nth].
+// (dlw, as StepPlanes::lw) and of the implicit operator (dimp, [Nr][3][Nth] pairs: dW's diagonal, dc_t, dW's off-diagonals).
+// In the context: delta, the sample's spin derivative on the extraction row
+// for the weights as they are, [2][Nth] (teuk_adjoint_prepare and, from then
+// on, teuk_set_weights form it).
 struct AdjPlanes {
     const double2 *pb, *af, *dlw, *dimp, *delta;
     const int *plan;
 };
 
-// Byte layout from offset 0 of their region: pb, af, dlw, dimp, delta, plan.
+// Byte layout from offset 0 of their region: pb, af, dlw, dimp, plan.
 struct AdjPlaneLayout {
-    size_t off[6];
+    size_t off[5];
     size_t total;
 };
 inline AdjPlaneLayout adj_plane_layout(long long Nr, long long Nth, int G)
 {
     const size_t pl = (size_t)Nr * (size_t)Nth, c2 = sizeof(double2);
-    const size_t sz[6] = {pl * c2, (size_t)Nr * (size_t)G * c2, kLwStencil * pl * c2, 3 * pl * c2, 2 * (size_t)Nth * c2,
-                          (size_t)Nr * sizeof(int)};
+    const size_t sz[5] = {pl * c2, (size_t)Nr * (size_t)G * c2, kLwStencil * pl * c2, 3 * pl * c2, (size_t)Nr * sizeof(int)};
     AdjPlaneLayout L;
     size_t o = 0;
-    for (int k = 0; k < 6; ++k) {
+    for (int k = 0; k < 5; ++k) {
         L.off[k] = o;
         o = (o + sz[k] + 255) & ~(size_t)255;
     }
@@ -365,7 +366,7 @@ __host__ __device__ inline PipeSmem pipe_smem_plan(int R, int N, int tsize)
 
 // ---------------------------------------------------------------- host side
 struct Layout {
-    size_t rtab64, rtabT, stab, dstab, th64, thT, piv, pivh, plan, planh, seg, segh, patch, patchu, patchd, w, seed, th2, ctl, raw, staging,
+    size_t rtab64, rtabT, stab, dstab, th64, thT, piv, pivh, plan, planh, seg, segh, patch, patchu, patchd, w, seed, delta, th2, ctl, raw, staging,
         scratch;
     size_t mat, mat_bytes;   // materialised coefficients (FP64 split scheme; 0 bytes otherwise)
     size_t total;

@@ -452,3 +452,63 @@ def test_adjoint_entry_points_reject_bad_calls():
         op.adjoint_spin(lam, lam2, s, 3, False, None)
         op.st.synchronize()
     op.close()
+
+
+@pytest.mark.parametrize("Nth", [16, 33, 130])
+def test_weights_set_after_the_adjoint_is_prepared(Nth):
+    """teuk_set_weights after teuk_adjoint_prepare: later adjoint steps with the
+    spin term, and replays of a captured one, give the bits of a context whose
+    weights were set before it was prepared, whatever was captured in between."""
+    import torch
+    from paper_0909_4039_gb300 import adjoint as A
+    from paper_0909_4039_gb300 import teuk
+    w, n = _w(110, Nth, a=0.6, m=2, sig_r=0.8), 17
+    prm = A.Params(0.8 - 0.5j, 6.0, 0.6)
+    rng = np.random.default_rng(3)
+    w1, w2 = rng.standard_normal(Nth), rng.standard_normal(Nth)
+    op, ref = A.Operator(w, prm, "fp64"), A.Operator(w, prm, "fp64")
+    s = _rand(op.shape, 21, op.st.device, op.ctype, zero_boundary=True)
+    lam = _rand(op.shape, 22, op.st.device, op.ctype)
+    g = torch.tensor([1.1 - 0.6j], dtype=torch.complex128, device=op.st.device)
+    out = torch.zeros_like(lam)
+    torch.cuda.synchronize()
+
+    def step(o):
+        with torch.cuda.stream(o.st.stream):
+            o.ws[:8].zero_()
+            out.zero_()
+            o.adjoint_spin(lam, out, s, n, False, g.data_ptr())
+
+    def result(o):
+        torch.cuda.synchronize()
+        return out.cpu().numpy(), o.ws[:8].cpu().numpy()
+
+    def captured():
+        torch.cuda.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=op.st.stream):
+            step(op)
+        return graph
+
+    want = []
+    for wt in (w1, w2):
+        ref.st.set_weights(wt)
+        teuk._check(teuk.lib().teuk_adjoint_prepare(ref.st.ctx, ref.ws.data_ptr(), ref.st.sh), ref.st.ctx)
+        step(ref)
+        want.append(result(ref))
+    assert want[0][1][4] != want[1][1][4]
+    step(op)                       # (a first launch outside capture)
+    op.st.set_weights(w1)
+    early = captured()             # the first step after the weights changed, not run yet
+    step(op)
+    got = [(0, result(op))]
+    op.st.set_weights(w2)
+    with torch.cuda.stream(op.st.stream):
+        early.replay()             # captured for the former weights
+    got.append((1, result(op)))
+    step(op)
+    got.append((1, result(op)))
+    for k, (u, acc) in got:
+        assert np.array_equal(u, want[k][0]) and np.array_equal(acc, want[k][1]), k
+    op.close()
+    ref.close()

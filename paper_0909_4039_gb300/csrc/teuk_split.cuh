@@ -182,7 +182,8 @@ __global__ void __launch_bounds__(256) k_scan_plans(const StepParams<T> p, int *
 // CTA waits (bounded) for the copies it issued and returns.
 constexpr int kPipeChunks = 4;
 
-template <typename T, int S, int NTH>
+// FAR: the paired theta table is read from global memory (PipeSmem::th2 is 0).
+template <typename T, int S, int NTH, bool FAR = false>
 __global__ void __launch_bounds__(NTH, (NTH == 256 && sizeof(T) == 4 && S <= 4) ? 2 : 1)
     k_split_pipe(const StepParams<T> p)
 {
@@ -274,8 +275,7 @@ __global__ void __launch_bounds__(NTH, (NTH == 256 && sizeof(T) == 4 && S <= 4) 
         if ((int)blockIdx.x < ntiles) issue((int)blockIdx.x, 0);
     }
     for (int idx = tid; idx < NTF * N; idx += NT) sTh[idx] = p.thtab[idx];
-    if constexpr (kPaired<T, S>)
-        if (L.th2) pair_th_fill(sTh2, p.thtab, N, tid, NT);
+    if constexpr (kPaired<T, S> && !FAR) pair_th_fill(sTh2, p.thtab, N, tid, NT);
     __syncthreads();
 
     const int g = tid % G;
@@ -327,15 +327,11 @@ __global__ void __launch_bounds__(NTH, (NTH == 256 && sizeof(T) == 4 && S <= 4) 
                         continue;
                     }
                 }
-                if constexpr (kPaired<T, S>) {
-                    auto row = [&](const unsigned long long *th2) {
-                        implicit_row_one<T, S>(K, sPhi + lrc * P, sPi + lrc * P, active ? gi : 1,
-                                               sSt + 2 * interior_row(lrc, g0, Nr) * NSF, sTh, th2, N, active, in_tile, g, G,
-                                               vec, plan);
-                    };
-                    if (L.th2) row(sTh2);
-                    else row(p.th2);
-                } else
+                if constexpr (kPaired<T, S>)
+                    implicit_row_one<T, S>(K, sPhi + lrc * P, sPi + lrc * P, active ? gi : 1,
+                                           sSt + 2 * interior_row(lrc, g0, Nr) * NSF, sTh, FAR ? p.th2 : sTh2, N, active,
+                                           in_tile, g, G, vec, plan);
+                else
                     implicit_row_fwd<T, S>(K, sPhi + lrc * P, sPi + lrc * P, K.piv + (size_t)(active ? gi : 1) * N, sSt + 2 * lrc * NSF, sTh, N,
                                            active, in_tile, g, G, vec, plan);
             }
@@ -503,9 +499,12 @@ size_t pipe_smem_bytes(int tile_rows, int Nth)
 // The pipelined kernel for Ntheta and `threads` per CTA (256 or 512; 512
 // only for segments of up to 8 elements), or nullptr.
 template <typename T>
-static void (*pipe_fn(int Nth, int threads))(const StepParams<T>)
+static void (*pipe_fn(int Nth, int threads, bool far = false))(const StepParams<T>)
 {
     const int seg = implicit_seg(Nth);
+    if constexpr (sizeof(T) == 4)
+        if (far && seg == kSeg)
+            return threads == 256 ? k_split_pipe<T, kSeg, 256, true> : (threads == 512 ? k_split_pipe<T, kSeg, 512, true> : nullptr);
     if (threads == 256)
         return seg == kSegNarrow ? k_split_pipe<T, kSegNarrow, 256>
                                  : (seg == kSeg ? k_split_pipe<T, kSeg, 256> : k_split_pipe<T, kSegWide, 256>);
@@ -535,7 +534,7 @@ template <typename T>
 cudaError_t launch_split_pipe(const StepParams<T> &p, int threads, int grid, size_t smem, cudaStream_t st)
 {
     if (p.first || p.imp_only || !p.bulk || p.nfix >= 0 || grid < 1) return cudaErrorInvalidValue;
-    auto fn = pipe_fn<T>(p.Nth, threads);
+    auto fn = pipe_fn<T>(p.Nth, threads, pipe_smem_plan(p.tile_rows + 4, p.Nth, (int)sizeof(T)).th2 == 0);
     if (!fn) return cudaErrorInvalidValue;
     cudaError_t e = smem_limit_max((const void *)fn);
     if (e != cudaSuccess) return e;

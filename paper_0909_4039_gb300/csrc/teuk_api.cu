@@ -256,8 +256,10 @@ double host_atheta_bound(const teuk_grid_desc &d)
 //
 // Pipelined and persistent kernels (see pipe_cand, persist_cand): measured
 // 20 to 100 % behind the tiled ones on every grid tried (16384 x 128 FP32 31
-// against 24.5 us, 1024 x 32 FP64 31.5 against 17.3), so their cost carries a
-// factor that keeps them out of the default choice; the autotuners time them.
+// against 24.5 us, 65536 x 32 FP32 29.8 against 25.2, 1024 x 32 FP64 31.5
+// against 17.3), which their cost does not always show.  The default choice
+// leaves them out (choose_tiles); their cost ranks the candidates of one kind
+// for the autotuners, which time them.
 struct TileCand {
     double cost;             // model cost per time step
     int R;                   // tile_rows + 2
@@ -445,13 +447,10 @@ int choose_tiles(teuk_ctx *c)
             c->one_smem = cand[k].smem;
             break;
         }
-    // FP32 defaults leave the pipelined kernel to the autotuners and to
-    // teuk_set_pipelined: its cost model ranks it first on large grids, where it
-    // takes longer than the tiled one (us per step: 16384 x 128 31.6 against 25.7, 65536 x 32
-    // 29.8 against 25.2).
+    // tiled kernels; another only if none of them fits
     for (int pass = 0; pass < 2; ++pass)
         for (int k = 0; k < n; ++k)
-            if ((pass == 1 || !cand[k].pipe || c->d.precision != TEUK_FP32) && apply_cand(c, cand[k])) return TEUK_OK;
+            if ((pass == 1 || (!cand[k].pipe && !cand[k].persist)) && apply_cand(c, cand[k])) return TEUK_OK;
     return set_err(c, TEUK_E_CUDA, "no tile of the split kernel fits on this device");
 }
 

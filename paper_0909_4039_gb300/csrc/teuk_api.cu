@@ -1797,14 +1797,13 @@ int batch_layout(teuk_batch *b)
         for (int h : {b->tr[i], batch_half(b, i)}) smem = std::max(smem, batch_tile_bytes(b->prec, h, N, b->ks, b->paired));
     }
     if (smem > 227 * 1024) return bset_err(b, TEUK_E_INVAL, "a tile of the batch does not fit in shared memory");
-    int k = b->prec == TEUK_FP32 ? split_batch_blocks_per_sm<float>(b->seg, smem, b->ks)
-                                 : split_batch_blocks_per_sm<double>(b->seg, smem, b->ks);
-    // the first step of a two-step batch runs the one-step kernel with this shared memory
-    if (k >= 1 && b->ks == 2)
-        k = b->prec == TEUK_FP32 ? split_batch_blocks_per_sm<float>(b->seg, smem, 1)
-                                 : split_batch_blocks_per_sm<double>(b->seg, smem, 1);
-    if (k >= 1 && b->paired) k = pair_batch_blocks_per_sm(b->ks, smem);
-    if (k < 1) return bset_err(b, TEUK_E_INVAL, "the batched kernel does not fit on this device with these tiles");
+    // CTAs per SM of the kernel that runs the steps, and whether the first step's fits
+    auto fit = [&](int ks) {
+        return b->prec == TEUK_FP32 ? split_batch_blocks_per_sm<float>(b->seg, smem, ks)
+                                    : split_batch_blocks_per_sm<double>(b->seg, smem, ks);
+    };
+    const int k = b->paired ? pair_batch_blocks_per_sm(b->ks, smem) : fit(b->ks);
+    if (k < 1 || fit(1) < 1) return bset_err(b, TEUK_E_INVAL, "the batched kernel does not fit on this device with these tiles");
     // A launch of several waves of tiles ends with the list's last ones, so the
     // last part of every instance goes in tiles of half the height: a quarter of
     // a wave's worth, measured on 16 uneven FP32 instances (5.4 waves) at 0, 0.2,

@@ -11,6 +11,8 @@
 
 #include <new>
 #include <algorithm>
+#include <functional>
+#include <queue>
 #include <vector>
 
 #include "teuk_internal.cuh"
@@ -1778,6 +1780,44 @@ int batch_half(const teuk_batch *b, int i)
     return h >= 1 && h < b->tr[i] ? h : b->tr[i];
 }
 
+// The tile list, instances interleaved tile by tile, with the last part `tail` of
+// every instance in tiles of half the height.
+void batch_tiles(teuk_batch *b, double tail)
+{
+    const int n = (int)b->c.size();
+    b->htiles.clear();
+    b->nt.assign(n, 0);
+    std::vector<int> row(n, 0);
+    for (int half = 0; half < 2; ++half)
+        for (bool more = true; more;) {
+            more = false;
+            for (int i = 0; i < n; ++i) {
+                const int Nr = (int)b->c[i]->d.Nr, h = half ? batch_half(b, i) : b->tr[i];
+                if (row[i] >= (half ? Nr : (int)((1.0 - tail) * Nr))) continue;
+                b->htiles.push_back(make_int2(i | h << kTileShift, row[i]));
+                row[i] += h;
+                ++b->nt[i];
+                more = true;
+            }
+        }
+}
+
+// When the last of the list's tiles ends on `slots` slots, in points of rows (halos included).
+long long batch_span(const teuk_batch *b, int slots)
+{
+    std::priority_queue<long long, std::vector<long long>, std::greater<long long>> free;
+    for (int k = 0; k < slots; ++k) free.push(0);
+    long long last = 0;
+    for (const int2 &e : b->htiles) {
+        const long long rows = (e.x >> kTileShift) + 2 * b->ks;
+        const long long end = free.top() + rows * b->c[e.x & ((1 << kTileShift) - 1)]->d.Ntheta;
+        free.pop();
+        free.push(end);
+        last = std::max(last, end);
+    }
+    return last;
+}
+
 // Tile list (instances interleaved tile by tile) and shared memory for the
 // current tile heights; drops the captured graph.
 int batch_layout(teuk_batch *b)
@@ -1805,27 +1845,22 @@ int batch_layout(teuk_batch *b)
     const int k = b->paired ? pair_batch_blocks_per_sm(b->ks, smem) : fit(b->ks);
     if (k < 1 || fit(1) < 1) return bset_err(b, TEUK_E_INVAL, "the batched kernel does not fit on this device with these tiles");
     // A launch of several waves of tiles ends with the list's last ones, so the
-    // last part of every instance goes in tiles of half the height: a quarter of
-    // a wave's worth, measured on 16 uneven FP32 instances (5.4 waves) at 0, 0.2,
-    // 0.4, 0.7 and 1 wave: 110.6, 108.4, 108.6, 109.9 and 111.1 us per step.
-    // (Instances interleaved tile by tile: the longest rows first took 113.3.)
-    const double slots = (double)k * sm_count();
+    // last part of every instance, a quarter of a wave's worth, goes in tiles of
+    // half the height: us per step without and with, 16 uneven FP32 instances (5.4
+    // waves) 111.1 and 109.9, 64 of them 500.9 and 497.1, 6 x 4000 x 250 FP32 119.2
+    // and 116.0, 8 uneven FP64 609.7 and 598.3.  Where the tiles fill their last
+    // wave it takes longer (4 x 3000 x 200 FP64, 3.95 waves: 607 and 633), so the
+    // list is scheduled both ways first, a tile taking its rows' time on the first
+    // slot that is free.  (Instances interleaved tile by tile: the longest rows
+    // first took 113.3.)
+    const int slots = k * sm_count();
     const double tail = (double)whole > 2.0 * slots ? 0.25 * slots / (double)whole : 0.0;
-    b->htiles.clear();
-    b->nt.assign(n, 0);
-    std::vector<int> row(n, 0);
-    for (int half = 0; half < 2; ++half)
-        for (bool more = true; more;) {
-            more = false;
-            for (int i = 0; i < n; ++i) {
-                const int Nr = (int)b->c[i]->d.Nr, h = half ? batch_half(b, i) : b->tr[i];
-                if (row[i] >= (half ? Nr : (int)((1.0 - tail) * Nr))) continue;
-                b->htiles.push_back(make_int2(i | h << kTileShift, row[i]));
-                row[i] += h;
-                ++b->nt[i];
-                more = true;
-            }
-        }
+    batch_tiles(b, 0.0);
+    if (tail > 0.0) {
+        const long long plain = batch_span(b, slots);
+        batch_tiles(b, tail);
+        if (batch_span(b, slots) > plain) batch_tiles(b, 0.0);
+    }
     b->ntot = (int)b->htiles.size();
     b->smem = smem;
     if ((size_t)b->ntot * sizeof(int2) > b->ws_bytes - b->off_tiles)

@@ -201,3 +201,19 @@ def test_fp32_tall_tiles_of_paired_widths(Nth, tall):
     st.close()
     for u, h in got[1:]:
         assert np.array_equal(u, got[0][0]) and np.array_equal(h, got[0][1])
+
+
+def test_batch_whose_tiles_fill_their_last_wave_keeps_them_whole():
+    """600 FP64 tiles on 152 SMs (3.95 waves): half-height tiles at the end of the
+    list would end a third of a tile later, so every tile has the full height."""
+    import torch
+    from paper_0909_4039_gb300 import teuk
+    if torch.cuda.get_device_properties(0).multi_processor_count != 152:
+        pytest.skip("the tile counts are for 152 SMs")
+    sts = [gpu_stepper(_w(3000, 200, m, r0), "fp64", wave_capacity=4) for m, r0 in ((2, 8.0), (1, 9.0), (3, 7.0), (4, 12.0))]
+    b = teuk.Batch(sts)
+    b.set_tiling([20] * 4, 2)
+    assert b.tiling()["total_tiles"] == 600
+    b.close()
+    for st in sts:
+        st.close()

@@ -240,8 +240,14 @@ double host_atheta_bound(const teuk_grid_desc &d)
 //   FP64: the FP64 pipe bounds it.  A scheduler starts one FP64 instruction
 //   per 64 cycles, so a step costs the busiest scheduler's count: per theta
 //   element of a lane's segment 57 (and 48 per segment for the scans) in the
-//   implicit stage, 26 per element in the Lax-Wendroff stages; 1.5 us of
-//   latency a step and 4.5 us a launch and wave come on top.  An SM's tiles
+//   implicit stage, 26 per element in the Lax-Wendroff stages.  On top come, for
+//   a tile of P thousand points, 4.5 + 2 P us a launch (its state has to arrive,
+//   with no second CTA to overlap that) and 1.5 us a step, 4 P % where an SM has
+//   one tile of up to 128 points a row (no other tile overlaps its barriers), and
+//   10 % for the kernels of more steps on rows of more than 256 points, which spill
+//   more.  (Over 31 grids with 140 tilings measured, the choice takes 0.6 % more
+//   than the best of them, 7.8 % at most; without the terms in P, 6000 x 110 176 us
+//   a step for 156, 12000 x 48 155 for 146, 25806 x 38 297 for 272.)  An SM's tiles
 //   share its pipes, so their counts add up.  (Model against measurement:
 //   16384 x 128, 36 rows, two steps 349 / 365 us; 1024 x 32, 7 rows, three
 //   steps 14 / 17.)
@@ -323,8 +329,15 @@ static bool tiled_cand(const teuk_ctx *c, int TR, int ks, int nsm, TileCand *out
             const int warps = N <= threads ? up(N * up(rl, sl), 32) : 8 * up(N, threads);
             pipe += 64.0 * up(warps, 4) * 26.0 * sl;
         }
-        cost = per * pipe / 2070.0 + waves * (4.5 + 1.5 * ks);
+        const double P = 0.001 * TR * N;   // the tile's points
+        cost = per * pipe / 2070.0 + waves * (4.5 + 2.0 * P + 1.5 * ks);
+        if (S == kSegWide && ks > 1) cost *= 1.1;
+        if (per == 1 && S == kSegNarrow) cost *= 1.0 + 0.04 * P;
     }
+    // FP32 rows of 129 to 256 points: the scalar kernel at a height that no pair tile
+    // has (8812 x 132, 58 rows 32.6 us a step; pair tiles of 29 rows 28.5), and
+    // tiles without a copy of the theta table (48122 x 194, 64 rows 198; 53 rows 183)
+    if (f32 && S == kSeg && !pair_runs(TR, N, ks) && (pair_eligible(N) || !split_smem_plan(TR + 2 * ks, N, 4).th2)) cost *= 1.25;
     out->cost = cost / ks;
     out->R = TR + 2;
     out->persist = 0;

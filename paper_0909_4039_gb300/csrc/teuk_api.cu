@@ -605,7 +605,12 @@ int unit_steps(const teuk_ctx *c) { return c->d.scheme == TEUK_SCHEME_SPLIT && c
 // Whether the tiles of a call of nsteps steps sample their own steps (own_samples).
 bool own_call(const teuk_ctx *c, int64_t nsteps)
 {
-    return nsteps <= kOwnSteps && own_samples(c->d.precision == TEUK_FP32 ? 4 : 8, implicit_seg((int)c->d.Ntheta));
+    if (c->d.precision != TEUK_FP32 || nsteps > kOwnSteps) return false;
+    const int N = (int)c->d.Ntheta, seg = implicit_seg(N);
+    if (seg == kSegNarrow || nsteps == 1) return true;
+    if (seg == kSeg) return false;
+    return c->ks <= 2 && (c->d.Nr + c->tile_rows - 1) / c->tile_rows > 2 * sm_count() &&
+           own_wide_bytes(c->tile_rows, N) <= 225 * 1024;
 }
 
 // One launch of ks steps (1, or 2 and 3 of a shifted state) from level in_level;
@@ -1910,9 +1915,16 @@ int batch_tables(teuk_batch *b, cudaStream_t st)
     return TEUK_OK;
 }
 
+// Whether the tiles of a call of nsteps steps sample their own steps (own_samples).
+bool batch_own(const teuk_batch *b, int64_t nsteps)
+{
+    const bool f32 = b->prec == TEUK_FP32;
+    return own_samples(f32 ? 4 : 8, b->seg) || (b->seg == kSegWide && nsteps <= (f32 ? kOwnSteps : 1));
+}
+
 // One launch from parameter table `table` with ks steps (the first-step
 // table always takes one).
-cudaError_t batch_launch(teuk_batch *b, int table, int ks, cudaStream_t st)
+cudaError_t batch_launch(teuk_batch *b, int table, int ks, bool own, cudaStream_t st)
 {
     const int2 *tiles = (const int2 *)(b->ws + b->off_tiles);
     if (table == 2) ks = 1;
@@ -1920,9 +1932,9 @@ cudaError_t batch_launch(teuk_batch *b, int table, int ks, cudaStream_t st)
         return launch_pair_batch((const StepParams<float> *)(b->ws + b->off_par[table]), tiles, b->ntot, b->smem, ks, st);
     if (b->prec == TEUK_FP32)
         return launch_split_batch<float>((const StepParams<float> *)(b->ws + b->off_par[table]), tiles, b->ntot, b->seg,
-                                         b->smem, ks, st);
+                                         b->smem, ks, own, st);
     return launch_split_batch<double>((const StepParams<double> *)(b->ws + b->off_par[table]), tiles, b->ntot, b->seg,
-                                      b->smem, ks, st);
+                                      b->smem, ks, own, st);
 }
 
 int batch_step_impl(teuk_batch *b, int64_t nsteps, cudaStream_t st)
@@ -1935,7 +1947,7 @@ int batch_step_impl(teuk_batch *b, int64_t nsteps, cudaStream_t st)
     for (teuk_ctx *c : b->c) Nmax = (int)c->d.Ntheta > Nmax ? (int)c->d.Ntheta : Nmax;
     int pending = 0;   // steps whose extraction rows wait for a sampling launch
     // (none where the tiles sample their own steps; any parameter table: it reads the rows, not the state)
-    const bool own = own_samples(b->prec == TEUK_FP32 ? 4 : 8, b->seg);
+    const bool own = batch_own(b, nsteps);
     auto samples = [&](int n) {
         if (own) return cudaSuccess;
         const char *tab = b->ws + b->off_par[0];
@@ -1947,7 +1959,7 @@ int batch_step_impl(teuk_batch *b, int64_t nsteps, cudaStream_t st)
     for (teuk_ctx *c : b->c) any_first = any_first || !c->shifted;
     if (any_first) {
         // first step from physical states: s_{n+1} = LW C_{dt/2} u_n where needed
-        BCK(batch_launch(b, 2, 1, st), "batched first step");
+        BCK(batch_launch(b, 2, 1, own, st), "batched first step");
         for (teuk_ctx *c : b->c) {
             c->cur ^= 1;
             c->shifted = 1;
@@ -1967,7 +1979,7 @@ int batch_step_impl(teuk_batch *b, int64_t nsteps, cudaStream_t st)
             BCK(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal), "begin capture");
             cudaError_t le = cudaSuccess;
             // kGraphChunk / ks launches: an even count, so the level parity is unchanged
-            for (int k = 0; k < kGraphChunk / b->ks && le == cudaSuccess; ++k) le = batch_launch(b, k & 1, b->ks, st);
+            for (int k = 0; k < kGraphChunk / b->ks && le == cudaSuccess; ++k) le = batch_launch(b, k & 1, b->ks, own, st);
             cudaError_t ee = cudaStreamEndCapture(st, &graph);
             if (le != cudaSuccess) return bcuda_err(b, le, "captured batched launch");
             if (ee != cudaSuccess) return bcuda_err(b, ee, "end capture");
@@ -1997,7 +2009,7 @@ int batch_step_impl(teuk_batch *b, int64_t nsteps, cudaStream_t st)
             BCK(samples(pending), "samples");
             pending = 0;
         }
-        BCK(batch_launch(b, (int)(launches & 1), k, st), "batched step");
+        BCK(batch_launch(b, (int)(launches & 1), k, own, st), "batched step");
         left -= k;
         pending += k;
     }
@@ -2151,9 +2163,10 @@ int teuk_batch_autotune(teuk_batch *b, int trial_steps, void *stream)
         int r = batch_tables(b, st);   // parameters for these tile heights
         if (r != TEUK_OK) return r;
         cudaError_t e = cudaSuccess;
-        for (int w = 0; w < 2 && e == cudaSuccess; ++w) e = batch_launch(b, w & 1, b->ks, st);
+        const bool own = batch_own(b, INT64_MAX);   // as in a long call
+        for (int w = 0; w < 2 && e == cudaSuccess; ++w) e = batch_launch(b, w & 1, b->ks, own, st);
         if (e == cudaSuccess) e = cudaEventRecord(e0, st);
-        for (int w = 0; w < trial_steps && e == cudaSuccess; ++w) e = batch_launch(b, w & 1, b->ks, st);
+        for (int w = 0; w < trial_steps && e == cudaSuccess; ++w) e = batch_launch(b, w & 1, b->ks, own, st);
         if (e == cudaSuccess) e = cudaEventRecord(e1, st);
         if (e == cudaSuccess) e = cudaEventSynchronize(e1);
         float ms = 0.0f;

@@ -12,6 +12,7 @@
 #include <math.h>
 #include <stdio.h>
 
+#include <algorithm>
 #include <mutex>
 #include <type_traits>
 #include <utility>
@@ -1902,7 +1903,7 @@ __device__ __forceinline__ void split_tile(const StepParams<T> &p, int i0, int n
     // those rows side by side (launch_sample_steps).  Solved here, one row by
     // one warp in every step, they ended the tile's every step: 17 of a
     // 1024 x 32 FP64 step's 35 us.  OWN: the tile samples its steps all the
-    // same (kOwnSamples).
+    // same (own_samples).
     const bool ext_row = p.i_ext >= i0 && p.i_ext < i0 + TR && p.i_ext < Nr;
     const bool ext = !p.imp_only && p.nfix < 0 && ext_row;
     const int lx = p.i_ext - g0;

@@ -236,14 +236,22 @@ constexpr int kSeg = 8;                 // theta elements per thread (Ntheta <= 
 constexpr int kSegWide = 32;            // theta elements per thread (Ntheta <= 1024)
 // theta elements per thread of the implicit row solves
 __host__ __device__ inline int implicit_seg(int Nth) { return Nth <= 128 ? kSegNarrow : (Nth <= 256 ? kSeg : kSegWide); }
-// Whether the split kernels' tiles can sample their own steps: FP32 rows of up
-// to 128 theta points (seg: the segment).  A batch's tiles do: two CTAs share an
-// SM there, and the others run while one warp solves the extraction row; leaving
-// the rows to a sampling launch took 1.6 % longer for 16 uneven instances (130
-// steps: 15.64 against 15.39 ms).  A lone state's do in calls of a few steps, to
-// which a sampling launch adds 5 us (16384 x 128, three steps a call, L2 flushed:
-// 71.3 against 75.9 Gpts/s); in long calls the launch is the faster way (200
-// steps: 4.99 against 5.23 ms; 1024 x 32, 100 steps: 0.44 against 0.76 in the tile).
+// Rows whose tiles sample their own steps in every batch and in a lone state's
+// calls of a few steps: FP32 of up to 128 theta points (seg: the segment).  In a
+// batch two CTAs share an SM there, and the others run while one warp solves the
+// extraction row; leaving the rows to a sampling launch took 1.6 % longer for 16
+// uneven instances (130 steps: 15.64 against 15.39 ms).  To a call of a few steps
+// a sampling launch adds 5 us (16384 x 128, three steps a call, L2 flushed: 71.3
+// against 75.9 Gpts/s); in long calls the launch is the faster way (200 steps:
+// 4.99 against 5.23 ms; 1024 x 32, 100 steps: 0.44 against 0.76 in the tile).
+// Wider FP32 rows leave them to the sampling launch (its solves of all pending
+// steps run side by side), but in calls of one step, which the launch at their
+// end lengthens (2000 x 130 23.5 us with it, 17.1 without; 16384 x 256 91 and 80;
+// 600 x 700 80 and 75), and, above 256 points, in calls of up to four steps on
+// grids of more than two tiles per SM, of which the others hide it (16384 x 300,
+// two steps 716 and 664).  Batches of rows of more than 256 points do so in calls
+// of up to four steps in FP32 and of one in FP64 (four instances of 1500 x 300,
+// one step: 230 and 194 us, 890 and 730).
 constexpr bool own_samples(size_t real_bytes, int seg) { return real_bytes == 4 && seg == kSegNarrow; }
 // shared memory of the extraction row's copy in a launch of two or three steps
 inline size_t own_copy_bytes(int Nth, size_t real_bytes)
@@ -308,6 +316,9 @@ inline size_t split_tile_bytes(int tile_rows, int Nth, int ks, size_t real_bytes
     }
     return most;
 }
+
+// The same for a self-sampling launch of up to two steps on FP32 rows of more than 256 points.
+inline size_t own_wide_bytes(int tile_rows, int Nth) { return split_tile_bytes(tile_rows, Nth, 2, 4) + 16 * (size_t)Nth; }
 
 // Shared-memory carve-up of the persistent split kernel: theta tables, a
 // copy of the extraction row (state and step-table entry) and two tile
@@ -522,11 +533,12 @@ constexpr int kMaxTileRows = 254;
 // instance must use the theta segment `seg` (implicit_seg of its Ntheta).
 // ks = 2 advances every instance by two steps per launch (no first steps);
 // it exists for segments of up to 8 elements only (split_batch_available).
+// own: the tiles of segments of 32 elements sample their steps (see own_samples).
 template <typename T>
 int split_batch_blocks_per_sm(int seg, size_t smem, int ks);
 template <typename T>
 cudaError_t launch_split_batch(const StepParams<T> *d_params, const int2 *d_tiles, int ntiles, int seg, size_t smem,
-                               int ks, cudaStream_t st);
+                               int ks, bool own, cudaStream_t st);
 // Dynamic shared memory of a batch tile with ks steps per launch, by the kernels
 // that run it: k_pair_batch for the full steps of a batch whose every instance
 // is eligible (paired; k_split_batch with one step then takes first steps at the

@@ -39,7 +39,7 @@ int pair_batch_blocks_per_sm(int ks, size_t smem) { return blocks_per_sm((const 
 cudaError_t launch_pair_step(const StepParams<float> &p, int ks, cudaStream_t st)
 {
     if (p.first || p.imp_only || p.nfix >= 0 || !pair_runs(p.tile_rows, p.Nth, ks)) return cudaErrorInvalidValue;
-    auto fn = pair_fn(ks);
+    auto fn = p.own && ks == 1 ? k_pair_step<1, true> : pair_fn(ks);
     cudaError_t e = smem_limit_max((const void *)fn);
     if (e != cudaSuccess) return e;
     return launch_dep(fn, dim3((unsigned)((p.Nr + p.tile_rows - 1) / p.tile_rows)), 256,

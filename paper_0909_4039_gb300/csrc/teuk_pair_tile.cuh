@@ -87,8 +87,9 @@ __device__ __forceinline__ int lw_pair_field(int q)
 }
 
 // The work of one CTA, as split_tile's for full steps of a context (no first
-// step, no state output, no caller buffers).
-template <int KS>
+// step, no state output, no caller buffers).  OWN (one step): the tile samples
+// its step.
+template <int KS, bool OWN = false>
 __device__ __forceinline__ void pair_tile(const StepParams<float> &p, int i0, int ntiles)
 {
     constexpr int kMaxChunks = 8;
@@ -449,13 +450,33 @@ __device__ __forceinline__ void pair_tile(const StepParams<float> &p, int i0, in
             }
         }
     }
+    if constexpr (OWN) {
+        static_assert(KS == 1, "the sample of the launch's last step");
+        if (!ext) return;
+        __syncthreads();   // the row is in p.raw, the tile's shared memory is free
+        if (warp == 0) {
+            float2 *rf = (float2 *)sPhi, *rg = (float2 *)sPi;
+            const float2 *src_row = raw_row(n_in + 1);
+            for (int j = lane; j < N; j += 32) {
+                rf[j] = src_row[j];
+                rg[j] = src_row[N + j];
+            }
+            __syncwarp();
+            const bool active = p.i_ext >= 1 && p.i_ext <= Nr - 2;
+            implicit_row_one<float, kSeg>(p.half, rf, rg, p.i_ext, p.stab + (size_t)(2 * p.i_ext) * NSF, nullptr, p.th2, N,
+                                          active, true, lane, 32, p.vec != 0, p.half.plan[p.i_ext]);
+            __syncwarp();
+            extract_warp<float>(p, rf, n_in + 1);
+            if (lane == 0) p.ctl->sampled = n_in + 1;
+        }
+    }
 }
 
-template <int KS>
+template <int KS, bool OWN = false>
 __global__ void __launch_bounds__(256, 1) k_pair_step(const StepParams<float> p)
 {
     launch_turn();
-    pair_tile<KS>(p, (int)blockIdx.x * p.tile_rows, (int)gridDim.x);
+    pair_tile<KS, OWN>(p, (int)blockIdx.x * p.tile_rows, (int)gridDim.x);
 }
 
 // Batched form, as k_split_batch: entry blockIdx.x of the tile list.

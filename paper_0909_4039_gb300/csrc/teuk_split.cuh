@@ -61,7 +61,7 @@ __global__ void __launch_bounds__(256, (sizeof(T) == 4 && S <= 4) ? 2 : 1) k_spl
 // step; the instances may differ in every parameter (grid, spin, mode,
 // source, tile height) as long as they share the state precision and the
 // theta segment S.  KS = 2: two time steps per launch, as k_split_step2.
-template <typename T, int S, int KS>
+template <typename T, int S, int KS, bool OWN = own_samples(sizeof(T), S)>
 __global__ void __launch_bounds__(256, (sizeof(T) == 4 && S <= 4) ? 2 : 1)
     k_split_batch(const StepParams<T> *params, const int2 *tiles)
 {
@@ -69,7 +69,7 @@ __global__ void __launch_bounds__(256, (sizeof(T) == 4 && S <= 4) ? 2 : 1)
     const int2 e = tiles[blockIdx.x];
     batch_params(sp, params, e);
     launch_turn();
-    split_tile<T, S, KS, own_samples(sizeof(T), S), true>(sp, e.y, sp.ntiles);
+    split_tile<T, S, KS, OWN, true>(sp, e.y, sp.ntiles);
 }
 
 // Stored scan plans: the levels scan_plan chooses for every row of the
@@ -608,8 +608,9 @@ cudaError_t launch_split_step(const StepParams<T> &p, int threads, size_t smem, 
     const int seg = implicit_seg(p.Nth);
     const int v = seg == kSegNarrow ? 0 : (seg == kSeg ? 1 : 2);
     auto fn = v == 0 ? k_split_step<T, kSegNarrow> : (v == 1 ? k_split_step<T, kSeg> : k_split_step<T, kSegWide>);
-    if constexpr (own_samples(sizeof(T), kSegNarrow))
-        if (p.own && !p.imp_only && p.nfix < 0) fn = k_split_step<T, kSegNarrow, true>;
+    if constexpr (sizeof(T) == 4)
+        if (p.own && !p.imp_only && p.nfix < 0)
+            fn = v == 0 ? k_split_step<T, kSegNarrow, true> : (v == 1 ? k_split_step<T, kSeg, true> : k_split_step<T, kSegWide, true>);
     cudaError_t e = smem_limit_max((const void *)fn);
     if (e != cudaSuccess) return e;
     int grid = (p.Nr + p.tile_rows - 1) / p.tile_rows;
@@ -617,8 +618,9 @@ cudaError_t launch_split_step(const StepParams<T> &p, int threads, size_t smem, 
 }
 
 template <typename T>
-static void (*batch_fn(int seg, int ks))(const StepParams<T> *, const int2 *)
+static void (*batch_fn(int seg, int ks, bool own = false))(const StepParams<T> *, const int2 *)
 {
+    if (own && seg == kSegWide) return ks == 1 ? k_split_batch<T, kSegWide, 1, true> : nullptr;
     // two steps per launch for segments of up to 8 elements (Ntheta <= 256)
     if (ks == 2) return seg == kSegNarrow ? k_split_batch<T, kSegNarrow, 2> : (seg == kSeg ? k_split_batch<T, kSeg, 2> : nullptr);
     return seg == kSegNarrow ? k_split_batch<T, kSegNarrow, 1>
@@ -644,9 +646,9 @@ int split_batch_blocks_per_sm(int seg, size_t smem, int ks)
 
 template <typename T>
 cudaError_t launch_split_batch(const StepParams<T> *d_params, const int2 *d_tiles, int ntiles, int seg, size_t smem,
-                               int ks, cudaStream_t st)
+                               int ks, bool own, cudaStream_t st)
 {
-    auto fn = batch_fn<T>(seg, ks);
+    auto fn = batch_fn<T>(seg, ks, own);
     if (!fn) return cudaErrorInvalidValue;
     cudaError_t e = smem_limit_max((const void *)fn);
     if (e != cudaSuccess) return e;
@@ -707,8 +709,11 @@ cudaError_t launch_split_step2(const StepParams<T> &p, int threads, size_t smem,
         if (pair_runs(p.tile_rows, p.Nth, 2)) return launch_pair_step(p, 2, st);
     if (smem < split_tile_bytes(p.tile_rows, p.Nth, 2, sizeof(T))) return cudaErrorInvalidValue;
     auto fn = split2_fn<T>(p.Nth);
-    if constexpr (own_samples(sizeof(T), kSegNarrow))
-        if (p.own) fn = k_split_step2<T, kSegNarrow, true>;
+    if constexpr (sizeof(T) == 4)
+        if (p.own && implicit_seg(p.Nth) != kSeg) {
+            fn = implicit_seg(p.Nth) == kSegNarrow ? k_split_step2<T, kSegNarrow, true> : k_split_step2<T, kSegWide, true>;
+            smem = std::max(smem, own_wide_bytes(p.tile_rows, p.Nth));
+        }
     cudaError_t e = smem_limit_max((const void *)fn);
     if (e != cudaSuccess) return e;
     int grid = (p.Nr + p.tile_rows - 1) / p.tile_rows;

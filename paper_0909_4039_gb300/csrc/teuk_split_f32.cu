@@ -8,7 +8,7 @@ template cudaError_t launch_scan_plans<float>(const StepParams<float> &, int *, 
                                                cudaStream_t);
 template int split_batch_blocks_per_sm<float>(int, size_t, int);
 template cudaError_t launch_split_batch<float>(const StepParams<float> *, const int2 *, int, int, size_t, int,
-                                               cudaStream_t);
+                                               bool, cudaStream_t);
 template size_t split2_smem_bytes<float>(int, int);
 template int split2_blocks_per_sm<float>(int, int, int, size_t);
 template cudaError_t launch_split_step2<float>(const StepParams<float> &, int, size_t, cudaStream_t);

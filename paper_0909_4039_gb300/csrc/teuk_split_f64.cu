@@ -8,7 +8,7 @@ template cudaError_t launch_scan_plans<double>(const StepParams<double> &, int *
                                                cudaStream_t);
 template int split_batch_blocks_per_sm<double>(int, size_t, int);
 template cudaError_t launch_split_batch<double>(const StepParams<double> *, const int2 *, int, int, size_t, int,
-                                                cudaStream_t);
+                                                bool, cudaStream_t);
 template size_t split2_smem_bytes<double>(int, int);
 template int split2_blocks_per_sm<double>(int, int, int, size_t);
 template cudaError_t launch_split_step2<double>(const StepParams<double> &, int, size_t, cudaStream_t);

@@ -217,3 +217,34 @@ def test_batch_whose_tiles_fill_their_last_wave_keeps_them_whole():
     b.close()
     for st in sts:
         st.close()
+
+
+@pytest.mark.parametrize("precision,Nr,Nth,tiling", [("fp32", 330, 130, None), ("fp32", 330, 200, None), ("fp32", 330, 256, (7, 1)),
+                                                     ("fp32", 700, 300, (2, 2)), ("fp32", 700, 300, (2, 1)),
+                                                     ("fp64", 330, 300, None)])
+def test_samples_of_short_calls_on_wide_rows(precision, Nr, Nth, tiling):
+    """Calls of one to a few steps on rows of more than 128 points, whose tiles
+    sample their own steps where a sampling launch would lengthen the call (FP32:
+    one step up to 256 points; up to four steps above, on grids of more than two
+    tiles per SM), give the samples, rows and state of one call; so do the calls
+    of a batch of one such instance."""
+    from paper_0909_4039_gb300 import teuk
+    w = _w(Nr, Nth)
+    u0, n, res = inputs.random_state(Nr, Nth, seed=60), 14, []
+    calls = [1, 1, 2, 3, 1, 4, 2]
+    for k, plan in enumerate(([n], calls, calls)):
+        st = gpu_stepper(w, precision, wave_capacity=n + 1)
+        if tiling and k < 2:
+            st.set_tiling(*tiling)
+        st.set_state(u0, 0)
+        b = teuk.Batch([st]) if k == 2 else None
+        for c in plan:
+            (b or st).step(c)
+        if b:
+            b.synchronize()
+            b.close()
+        h, rows = st.waveform(0, n + 1, rows=True)
+        res.append((st.get_state(), np.asarray(h), np.asarray(rows)))
+        st.close()
+    for r in res[1:]:
+        assert all(np.array_equal(x, y) for x, y in zip(r, res[0]))

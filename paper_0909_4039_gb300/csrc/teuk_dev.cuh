@@ -818,7 +818,7 @@ __device__ __forceinline__ void apply_W(const ImpCoef<T, S> &C, const typename V
 // elements [g S, g S + S)); f is the row's step-table entry; plan the row's
 // stored scan levels (0 for a row that is not active).  Same map as
 // implicit_row_group.
-template <typename T, int S, bool MAT = false>
+template <typename T, int S>
 __device__ void implicit_row_fwd(const ImpConst<T> &K0, typename V2<T>::t *phi, typename V2<T>::t *pi,
                                  const typename V2<T>::t *prow, const T *f, const T *th, int N, bool active,
                                  bool in_tile, int g, int G, bool vec, int plan, typename V2<T>::t *u1phi = nullptr,
@@ -1321,8 +1321,7 @@ __device__ void lw_segment(const StepParams<T> &p, typename V2<T>::t *sPhi, type
 
     // beta and kap at tile position e (2 lr: node, 2 k + 1: half node), and
     // 1/Sigma^2 there when the source needs it
-    auto coef = [&](int e, T &beta, c2 &kap, T &sg, bool need_sg) {
-        (void)need_sg;
+    auto coef = [&](int e, T &beta, c2 &kap, T &sg) {
         lw_coef<T>(sSt + e * NSF, S2, C, beta, kap, &sg);
     };
     // source at tile position e times the scaled phase ph (zero outside the
@@ -1346,7 +1345,7 @@ __device__ void lw_segment(const StepParams<T> &p, typename V2<T>::t *sPhi, type
         T beta, sg;
         c2 kap;
         const bool s_row = SRC && src && gl >= p.patch_p0 && gl < p.patch_p0 + p.patch_np;
-        coef(2 * k + 1, beta, kap, sg, s_row);
+        coef(2 * k + 1, beta, kap, sg);
         const c2 df = csub(fb, fa);
         mf = caxpy(-beta, df, cscale<c2>(half, cadd(fa, fb)));
         c2 t = caxpy(beta, csub(gb, ga), cscale<c2>(half, cadd(ga, gb)));
@@ -1379,7 +1378,7 @@ __device__ void lw_segment(const StepParams<T> &p, typename V2<T>::t *sPhi, type
             T beta, sg;
             c2 kap;
             const bool s_row = SRC && src && gi >= p.patch_p0 && gi < p.patch_p0 + p.patch_np;
-            coef(2 * lr, beta, kap, sg, s_row);
+            coef(2 * lr, beta, kap, sg);
             const c2 dmf = csub(mf, mfp);
             nfv = caxpy(-beta, dmf, fb);
             c2 t = caxpy(beta, csub(mg, mgp), gb);

@@ -249,7 +249,7 @@ double host_atheta_bound(const teuk_grid_desc &d)
 //   than the best of them, 7.8 % at most; without the terms in P, 6000 x 110 176 us
 //   a step for 156, 12000 x 48 155 for 146, 25806 x 38 297 for 272.)  An SM's tiles
 //   share its pipes, so their counts add up.  (Model against measurement:
-//   16384 x 128, 36 rows, two steps 349 / 365 us; 1024 x 32, 7 rows, three
+//   16384 x 128, 36 rows, two steps 363 / 367 us; 1024 x 32, 7 rows, three
 //   steps 14 / 17.)
 //   FP32: 0.6 Rpad + 0.4 R row-times a step (Rpad: whole warps of rows; whole
 //   passes of the eight warps for Ntheta > 256, whose spilled rows leave an SM's

@@ -1,6 +1,6 @@
 // teuk_split.cuh -- split-scheme step kernels for sm_103a (tiled, two steps
 // per launch, batched) and their launchers, for one state precision T;
-// teuk_split_f32.cu and teuk_split_f64.cu instantiate them.
+// teuk_split_*.cu, teuk_batch_*.cu and teuk_pipe_*.cu instantiate them.
 //
 // Split scheme (default), one fused kernel per time step.  Each CTA owns a
 // tile of TR consecutive r* rows with full theta rows and holds rows
